@@ -11,7 +11,7 @@
 //       rho = 3 chi u~'/2 - 2; stored scaled by e^{8/(3 chi)}.
 // Each row integrates panels of width 1/16 in t with 12-point Gauss-Legendre, sums them into the
 // CDF at the panel edges, and inverts the CDF at each r_m by Newton's method inside the bracketing
-// panel (partial integrals again by 12-point Gauss-Legendre).
+// panel, on the density's Legendre series there (from the same 12 nodes).
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -27,6 +27,7 @@ constexpr int kGL = 12;
 constexpr double kPanel = 1.0 / 16.0;
 __constant__ double c_gl_x[kGL];
 __constant__ double c_gl_w[kGL];
+__constant__ double c_legendre[kGL][kGL];  // [k][i] = (2k + 1)/2 w_i P_k(x_i): values at the nodes -> coefficients
 
 // Gauss-Legendre nodes and weights on [-1, 1] by Newton's method on the Legendre recurrence.
 static void gauss_legendre(int n, double* x, double* w) {
@@ -49,100 +50,176 @@ static void gauss_legendre(int n, double* x, double* w) {
     }
 }
 
-__global__ void bessel_table_kernel(double* tab64, float* tab32) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per node: the lanes take the terms of the three trapezoid sums (up to ~230 of them, each five
+// FP64 transcendentals, which one thread alone would chain: 295 us for the table against 38 us, 82 % of the FP64
+// pipe's cycles).
+__global__ void __launch_bounds__(128) bessel_table_kernel(double* tab64, float* tab32) {
+    const int j = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= kBesN) return;
     const double x = exp(log(kBesLo) + kBesH * j);
-    double o[3];
-    bessel_trapezoid(x, o);
+    double T, h;
+    const int n = bessel_steps(x, T, h);
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int m = 1 + lane; m <= n; m += 32) bessel_term(x, m * h, s);
     for (int f = 0; f < 3; ++f) {
-        tab64[f * kBesN + j] = o[f];
-        tab32[f * kBesN + j] = (float)o[f];
+        for (int o = 16; o > 0; o >>= 1) s[f] += __shfl_down_sync(0xffffffffu, s[f], o);
+        if (lane == 0) {
+            const double v = (0.5 + s[f]) * h;  // t = 0: exp(0) * cosh(0) terms, weight 1/2
+            tab64[f * kBesN + j] = v;
+            tab32[f * kBesN + j] = (float)v;
+        }
     }
 }
 
-__device__ __forceinline__ double row_density(const double* __restrict__ bes, bool nbw, double chi, double sigma, double t) {
+// the densities in t at both signs sigma = +1, -1 (they share the Bessel functions and all but one product)
+__device__ __forceinline__ void row_density(const double* __restrict__ bes, bool nbw, double chi, double t, double& dp,
+                                            double& dm) {
     double b[3];
     if (!nbw) {
         const double up = t * t * t;
-        const double den = 2.0 + 3.0 * chi * up;
-        const double lam = 3.0 * chi * up / den, one_m = 2.0 / den;
+        const double iden = 1.0 / (2.0 + 3.0 * chi * up);
+        const double lam = 3.0 * chi * up * iden, one_m = 2.0 * iden;
         bessel64(bes, up, b);
         const double kappa = 1.0 / one_m + one_m;
-        const double w = exp(-up) * (-b[2] + kappa * b[1] + sigma * lam * b[0]);
-        return w * 6.0 * chi / (den * den) * 3.0 * t * t;
+        const double f = exp(-up) * 18.0 * chi * iden * iden * t * t;
+        const double w = -b[2] + kappa * b[1], wl = lam * b[0];
+        dp = f * (w + wl);
+        dm = f * (w - wl);
+        return;
     }
     const double ut = 8.0 / (3.0 * chi) + t * t;
     bessel64(bes, ut, b);
     const double rho = 1.5 * chi * ut - 2.0;
-    const double w0 = b[2] + rho * b[1] - sigma * b[1];
-    return w0 * exp(-t * t) * 4.0 / (3.0 * chi * ut * sqrt(ut));
+    const double f = exp(-t * t) * 4.0 / (3.0 * chi * ut * sqrt(ut));
+    const double w = b[2] + rho * b[1];
+    dp = f * (w - b[1]);
+    dm = f * (w + b[1]);
 }
 
-__device__ __forceinline__ double gl_integral(const double* bes, bool nbw, double chi, double sigma, double a, double b) {
-    const double m = 0.5 * (a + b), r = 0.5 * (b - a);
-    double s = 0.0;
-#pragma unroll 4
-    for (int i = 0; i < kGL; ++i) s += c_gl_w[i] * row_density(bes, nbw, chi, sigma, m + r * c_gl_x[i]);
-    return s * r;
+constexpr int kMaxPanels = 144;  // sqrt(80) * 16 = 143.1 -> 144 panels for NBW, 69 for NLC
+
+// On a panel [a, a + d] with t = a + d s, x = 2 s - 1 and the density's Legendre coefficients c:
+//   dH/ds = d sum_k c_k P_k(x),   H(s) = int_a^t = d s [c_0 + (x - 1) sum_{k>=1} c_k P_k'(x) / (k (k + 1))]
+// (int_{-1}^x P_k = (x^2 - 1) P_k'(x) / (k (k + 1))): the factor s in front keeps the relative precision of H
+// down to s = 0, where the smallest r_m of a grid lie.
+__device__ __forceinline__ void panel_cdf(const double* c, double d, double s, double& H, double& h) {
+    const double x = 2.0 * s - 1.0;
+    double p0 = 1.0, p1 = x, q0 = 0.0, q1 = 1.0;  // P_k and P_k'
+    double f = fma(c[1], p1, c[0]), g = 0.5 * c[1];
+#pragma unroll
+    for (int k = 2; k < kGL; ++k) {
+        const double p = ((2.0 * k - 1.0) / k) * x * p1 - ((k - 1.0) / k) * p0;
+        const double q = fma(2.0 * k - 1.0, p1, q0);
+        f = fma(c[k], p, f);
+        g = fma(c[k] * (1.0 / (k * (k + 1.0))), q, g);
+        p0 = p1;
+        p1 = p;
+        q0 = q1;
+        q1 = q;
+    }
+    h = d * f;
+    H = d * s * fma(x - 1.0, g, c[0]);
 }
 
-constexpr int kMaxPanels = 160;  // sqrt(80) * 16 = 143.1 -> 144 panels for NBW, 69 for NLC
-
-// one block per (kind, sign, chi row)
+// One block per (kind, chi row), both signs.  FP64-bound: the density is evaluated at the panels' nodes only,
+// 1.3e6 Bessel triples for a 256 x 256 table.  Inverting the CDF with a quadrature and a density evaluation per
+// Newton step took 65 ms for that table (and its stopping rule, one rounding error of t, sent most entries
+// through a bisection); on the Legendre series a step is ~100 fused multiply-adds and the whole kernel 1.63 ms
+// (1.40e7 FP64 warp instructions, 83 % of the FP64 pipe's cycles).
 __global__ void __launch_bounds__(256) table_rows_kernel(const double* __restrict__ bes, qed_table_desc d, double* rates,
                                                          double* icdf) {
-    __shared__ double cum[kMaxPanels + 1];
+    __shared__ double coef[2][kMaxPanels][kGL];  // density at the nodes, then its Legendre coefficients
+    __shared__ double cum[2][kMaxPanels + 1];
     const int n_chi = d.n_chi;
-    const int job = blockIdx.x;
-    const bool nbw = job >= 2 * n_chi;
-    const int s = (job / n_chi) % 2;
-    const int i = job % n_chi;
-    const double sigma = s == 0 ? 1.0 : -1.0;
+    const bool nbw = (int)blockIdx.x >= n_chi;
+    const int i = blockIdx.x % n_chi;
     const double dl = (log(d.chi_max) - log(d.chi_min)) / (n_chi - 1);
     const double chi = exp(log(d.chi_min) + i * dl);
     const double tend = nbw ? sqrt(80.0) : cbrt(80.0);
     const int np = (int)ceil(tend / kPanel);
-    for (int p = threadIdx.x; p < np; p += blockDim.x) {
+    for (int e = threadIdx.x; e < np * kGL; e += blockDim.x) {
+        const int p = e / kGL, k = e % kGL;
         const double a = p * kPanel, b = fmin(tend, (p + 1) * kPanel);
-        cum[p + 1] = gl_integral(bes, nbw, chi, sigma, a, b);
+        row_density(bes, nbw, chi, 0.5 * (a + b) + 0.5 * (b - a) * c_gl_x[k], coef[0][p][k], coef[1][p][k]);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        cum[0] = 0.0;
-        for (int p = 0; p < np; ++p) cum[p + 1] += cum[p];
-        const double total = cum[np];
-        rates[(nbw ? 2 * n_chi : 0) + s * n_chi + i] = nbw ? log(2.0 * total) : log(total);
+    for (int e = threadIdx.x; e < 2 * np; e += blockDim.x) {
+        const int s = e / np, p = e % np;
+        double f[kGL], sum = 0.0;
+        for (int k = 0; k < kGL; ++k) {
+            f[k] = coef[s][p][k];
+            sum += c_gl_w[k] * f[k];
+        }
+        cum[s][p + 1] = sum * 0.5 * (fmin(tend, (p + 1) * kPanel) - p * kPanel);
+        for (int k = 0; k < kGL; ++k) {
+            double v = 0.0;
+            for (int q = 0; q < kGL; ++q) v += c_legendre[k][q] * f[q];
+            coef[s][p][k] = v;
+        }
     }
     __syncthreads();
-    const double total = cum[np];
+    if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) {  // one warp per sign
+        const int s = threadIdx.x >> 5;
+        double c = 0.0;
+        cum[s][0] = 0.0;
+        for (int p = 1; p <= np; ++p) {
+            c += cum[s][p];
+            cum[s][p] = c;
+        }
+        rates[(nbw ? 2 * n_chi : 0) + s * n_chi + i] = nbw ? log(2.0 * c) : log(c);
+    }
+    __syncthreads();
     const double dy = (d.y_hi - d.y_lo) / (d.n_r - 1);
-    double* out = icdf + ((size_t)((nbw ? 2 : 0) + s) * n_chi + i) * d.n_r;
-    for (int m = threadIdx.x; m < d.n_r; m += blockDim.x) {
-        const double y = d.y_lo + m * dy;
-        const double r = 1.0 / (1.0 + exp(-y));
-        const double target = r * total;
+    for (int e = threadIdx.x; e < 2 * d.n_r; e += blockDim.x) {
+        const int s = e / d.n_r, m = e % d.n_r;
+        const double r = 1.0 / (1.0 + exp(-(d.y_lo + m * dy)));
+        const double target = r * cum[s][np];
         // panel with cum[p] <= target < cum[p+1]
         int lo = 0, hi = np - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (cum[mid] <= target) lo = mid; else hi = mid - 1;
+            if (cum[s][mid] <= target) lo = mid; else hi = mid - 1;
         }
-        const int p = lo;
-        const double a = p * kPanel, b = fmin(tend, (p + 1) * kPanel);
-        double tl = a, th = b;
-        double t = a + (b - a) * (target - cum[p]) / (cum[p + 1] - cum[p]);
-        for (int it = 0; it < 100; ++it) {
-            const double F = cum[p] + gl_integral(bes, nbw, chi, sigma, a, t) - target;
-            if (F > 0.0) th = t; else tl = t;
-            const double dF = row_density(bes, nbw, chi, sigma, t);
-            double tn = t - F / dF;
-            if (!(tn > tl && tn < th)) tn = 0.5 * (tl + th);
-            const bool done = fabs(tn - t) <= 1e-15 * fmax(t, 1e-300) || th - tl <= 1e-15 * th;
-            t = tn;
-            if (done) break;
+        const double a = lo * kPanel, w = fmin(tend, (lo + 1) * kPanel) - a;
+        // The entry is the largest t whose CDF, rounded to FP64, does not exceed the target: half a rounding unit
+        // of the target above target - cum (near r = 1, where 1 - r is ~1e-9, that is what the entry hangs on).
+        const double ulp = __longlong_as_double(__double_as_longlong(target) + 1ll) - target;
+        const double T = (target - cum[s][lo]) + 0.5 * ulp, whole = cum[s][lo + 1] - cum[s][lo];
+        double u = whole > 0.0 ? fmin(T / whole, 1.0) : 0.5, ul = 0.0, uh = 1.0;
+        if (!(target > 0.0)) u = 0x1.0p-100;  // r below the FP64 range: a finite entry
+        else
+            for (int it = 0; it < 60; ++it) {
+                double H, h;
+                panel_cdf(coef[s][lo], w, u, H, h);
+                if (H > T) uh = u; else ul = u;
+                double un = u - (H - T) / h;
+                // a step below 1e-9 of u leaves an error below 1e-17 of it (the convergence is quadratic)
+                const bool found = fabs(un - u) <= 1e-9 * u;
+                if (!(un >= ul && un <= uh) && !found) un = 0.5 * (ul + uh);
+                u = un;
+                if (found) break;
+            }
+        double t = a + w * u;
+        // where the series has not converged within its 12 terms (the lowest panels of NBW rows with large chi,
+        // whose spectrum varies over t ~ chi^{-1/2}; the falling end of the NLC ones) the root is finished on
+        // the quadrature itself, one step from the series' root (about a quarter of a table's entries)
+        const double* c = coef[s][lo];
+        if (fabs(c[kGL - 1]) + fabs(c[kGL - 2]) > 2e-14 * fabs(c[0]) && t > a) {
+            for (int it = 0; it < 4; ++it) {
+                double dens[2], sum = 0.0;
+                for (int k = 0; k < kGL; ++k) {
+                    row_density(bes, nbw, chi, 0.5 * (a + t) + 0.5 * (t - a) * c_gl_x[k], dens[0], dens[1]);
+                    sum += c_gl_w[k] * (s ? dens[1] : dens[0]);
+                }
+                row_density(bes, nbw, chi, t, dens[0], dens[1]);
+                const double tn = t - (sum * 0.5 * (t - a) - T) / (s ? dens[1] : dens[0]);
+                if (!(tn >= a && tn <= a + w)) break;
+                const bool found = fabs(tn - t) <= 1e-9 * t;
+                t = tn;
+                if (found) break;
+            }
         }
-        out[m] = nbw ? 2.0 * log(t) : 3.0 * log(t);
+        icdf[((size_t)((nbw ? 2 : 0) + s) * n_chi + i) * d.n_r + m] = nbw ? 2.0 * log(t) : 3.0 * log(t);
     }
 }
 
@@ -167,46 +244,70 @@ __global__ void split_float_kernel(const double* __restrict__ a, float* hi, floa
 // taken along the ray t = e^{i pi/6} s (the integrand is analytic and bounded between the two rays):
 //   pi Gi(z) = int_0^inf exp(-s^3/3 - z s/2) sin(sqrt(3) z s/2 + pi/6) ds,
 // a decaying integrand with at most ~13 oscillations before the exponential falls below e^-46:
-// 40 panels of 12-point Gauss-Legendre on [0, min(5.2, 92/z)].
-__device__ double scorer_gi(double z) {
+// 40 panels of 12-point Gauss-Legendre on [0, min(5.2, 92/z)], the points shared out over a warp.
+__device__ double scorer_gi_warp(double z) {
     const double S = fmin(5.2, 92.0 / fmax(z, 1e-300));
     constexpr int np = 40;
     const double h = S / np, w = 0.86602540378443864676 * z, r = 0.5 * h;
     double acc = 0.0;
-    for (int p = 0; p < np; ++p) {
-        const double m = (p + 0.5) * h;
-        double ps = 0.0;
-        for (int i = 0; i < kGL; ++i) {
-            const double t = m + r * c_gl_x[i];
-            ps += c_gl_w[i] * exp(-t * t * t / 3.0 - 0.5 * z * t) * sin(w * t + kPi / 6.0);
-        }
-        acc += ps * r;
+    for (int e = threadIdx.x & 31; e < np * kGL; e += 32) {
+        const double t = (e / kGL + 0.5) * h + r * c_gl_x[e % kGL];
+        acc += c_gl_w[e % kGL] * exp(-t * t * t / 3.0 - 0.5 * z * t) * sin(w * t + kPi / 6.0);
     }
-    return acc / kPi;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc * r / kPi;
 }
 
-// One block per chi node: a(chi) = (alpha/chi) int_0^inf du u/(1+u)^3 Gi(z)/sqrt(z), z = (u/chi)^{2/3}
-// (= (alpha/chi) int_0^1 dlambda lambda Gi(z)/sqrt(z) with u = lambda/(1-lambda)), integrated in x = ln u
-// on [min(ln chi, 0) - 21, max(ln chi, 0) + 21] (the ends add below 1e-17 of the result) with panels of
-// width 1/4, one per thread, summed in a fixed tree order.  Stores ln a.
-__global__ void __launch_bounds__(256) amm_table_kernel(qed_table_desc d, double* amm64, float* amm32) {
+// a(chi) = (alpha/chi) int_0^inf du u^2/(1+u)^3 Gi(z)/sqrt(z), z = (u/chi)^{2/3}
+// (= (alpha/chi) int_0^1 dlambda lambda Gi(z)/sqrt(z) with u = lambda/(1-lambda)).  With u = chi e^v the factor
+// g(v) = Gi(e^{2v/3}) e^{-v/3} does not depend on chi, so it is taken once on nodes in v common to every row:
+// panels of width at most 1/4 from v0 = -21 - max(ln chi_max, 0) to v1 = 21 + max(-ln chi_min, 0), 12-point
+// Gauss-Legendre in each (2796 nodes for chi in [1e-4, 1e3]).  A row that took the integral on nodes of its own
+// evaluated g 2100 times, each 480 exponentials and sines: 36 ms for 256 rows against 0.16 ms for the nodes and
+// 0.06 ms for the rows (82-86 % of the FP64 pipe's cycles).
+struct AmmGrid {
+    double v0, h;
+    int panels;
+};
+
+static AmmGrid amm_grid(const qed_table_desc& d) {
+    AmmGrid g;
+    g.v0 = -21.0 - std::max(std::log(d.chi_max), 0.0);
+    const double v1 = 21.0 + std::max(-std::log(d.chi_min), 0.0);
+    g.panels = (int)std::ceil((v1 - g.v0) * 4.0);
+    g.h = (v1 - g.v0) / g.panels;
+    return g;
+}
+
+__device__ __forceinline__ double amm_node(const AmmGrid& G, int k) {
+    return G.v0 + (k / kGL + 0.5) * G.h + 0.5 * G.h * c_gl_x[k % kGL];
+}
+
+// one warp per node: g(v) with its quadrature weight
+__global__ void __launch_bounds__(128) amm_nodes_kernel(AmmGrid G, double* gv) {
+    const int k = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    if (k >= G.panels * kGL) return;
+    const double sz = exp(amm_node(G, k) / 3.0);  // sqrt(z)
+    const double gi = scorer_gi_warp(sz * sz);
+    if ((threadIdx.x & 31) == 0) gv[k] = c_gl_w[k % kGL] * 0.5 * G.h * gi / sz;
+}
+
+// One block per chi node; x = ln u runs over [min(ln chi, 0) - 21, max(ln chi, 0) + 21] (the ends add below
+// 1e-17 of the result), summed in a fixed tree order.  Stores ln a.
+__global__ void __launch_bounds__(256) amm_table_kernel(qed_table_desc d, AmmGrid G, const double* __restrict__ gv,
+                                                        double* amm64, float* amm32) {
     __shared__ double part[256];
     const int i = blockIdx.x;
     const double dl = (log(d.chi_max) - log(d.chi_min)) / (d.n_chi - 1);
     const double lnchi = log(d.chi_min) + i * dl, chi = exp(lnchi);
     const double x0 = fmin(lnchi, 0.0) - 21.0, x1 = fmax(lnchi, 0.0) + 21.0;
-    const int np = (int)ceil((x1 - x0) * 4.0);
-    const double h = (x1 - x0) / np, r = 0.5 * h;
     double acc = 0.0;
-    for (int p = threadIdx.x; p < np; p += blockDim.x) {
-        const double m = x0 + (p + 0.5) * h;
-        for (int k = 0; k < kGL; ++k) {
-            const double x = m + r * c_gl_x[k];
-            const double u = exp(x);
-            const double sz = exp((x - lnchi) / 3.0);  // sqrt(z) = (u/chi)^{1/3}
-            const double q = 1.0 / (1.0 + u);
-            acc += c_gl_w[k] * r * u * u * q * q * q * scorer_gi(sz * sz) / sz;
-        }
+    for (int k = threadIdx.x; k < G.panels * kGL; k += blockDim.x) {
+        const double x = amm_node(G, k) + lnchi;
+        if (x < x0 || x > x1) continue;
+        const double u = exp(x);
+        const double q = 1.0 / (1.0 + u);
+        acc += gv[k] * u * u * q * q * q;
     }
     part[threadIdx.x] = acc;
     __syncthreads();
@@ -227,15 +328,7 @@ using namespace qed;
 
 static void free_tables(qed_tables_s* t) {
     if (!t) return;
-    cudaFree(t->rate64);
-    cudaFree(t->icdf64);
-    cudaFree(t->rate32);
-    cudaFree(t->icdf32);
-    cudaFree(t->icdf32lo);
-    cudaFree(t->bes64);
-    cudaFree(t->bes32);
-    cudaFree(t->amm64);
-    cudaFree(t->amm32);
+    cudaFree(t->rate64);  // the start of the tables' one allocation
     t->magic = 0;
     delete t;
 }
@@ -254,31 +347,58 @@ extern "C" qed_status qed_tables_build(const qed_table_desc* desc, qed_tables_t*
     t->desc = d;
     cudaGetDevice(&t->device);
     const size_t nr = 4 * (size_t)d.n_chi, ni = 4 * (size_t)d.n_chi * d.n_r;
-    bool ok = cudaMalloc(&t->rate64, nr * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&t->icdf64, ni * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&t->rate32, nr * sizeof(float)) == cudaSuccess &&
-              cudaMalloc(&t->icdf32, ni * sizeof(float)) == cudaSuccess &&
-              cudaMalloc(&t->icdf32lo, ni * sizeof(float)) == cudaSuccess &&
-              cudaMalloc(&t->bes64, 3 * kBesN * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&t->bes32, 3 * kBesN * sizeof(float)) == cudaSuccess &&
-              cudaMalloc(&t->amm64, d.n_chi * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&t->amm32, d.n_chi * sizeof(float)) == cudaSuccess;
-    if (!ok) {
+    const AmmGrid G = amm_grid(d);
+    // one allocation for every table and the scratch of the a(chi) nodes (nine took 0.1 ms to make and free)
+    size_t bytes = 0;
+    auto place = [&bytes](size_t n) {
+        const size_t at = bytes;
+        bytes += (n + 255) & ~size_t(255);
+        return at;
+    };
+    const size_t at[10] = {place(nr * sizeof(double)),        place(ni * sizeof(double)),
+                           place(nr * sizeof(float)),         place(ni * sizeof(float)),
+                           place(ni * sizeof(float)),         place(3 * kBesN * sizeof(double)),
+                           place(3 * kBesN * sizeof(float)),  place(d.n_chi * sizeof(double)),
+                           place(d.n_chi * sizeof(float)),    place((size_t)G.panels * kGL * sizeof(double))};
+    unsigned char* mem = nullptr;
+    if (cudaMalloc(&mem, bytes) != cudaSuccess) {
+        cudaGetLastError();
         free_tables(t);
         return QED_ERR_NOMEM;
     }
-    double glx[kGL], glw[kGL];
+    t->rate64 = (double*)(mem + at[0]);
+    t->icdf64 = (double*)(mem + at[1]);
+    t->rate32 = (float*)(mem + at[2]);
+    t->icdf32 = (float*)(mem + at[3]);
+    t->icdf32lo = (float*)(mem + at[4]);
+    t->bes64 = (double*)(mem + at[5]);
+    t->bes32 = (float*)(mem + at[6]);
+    t->amm64 = (double*)(mem + at[7]);
+    t->amm32 = (float*)(mem + at[8]);
+    double* gv = (double*)(mem + at[9]);
+    double glx[kGL], glw[kGL], leg[kGL][kGL];
     gauss_legendre(kGL, glx, glw);
+    for (int i = 0; i < kGL; ++i) {
+        double p0 = 1.0, p1 = glx[i];
+        for (int k = 0; k < kGL; ++k) {
+            leg[k][i] = (k + 0.5) * glw[i] * p0;
+            const double p2 = ((2.0 * k + 3.0) * glx[i] * p1 - (k + 1.0) * p0) / (k + 2.0);
+            p0 = p1;
+            p1 = p2;
+        }
+    }
     if (cudaMemcpyToSymbolAsync(c_gl_x, glx, sizeof(glx), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_gl_w, glw, sizeof(glw), 0, cudaMemcpyHostToDevice, st) != cudaSuccess) {
+        cudaMemcpyToSymbolAsync(c_gl_w, glw, sizeof(glw), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(c_legendre, leg, sizeof(leg), 0, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         free_tables(t);
         return QED_ERR_CUDA;
     }
-    bessel_table_kernel<<<(kBesN + 127) / 128, 128, 0, st>>>(t->bes64, t->bes32);
-    table_rows_kernel<<<4 * d.n_chi, 256, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
+    bessel_table_kernel<<<(kBesN + 3) / 4, 128, 0, st>>>(t->bes64, t->bes32);
+    table_rows_kernel<<<2 * d.n_chi, 256, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
     to_float_kernel<<<64, 256, 0, st>>>(t->rate64, t->rate32, nr);
     split_float_kernel<<<256, 256, 0, st>>>(t->icdf64, t->icdf32, t->icdf32lo, ni);
-    amm_table_kernel<<<d.n_chi, 256, 0, st>>>(d, t->amm64, t->amm32);
+    amm_nodes_kernel<<<(G.panels * kGL + 3) / 4, 128, 0, st>>>(G, gv);
+    amm_table_kernel<<<d.n_chi, 256, 0, st>>>(d, G, gv, t->amm64, t->amm32);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
         free_tables(t);
         return QED_ERR_CUDA;
