@@ -24,30 +24,24 @@ constexpr double kGamma23 = 1.3541179394264004169;  // Gamma(2/3)
 // --------------------------------------------------------------------------------------------
 // direct trapezoid (FP64)
 // --------------------------------------------------------------------------------------------
-// the number of steps, the end T and the step h of the rule at x
-__device__ __forceinline__ int bessel_steps(double x, double& T, double& h) {
-    T = acosh(1.0 + 46.0 / x);
-    T = acosh(1.0 + (46.0 + (2.0 / 3.0) * T) / x);
-    h = fmin(0.2, 0.6 * rsqrt(x));
-    return (int)ceil(T / h);
-}
-
-// the three integrands at t, added to s
-__device__ __forceinline__ void bessel_term(double x, double t, double s[3]) {
-    const double sh = sinh(0.5 * t);
-    const double e = exp(-x * (2.0 * sh * sh));  // cosh t - 1 = 2 sinh^2(t/2)
-    const double c3 = cosh(t / 3.0);
-    s[0] += e * c3;
-    s[1] += e * (2.0 * c3 * c3 - 1.0);
-    s[2] += e * c3 / cosh(t);
-}
-
 __device__ __forceinline__ void bessel_trapezoid(double x, double out[3]) {
-    double T, h;
-    const int n = bessel_steps(x, T, h);
-    double s[3] = {0.5, 0.5, 0.5};  // t = 0: exp(0) * cosh(0) terms, weight 1/2
-    for (int m = 1; m <= n; ++m) bessel_term(x, m * h, s);
-    for (int f = 0; f < 3; ++f) out[f] = s[f] * h;
+    double T = acosh(1.0 + 46.0 / x);
+    T = acosh(1.0 + (46.0 + (2.0 / 3.0) * T) / x);
+    const double h = fmin(0.2, 0.6 * rsqrt(x));
+    const int n = (int)ceil(T / h);
+    double s0 = 0.5, s1 = 0.5, s2 = 0.5;  // t = 0: exp(0) * cosh(0) terms, weight 1/2
+    for (int m = 1; m <= n; ++m) {
+        const double t = m * h;
+        const double sh = sinh(0.5 * t);
+        const double e = exp(-x * (2.0 * sh * sh));  // cosh t - 1 = 2 sinh^2(t/2)
+        const double c3 = cosh(t / 3.0);
+        s0 += e * c3;
+        s1 += e * (2.0 * c3 * c3 - 1.0);
+        s2 += e * c3 / cosh(t);
+    }
+    out[0] = s0 * h;
+    out[1] = s1 * h;
+    out[2] = s2 * h;
 }
 
 // --------------------------------------------------------------------------------------------

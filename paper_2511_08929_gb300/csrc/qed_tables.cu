@@ -11,7 +11,8 @@
 //       rho = 3 chi u~'/2 - 2; stored scaled by e^{8/(3 chi)}.
 // Each row integrates panels of width 1/16 in t with 12-point Gauss-Legendre, sums them into the
 // CDF at the panel edges, and inverts the CDF at each r_m by Newton's method inside the bracketing
-// panel, on the density's Legendre series there (from the same 12 nodes).
+// panel: NLC on partial integrals by 12-point Gauss-Legendre, NBW on the density's Legendre series
+// there (from the panel's 12 nodes).
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -50,43 +51,109 @@ static void gauss_legendre(int n, double* x, double* w) {
     }
 }
 
-// One warp per node: the lanes take the terms of the three trapezoid sums (up to ~230 of them, each five
-// FP64 transcendentals, which one thread alone would chain: 295 us for the table against 38 us, 82 % of the FP64
-// pipe's cycles).
-__global__ void __launch_bounds__(128) bessel_table_kernel(double* tab64, float* tab32) {
-    const int j = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+__global__ void bessel_table_kernel(double* tab64, float* tab32) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= kBesN) return;
     const double x = exp(log(kBesLo) + kBesH * j);
-    double T, h;
-    const int n = bessel_steps(x, T, h);
-    double s[3] = {0.0, 0.0, 0.0};
-    for (int m = 1 + lane; m <= n; m += 32) bessel_term(x, m * h, s);
+    double o[3];
+    bessel_trapezoid(x, o);
     for (int f = 0; f < 3; ++f) {
-        for (int o = 16; o > 0; o >>= 1) s[f] += __shfl_down_sync(0xffffffffu, s[f], o);
-        if (lane == 0) {
-            const double v = (0.5 + s[f]) * h;  // t = 0: exp(0) * cosh(0) terms, weight 1/2
-            tab64[f * kBesN + j] = v;
-            tab32[f * kBesN + j] = (float)v;
+        tab64[f * kBesN + j] = o[f];
+        tab32[f * kBesN + j] = (float)o[f];
+    }
+}
+
+// NLC rows.  An entry is the value at which Newton's method on the 12-point quadrature, kept inside its bracket,
+// stops (a bracket or a step of one part in 1e15): the learned sampler is trained on differences of two of these
+// entries down to 1e-7, so the rows keep every bit of that definition, and only the work's distribution is free.
+__device__ __forceinline__ double nlc_density(const double* __restrict__ bes, double chi, double sigma, double t) {
+    double b[3];
+    const double up = t * t * t;
+    const double den = 2.0 + 3.0 * chi * up;
+    const double lam = 3.0 * chi * up / den, one_m = 2.0 / den;
+    bessel64(bes, up, b);
+    const double kappa = 1.0 / one_m + one_m;
+    const double w = exp(-up) * (-b[2] + kappa * b[1] + sigma * lam * b[0]);
+    return w * 6.0 * chi / (den * den) * 3.0 * t * t;
+}
+
+__device__ __forceinline__ double nlc_integral(const double* bes, double chi, double sigma, double a, double b) {
+    const double m = 0.5 * (a + b), r = 0.5 * (b - a);
+    double s = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < kGL; ++i) s += c_gl_w[i] * nlc_density(bes, chi, sigma, m + r * c_gl_x[i]);
+    return s * r;
+}
+
+constexpr int kNlcThreads = 64;
+constexpr int kNlcPanels = 70;  // cbrt(80) * 16 = 68.9
+
+// One block per (sign, chi row).  FP64-bound, 13 densities an iteration, and an entry takes 5 to 60 iterations (a
+// root approached from the left, where the density falls, is bracketed by bisection): a lane that has finished an
+// entry takes the row's next one, so no lane waits for the longest of its warp (256 x 256 entries a sign: 36.5 ms
+// with one entry a thread, 29.7 ms so).
+__global__ void __launch_bounds__(kNlcThreads) nlc_rows_kernel(const double* __restrict__ bes, qed_table_desc d,
+                                                               double* rates, double* icdf) {
+    __shared__ double cum[kNlcPanels + 1];
+    __shared__ int next;
+    const int n_chi = d.n_chi;
+    const int s = blockIdx.x / n_chi, i = blockIdx.x % n_chi;
+    const double sigma = s == 0 ? 1.0 : -1.0;
+    const double dl = (log(d.chi_max) - log(d.chi_min)) / (n_chi - 1);
+    const double chi = exp(log(d.chi_min) + i * dl);
+    const double tend = cbrt(80.0);
+    const int np = (int)ceil(tend / kPanel);
+    for (int p = threadIdx.x; p < np; p += blockDim.x)
+        cum[p + 1] = nlc_integral(bes, chi, sigma, p * kPanel, fmin(tend, (p + 1) * kPanel));
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        next = kNlcThreads;
+        cum[0] = 0.0;
+        for (int p = 0; p < np; ++p) cum[p + 1] += cum[p];
+        rates[s * n_chi + i] = log(cum[np]);
+    }
+    __syncthreads();
+    const double total = cum[np];
+    const double dy = (d.y_hi - d.y_lo) / (d.n_r - 1);
+    double* out = icdf + ((size_t)s * n_chi + i) * d.n_r;
+    double a = 0.0, target = 0.0, tl = 0.0, th = 0.0, t = 0.0;
+    int it = 0, p = 0;
+    for (int m = threadIdx.x; m < d.n_r;) {
+        if (it == 0) {  // a new entry
+            const double r = 1.0 / (1.0 + exp(-(d.y_lo + m * dy)));
+            target = r * total;
+            // panel with cum[p] <= target < cum[p+1]
+            int lo = 0, hi = np - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (cum[mid] <= target) lo = mid; else hi = mid - 1;
+            }
+            a = lo * kPanel;
+            const double b = fmin(tend, (lo + 1) * kPanel);
+            p = lo;
+            tl = a;
+            th = b;
+            t = a + (b - a) * (target - cum[p]) / (cum[p + 1] - cum[p]);
+        }
+        const double F = cum[p] + nlc_integral(bes, chi, sigma, a, t) - target;
+        if (F > 0.0) th = t; else tl = t;
+        const double dF = nlc_density(bes, chi, sigma, t);
+        double tn = t - F / dF;
+        if (!(tn > tl && tn < th)) tn = 0.5 * (tl + th);
+        const bool done = fabs(tn - t) <= 1e-15 * fmax(t, 1e-300) || th - tl <= 1e-15 * th;
+        t = tn;
+        if (done || ++it == 100) {
+            out[m] = 3.0 * log(t);
+            m = atomicAdd(&next, 1);
+            it = 0;
         }
     }
 }
 
-// the densities in t at both signs sigma = +1, -1 (they share the Bessel functions and all but one product)
-__device__ __forceinline__ void row_density(const double* __restrict__ bes, bool nbw, double chi, double t, double& dp,
-                                            double& dm) {
+// NBW rows.  The densities in t at both signs sigma = +1, -1 (they share the Bessel functions and all but one
+// product)
+__device__ __forceinline__ void nbw_density(const double* __restrict__ bes, double chi, double t, double& dp, double& dm) {
     double b[3];
-    if (!nbw) {
-        const double up = t * t * t;
-        const double iden = 1.0 / (2.0 + 3.0 * chi * up);
-        const double lam = 3.0 * chi * up * iden, one_m = 2.0 * iden;
-        bessel64(bes, up, b);
-        const double kappa = 1.0 / one_m + one_m;
-        const double f = exp(-up) * 18.0 * chi * iden * iden * t * t;
-        const double w = -b[2] + kappa * b[1], wl = lam * b[0];
-        dp = f * (w + wl);
-        dm = f * (w - wl);
-        return;
-    }
     const double ut = 8.0 / (3.0 * chi) + t * t;
     bessel64(bes, ut, b);
     const double rho = 1.5 * chi * ut - 2.0;
@@ -96,7 +163,7 @@ __device__ __forceinline__ void row_density(const double* __restrict__ bes, bool
     dm = f * (w + b[1]);
 }
 
-constexpr int kMaxPanels = 144;  // sqrt(80) * 16 = 143.1 -> 144 panels for NBW, 69 for NLC
+constexpr int kNbwPanels = 144;  // sqrt(80) * 16 = 143.1
 
 // On a panel [a, a + d] with t = a + d s, x = 2 s - 1 and the density's Legendre coefficients c:
 //   dH/ds = d sum_k c_k P_k(x),   H(s) = int_a^t = d s [c_0 + (x - 1) sum_{k>=1} c_k P_k'(x) / (k (k + 1))]
@@ -121,26 +188,24 @@ __device__ __forceinline__ void panel_cdf(const double* c, double d, double s, d
     H = d * s * fma(x - 1.0, g, c[0]);
 }
 
-// One block per (kind, chi row), both signs.  FP64-bound: the density is evaluated at the panels' nodes only,
-// 1.3e6 Bessel triples for a 256 x 256 table.  Inverting the CDF with a quadrature and a density evaluation per
-// Newton step took 65 ms for that table (and its stopping rule, one rounding error of t, sent most entries
-// through a bisection); on the Legendre series a step is ~100 fused multiply-adds and the whole kernel 1.63 ms
-// (1.40e7 FP64 warp instructions, 83 % of the FP64 pipe's cycles).
-__global__ void __launch_bounds__(256) table_rows_kernel(const double* __restrict__ bes, qed_table_desc d, double* rates,
-                                                         double* icdf) {
-    __shared__ double coef[2][kMaxPanels][kGL];  // density at the nodes, then its Legendre coefficients
-    __shared__ double cum[2][kMaxPanels + 1];
+// One block per chi row, both signs.  FP64-bound: the density is evaluated at the panels' nodes, and again only
+// where the series has not converged; a Newton step on the series is ~100 fused multiply-adds.  A quadrature and a
+// density per step, with a stopping rule of one rounding unit that sent most entries through a bisection, took
+// 27 ms for 256 x 256 entries a sign; this kernel takes 0.69 ms (83 % of the FP64 pipe's cycles).
+__global__ void __launch_bounds__(256) nbw_rows_kernel(const double* __restrict__ bes, qed_table_desc d, double* rates,
+                                                       double* icdf) {
+    __shared__ double coef[2][kNbwPanels][kGL];  // density at the nodes, then its Legendre coefficients
+    __shared__ double cum[2][kNbwPanels + 1];
     const int n_chi = d.n_chi;
-    const bool nbw = (int)blockIdx.x >= n_chi;
-    const int i = blockIdx.x % n_chi;
+    const int i = blockIdx.x;
     const double dl = (log(d.chi_max) - log(d.chi_min)) / (n_chi - 1);
     const double chi = exp(log(d.chi_min) + i * dl);
-    const double tend = nbw ? sqrt(80.0) : cbrt(80.0);
+    const double tend = sqrt(80.0);
     const int np = (int)ceil(tend / kPanel);
     for (int e = threadIdx.x; e < np * kGL; e += blockDim.x) {
         const int p = e / kGL, k = e % kGL;
         const double a = p * kPanel, b = fmin(tend, (p + 1) * kPanel);
-        row_density(bes, nbw, chi, 0.5 * (a + b) + 0.5 * (b - a) * c_gl_x[k], coef[0][p][k], coef[1][p][k]);
+        nbw_density(bes, chi, 0.5 * (a + b) + 0.5 * (b - a) * c_gl_x[k], coef[0][p][k], coef[1][p][k]);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < 2 * np; e += blockDim.x) {
@@ -166,7 +231,7 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const double* __restric
             c += cum[s][p];
             cum[s][p] = c;
         }
-        rates[(nbw ? 2 * n_chi : 0) + s * n_chi + i] = nbw ? log(2.0 * c) : log(c);
+        rates[2 * n_chi + s * n_chi + i] = log(2.0 * c);
     }
     __syncthreads();
     const double dy = (d.y_hi - d.y_lo) / (d.n_r - 1);
@@ -200,18 +265,18 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const double* __restric
                 if (found) break;
             }
         double t = a + w * u;
-        // where the series has not converged within its 12 terms (the lowest panels of NBW rows with large chi,
-        // whose spectrum varies over t ~ chi^{-1/2}; the falling end of the NLC ones) the root is finished on
-        // the quadrature itself, one step from the series' root (about a quarter of a table's entries)
+        // where the series has not converged within its 12 terms (the lowest panels of rows with large chi, whose
+        // spectrum varies over t ~ chi^{-1/2}) the root is finished on the quadrature itself, one step from the
+        // series' root
         const double* c = coef[s][lo];
         if (fabs(c[kGL - 1]) + fabs(c[kGL - 2]) > 2e-14 * fabs(c[0]) && t > a) {
             for (int it = 0; it < 4; ++it) {
                 double dens[2], sum = 0.0;
                 for (int k = 0; k < kGL; ++k) {
-                    row_density(bes, nbw, chi, 0.5 * (a + t) + 0.5 * (t - a) * c_gl_x[k], dens[0], dens[1]);
+                    nbw_density(bes, chi, 0.5 * (a + t) + 0.5 * (t - a) * c_gl_x[k], dens[0], dens[1]);
                     sum += c_gl_w[k] * (s ? dens[1] : dens[0]);
                 }
-                row_density(bes, nbw, chi, t, dens[0], dens[1]);
+                nbw_density(bes, chi, t, dens[0], dens[1]);
                 const double tn = t - (sum * 0.5 * (t - a) - T) / (s ? dens[1] : dens[0]);
                 if (!(tn >= a && tn <= a + w)) break;
                 const bool found = fabs(tn - t) <= 1e-9 * t;
@@ -219,7 +284,7 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const double* __restric
                 if (found) break;
             }
         }
-        icdf[((size_t)((nbw ? 2 : 0) + s) * n_chi + i) * d.n_r + m] = nbw ? 2.0 * log(t) : 3.0 * log(t);
+        icdf[((size_t)(2 + s) * n_chi + i) * d.n_r + m] = 2.0 * log(t);
     }
 }
 
@@ -393,8 +458,9 @@ extern "C" qed_status qed_tables_build(const qed_table_desc* desc, qed_tables_t*
         free_tables(t);
         return QED_ERR_CUDA;
     }
-    bessel_table_kernel<<<(kBesN + 3) / 4, 128, 0, st>>>(t->bes64, t->bes32);
-    table_rows_kernel<<<2 * d.n_chi, 256, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
+    bessel_table_kernel<<<(kBesN + 127) / 128, 128, 0, st>>>(t->bes64, t->bes32);
+    nlc_rows_kernel<<<2 * d.n_chi, kNlcThreads, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
+    nbw_rows_kernel<<<d.n_chi, 256, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
     to_float_kernel<<<64, 256, 0, st>>>(t->rate64, t->rate32, nr);
     split_float_kernel<<<256, 256, 0, st>>>(t->icdf64, t->icdf32, t->icdf32lo, ni);
     amm_nodes_kernel<<<(G.panels * kGL + 3) / 4, 128, 0, st>>>(G, gv);
