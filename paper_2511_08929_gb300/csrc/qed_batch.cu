@@ -2,7 +2,7 @@
 // time step, the step index and time on the device (so a CUDA graph of whole steps replays unchanged),
 // and an autotuner for the launch shape.
 //
-// One time step of the batch is seven launches on one stream:
+// One time step of the batch is eight launches on one stream:
 //   plan      alive counts at step start (counts clamped to capacity), the tile list over all segments
 //             (segment = one species of one instance, species-major), each segment's step context,
 //             particle-step accounting;
@@ -14,7 +14,8 @@
 //             the step's event list, 32 entries per atomic add;
 //   events    the event branch for every listed particle, 32 per warp with a context per lane (out of
 //             the persistent kernel, whose registers then hold only the streaming pass: no calls, no
-//             spills);
+//             spills): one kernel for the lepton events in FP32, one for what is FP64 (the photon events,
+//             and the lepton events whose FP32 spectra cancel);
 //   compact   head / classify / tail / move of every instance's photons (converted photons leave,
 //             Sec. 4.3), the last one also advancing the device step counter.
 // Daughters appended during a step sit beyond the counts taken by `plan`, so they are first stepped in
@@ -58,7 +59,9 @@ struct ClockDev {
     unsigned long long species_steps[kSpecies];
     long long alive[kSpecies];
     int next_tile;  // the persistent kernel's work counter (tiles handed out), reset by the plan kernel
-    unsigned long long n_events;  // entries in the step's event list, reset by the plan kernel
+    unsigned long long n_list[2];  // the step's listed events (leptons, photons), reset by the plan kernel
+    unsigned long long n_exact;    // lepton events to be taken again in FP64, reset by the plan kernel
+    unsigned long long n_events;   // events of the last step (both kinds)
 };
 
 struct BatchP {
@@ -164,7 +167,7 @@ __global__ void __launch_bounds__(kPlanThreads)
     }
     if (threadIdx.x == 0) {
         clk->next_tile = 0;
-        clk->n_events = 0;
+        clk->n_list[0] = clk->n_list[1] = clk->n_exact = 0;
         clk->psteps += tot[0] + tot[1] + tot[2];
         for (int k = 0; k < kSpecies; ++k) {
             clk->species_steps[k] += tot[k];
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     batch_step_kernel(TabP<float> T, float* bes_g, const InstDev* __restrict__ inst,
                       const SegDev* __restrict__ seg, const int64_t* __restrict__ tile0_g, int n_inst,
                       const ClockDev* __restrict__ clk, BatchP P, int chunk, int* work, long long* ev,
-                      unsigned long long* n_ev, qed_counters* ctr) {
+                      long long ev_cap, unsigned long long* n_ev, qed_counters* ctr) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int n_seg = kSpecies * n_inst;
     Shared32 sh;
@@ -322,7 +325,16 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     __syncwarp();
     int2 ch = ring[0];
     int t = ch.x, te = ch.y, rk = 1;  // the compute walk: tile t of a chunk ending at te; ring entries read
-    int qn = 0;    // queued event entries, segment << 32 | index (warp-uniform), flushed 32 at a time
+    // queued event entries, segment << 32 | index (warp-uniform), flushed 32 at a time: leptons' to the front of the
+    // step's event list, photons' (which every warp reaches after its last lepton tile) to its back
+    int qn = 0;
+    auto flush = [&](int from, int cnt, int photons) {
+        const unsigned long long base =
+            __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(&n_ev[photons], (unsigned long long)cnt) : 0ull, 0);
+        const long long at = (long long)base + lane;
+        if (lane < cnt) ev[photons ? ev_cap - 1 - at : at] = wq[from + lane];
+        __syncwarp();
+    };
     int cur = -1;  // current segment
     int sp = 0, ii = 0;
     int st = 0;  // stage of the current tile
@@ -331,6 +343,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
         if (t >= WS.t1) {  // the tile lies in a later segment
             do ++cur;
             while (s_tile0[cur + 1] <= t);
+            if (cur >= 2 * n_inst && sp < 2 && qn > 0) {  // from leptons to photons
+                flush(0, qn, 0);
+                qn = 0;
+            }
             sp = cur / n_inst;
             ii = cur - sp * n_inst;
             __syncwarp();
@@ -400,10 +416,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
         qn += __popc(m);
         __syncwarp();
         if (qn >= 32) {  // 32 entries to the step's event list with one atomic add
-            const unsigned long long base = __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(n_ev, 32ull) : 0ull, 0);
-            ev[base + lane] = wq[qn - 32 + lane];
             qn -= 32;
-            __syncwarp();
+            flush(qn, 32, sp == 2);
         }
         if (++t == te) {  // the chunk is done: the next one (its entry was written when its copies began)
             ch = ring[rk++ & (kChunkRing - 1)];
@@ -412,97 +426,113 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
         }
     }
     cp_async_wait<0>();  // no copy outlives the kernel (the trailing groups are empty)
-    if (qn > 0) {
-        const unsigned long long base =
-            __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(n_ev, (unsigned long long)qn) : 0ull, 0);
-        if (lane < qn) ev[base + lane] = wq[lane];
-    }
+    if (qn > 0) flush(0, qn, sp == 2);
     flush_warp(c, ctr);
 }
 
 // ------------------------------------------------------------------------------------------------
 // the event pass of the step: every event the persistent kernel listed (a particle whose optical depth
-// ran out, left untouched by it), 32 per warp, each lane with the context of its own segment
+// ran out, left untouched by it), 32 per warp, each lane with the context of its own segment.  Two kernels:
+//   batch_event_kernel    the lepton events (FP32); those whose spectra cancel go to a list
+//   batch_event64_kernel  the photon events and that list (FP64 after the decision), in full warps
+// Chunk c of 32 events goes to block c mod grid, so few events spread over all SMs: consecutive chunks in one
+// block shared one SM's FP64 pipe (8 warps x 16 cycles an instruction), 76-152 us a step for 1e3 events.
 // ------------------------------------------------------------------------------------------------
 constexpr int kEventThreads = 256;
+constexpr int kEvent64Threads = 128;
+
+__device__ __forceinline__ unsigned long long first_chunk() {
+    return (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+}
+
+// the list of the events taken again in FP64: the free middle of the event list (lepton events in front, photon
+// events at the back, three words an entry)
+__device__ __forceinline__ ExactList exact_list(long long* ev, long long ev_cap, ClockDev* clk) {
+    const unsigned long long n = clk->n_list[0];
+    return ExactList{ev + n, &clk->n_exact, ((unsigned long long)ev_cap - n - clk->n_list[1]) / 3};
+}
 
 // (two blocks per SM: the register cap keeps 16 warps per SM to hide the global-memory latency of the
 // event branch)
 __global__ void __launch_bounds__(kEventThreads, 2) batch_event_kernel(const InstDev* __restrict__ inst,
-                                                                   const SegCtx* __restrict__ ctx,
-                                                                   const long long* __restrict__ ev,
-                                                                   const ClockDev* __restrict__ clk, Tab64 X64,
+                                                                   const SegCtx* __restrict__ ctx, long long* ev,
+                                                                   long long ev_cap, ClockDev* clk, Tab64 X64,
                                                                    qed_counters* ctr,
                                                                    const float* __restrict__ lnup = nullptr) {
-    __shared__ ExactQ eq[kEventThreads / 32];  // per warp: the events taken again in FP64
-    const unsigned long long n = clk->n_events;
+    const unsigned long long n = clk->n_list[0];
+    const ExactList q = exact_list(ev, ev_cap, clk);
     unsigned long long c[C_N] = {};
     const int lane = threadIdx.x & 31;
-    ExactQ& q = eq[threadIdx.x >> 5];
-    if (lane == 0) q.n = 0;
-    __syncwarp();
-    // lanes take queued entries [from, from + cnt), each with the context of its own segment
-    auto drain = [&](int from, int cnt) {
-        if (lane < cnt) {
-            const int key = q.key[from + lane];
-            const SegCtx& X = ctx[key & 0x3FFFFFFF];
-            const InstDev& I = inst[X.ii];
-            lepton_exact_one(X.C, X64, I.F64, I.sp[X.sp], I.sp[2], q.j[from + lane], q.slot[from + lane],
-                             (key >> 30) & 1, lnup != nullptr, q.lnu[from + lane]);
-        }
-        __syncwarp();
-    };
     const unsigned long long warps = (unsigned long long)gridDim.x * (kEventThreads / 32);
-    for (unsigned long long k = ((unsigned long long)blockIdx.x * (kEventThreads / 32) + (threadIdx.x >> 5)) * 32; k < n;
-         k += warps * 32) {
+    for (unsigned long long k = first_chunk() * 32; k < n; k += warps * 32) {
         const long long e = k + lane < n ? ev[k + lane] : -1;
         const int seg0 = __shfl_sync(0xffffffffu, (int)(e >> 32), 0);  // lane 0 always holds an entry
         const int s = e >= 0 ? (int)(e >> 32) : seg0;
-        const int64_t j = e >= 0 ? (int64_t)(uint32_t)e : -1;
         const SegCtx& X = ctx[s];
         const InstDev& I = inst[X.ii];
-        const bool ph = X.sp == 2;
         const float lnu = lnup != nullptr && e >= 0 ? lnup[4 * (k + lane)] : 0.0f;  // the learned sampler's ln u'
-        // both passes are warp-collective; a lane takes part in the one of its species with its particle
-        if (__ballot_sync(0xffffffffu, j >= 0 && !ph))
-            lepton_events(X.C, X64, I.F64, ph ? -1 : j, I.sp[ph ? 0 : X.sp], I.sp[2], &I.app[0], ctr, c, &q, s,
-                          lnup != nullptr, lnu);
-        if (__ballot_sync(0xffffffffu, j >= 0 && ph))
-            photon_events(X.C, X64, ph ? j : -1, I.sp[2], I.sp[0], I.sp[1], &I.app[1], ctr, c);
-        const int qn = q.n;
-        if (qn >= 32) {  // 32 queued events in FP64 with every lane busy
-            drain(qn - 32, 32);
-            if (lane == 0) q.n = qn - 32;
+        lepton_events(X.C, X64, I.F64, e >= 0 ? (int64_t)(uint32_t)e : -1, I.sp[X.sp], I.sp[2], &I.app[0], ctr, c, &q,
+                      e, lnup != nullptr, lnu);
+    }
+    flush_warp(c, ctr);
+}
+
+__global__ void __launch_bounds__(kEvent64Threads) batch_event64_kernel(const InstDev* __restrict__ inst,
+                                                                      const SegCtx* __restrict__ ctx, long long* ev,
+                                                                      long long ev_cap, ClockDev* clk, Tab64 X64,
+                                                                      qed_counters* ctr, bool net) {
+    const unsigned long long n = clk->n_list[1], nc = (n + 31) / 32;
+    const ExactList q = exact_list(ev, ev_cap, clk);
+    const unsigned long long nx = min(*q.n, q.cap), xc = (nx + 31) / 32;
+    unsigned long long c[C_N] = {};
+    const int lane = threadIdx.x & 31;
+    const unsigned long long warps = (unsigned long long)gridDim.x * (kEvent64Threads / 32);
+    for (unsigned long long k = first_chunk(); k < nc + xc; k += warps) {
+        if (k < nc) {  // (warp-uniform)
+            const unsigned long long i = k * 32 + lane;
+            const long long e = i < n ? ev[ev_cap - 1 - (long long)i] : -1;
+            const int seg0 = __shfl_sync(0xffffffffu, (int)(e >> 32), 0);
+            const SegCtx& X = ctx[e >= 0 ? (int)(e >> 32) : seg0];
+            const InstDev& I = inst[X.ii];
+            photon_events(X.C, X64, e >= 0 ? (int64_t)(uint32_t)e : -1, I.sp[2], I.sp[0], I.sp[1], &I.app[1], ctr, c);
+        } else {
+            const unsigned long long i = (k - nc) * 32 + lane;
+            if (i < nx) {
+                const long long e = q.item[3 * i];
+                const SegCtx& X = ctx[(int)((e >> 32) & 0x3FFFFFFF)];
+                const InstDev& I = inst[X.ii];
+                lepton_exact_one(X.C, X64, I.F64, I.sp[X.sp], I.sp[2], (int64_t)(uint32_t)e, q.item[3 * i + 1],
+                                 (e >> 62) & 1, net, __uint_as_float((unsigned)q.item[3 * i + 2]));
+            }
             __syncwarp();
         }
     }
-    drain(0, q.n);
     flush_warp(c, ctr);
 }
 
 // ------------------------------------------------------------------------------------------------
 // the learned sampler's inputs for every listed event (Sec. 5.1): a lepton's (chi, r2, s.beta) as its
 // event will see them (the streaming pass's classical step with accurate fields; r2 the uniform of its
-// energy-fraction draw, which the ICDF row would take); a pair event gets placeholders (chi 1, r 1/2,
-// s 0) and lep 0, so that list position k is sample k
+// energy-fraction draw, which the ICDF row would take), list position k being sample k; the pair events follow
+// with placeholders (chi 1, r 1/2, s 0) and lep 0
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) batch_mlp_prep_kernel(const InstDev* __restrict__ inst,
                                                              const SegCtx* __restrict__ ctx,
-                                                             const long long* __restrict__ ev,
-                                                             const ClockDev* __restrict__ clk, double* chi, double* r,
-                                                             double* sb, uint8_t* lep) {
-    const unsigned long long n = clk->n_events;
-    for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+                                                             const long long* __restrict__ ev, ClockDev* clk,
+                                                             double* chi, double* r, double* sb, uint8_t* lep) {
+    const unsigned long long n = clk->n_list[0], all = n + clk->n_list[1];
+    if (blockIdx.x == 0 && threadIdx.x == 0) clk->n_events = all;
+    for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < all;
          k += (unsigned long long)gridDim.x * blockDim.x) {
-        const long long e = ev[k];
-        const SegCtx& X = ctx[(int)(e >> 32)];
-        if (X.sp == 2) {
+        if (k >= n) {
             chi[k] = 1.0;
             r[k] = 0.5;
             sb[k] = 0.0;
             lep[k] = 0;
             continue;
         }
+        const long long e = ev[k];
+        const SegCtx& X = ctx[(int)(e >> 32)];
         const int64_t j = (int64_t)(uint32_t)e;
         const PartDev& L = inst[X.ii].sp[X.sp];
         const float4 a = __ldcg(L.q0 + j), b = __ldcg(L.q1 + j), cc = __ldcg(L.q2 + j);
@@ -571,7 +601,10 @@ __global__ void batch_compact_move(const InstDev* __restrict__ inst, ClockDev* c
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *G.count = I.hdr[0] - I.hdr[1];
         *G.n_dead = 0;
-        if (blockIdx.y == 0) clk->step += 1;  // the step is complete: advance the device clock
+        if (blockIdx.y == 0) {
+            clk->step += 1;  // the step is complete: advance the device clock
+            clk->n_events = clk->n_list[0] + clk->n_list[1];
+        }
     }
 }
 
@@ -604,8 +637,8 @@ struct qed_batch_s {
     InstDev* d_inst;
     SegDev* d_seg;
     SegCtx* d_ctx;     // per-segment step contexts (plan kernel -> event kernel)
-    long long* d_ev;   // the step's event list: segment << 32 | particle index, one slot per particle
-    int ev_grid;       // event kernel grid
+    long long* d_ev;   // the step's event list: segment << 32 | particle index, one slot per particle of capacity
+    int ev_grid, ev64_grid;  // event kernels' grids
     int64_t* d_tile0;
     ClockDev* d_clk;
     int64_t* d_hdr;
@@ -641,7 +674,7 @@ static void launch_variant(const qed_batch_s* b, int grid, cudaStream_t st) {
     P.chi_floor = b->desc.chi_floor;
     batch_step_kernel<WARPS, STAGES, MINB, FIX><<<grid, WARPS * 32, smem, st>>>(
         tab_params<float>(t), t->bes32, b->d_inst, b->d_seg, b->d_tile0, b->n_inst, b->d_clk, P, b->tuning.chunk,
-        &b->d_clk->next_tile, b->d_ev, &b->d_clk->n_events, b->ctr);
+        &b->d_clk->next_tile, b->d_ev, b->capacity_total, b->d_clk->n_list, b->ctr);
 }
 
 #define QED_VARIANTS(FIX)                                                                \
@@ -694,9 +727,11 @@ static void launch_batch_step(const qed_batch_s* b, cudaStream_t st, cudaEvent_t
         mlp_sample_listed(b->mlp, b->tables, b->d_mchi, b->d_mr, b->d_ms, b->capacity_total, &b->d_clk->n_events,
                           b->mlp_tol, b->d_mout, b->d_mfb, b->mlp_grid, st);
     }
-    batch_event_kernel<<<b->ev_grid, kEventThreads, 0, st>>>(b->d_inst, b->d_ctx, b->d_ev, b->d_clk,
-                                                             Tab64{tab_params<double>(b->tables), b->tables->bes64},
-                                                             b->ctr, b->mlp ? b->d_mout : nullptr);
+    const Tab64 X64{tab_params<double>(b->tables), b->tables->bes64};
+    batch_event_kernel<<<b->ev_grid, kEventThreads, 0, st>>>(b->d_inst, b->d_ctx, b->d_ev, b->capacity_total, b->d_clk,
+                                                             X64, b->ctr, b->mlp ? b->d_mout : nullptr);
+    batch_event64_kernel<<<b->ev64_grid, kEvent64Threads, 0, st>>>(b->d_inst, b->d_ctx, b->d_ev, b->capacity_total,
+                                                                   b->d_clk, X64, b->ctr, b->mlp != nullptr);
     if (e1) cudaEventRecordWithFlags(e1, st, rec);
     batch_compact_head<<<(b->n_inst + 255) / 256, 256, 0, st>>>(b->d_inst, b->n_inst);
     const dim3 g(kCompactBlocks, b->n_inst);
@@ -870,6 +905,9 @@ extern "C" qed_status qed_batch_create(qed_tables_t t, const qed_instance* insta
     int ev_per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ev_per_sm, batch_event_kernel, kEventThreads, 0);
     b->ev_grid = b->sms * std::max(1, ev_per_sm);
+    ev_per_sm = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ev_per_sm, batch_event64_kernel, kEvent64Threads, 0);
+    b->ev64_grid = b->sms * std::max(1, ev_per_sm);
     const qed_batch_tuning def{0, 0, 64, 8};
     if (qed_batch_set_tuning(b, &def) != QED_OK) {
         qed_batch_destroy(b);

@@ -680,17 +680,15 @@ static __device__ __noinline__ void lepton_event64(const Ctx& C, const Tab64& X,
     P_out = narrow(stokes_to_P(xi, eps, beta, khat));
 }
 
-// Events to be taken again in FP64, queued per warp so that the FP64 code runs with all 32 lanes busy
-// (one ill-conditioned lane would otherwise make its whole warp run it).  An entry names the lepton, the
-// photon's reserved slot (-1: no photon stored), the caller's context key with the branch in bit 30 and
-// the learned sampler's ln u' (when the caller uses it).
-constexpr int kExactQ = 64;  // entries per warp; drained 32 at a time
-struct ExactQ {
-    int64_t j[kExactQ];
-    int64_t slot[kExactQ];
-    int key[kExactQ];
-    float lnu[kExactQ];
-    int n;
+// Events to be taken again in FP64, listed so that the FP64 code runs with every lane of a few warps busy (one
+// ill-conditioned lane would otherwise make its whole warp run it; even a queue per warp leaves every warp of the
+// grid one nearly empty pass of ~2000 FP64 instructions, 16 cycles of the SM's FP64 pipe each).  An entry is three
+// words: the caller's event word (its context key above the particle index) with the branch in bit 62, the
+// photon's reserved slot (-1: no photon stored), and the learned sampler's ln u' (when the caller uses it).
+struct ExactList {
+    long long* item;        // [cap][3]
+    unsigned long long* n;  // entries asked for (those beyond cap were taken by their own lane)
+    unsigned long long cap;
 };
 
 // One queued event in FP64 (per lane, not warp-collective): the lepton's stored state is still the one
@@ -718,14 +716,14 @@ static __device__ __noinline__ void lepton_exact_one(const Ctx& C, const Tab64& 
 
 // the event pass of one warp (all 32 lanes call it): a lane with j >= 0 takes particle j of buffer L,
 // whose step context is C and whose photons go to G through the reservation A (lanes may differ in all
-// three; A is NULL when the caller keeps no photons).  q (may be NULL): the warp's queue for the events
-// taken again in FP64, with the lane's context key; without it they are taken here.  net: the energy
+// three; A is NULL when the caller keeps no photons).  q (may be NULL): the list for the events taken again
+// in FP64, with the lane's event word; without it they are taken here.  net: the energy
 // fraction is u' = exp(lnu), drawn by the learned sampler from the same uniform (Sec. 5.1), instead of
 // the branch's ICDF row.
 static __device__ QED_EVENT_PASS void lepton_events(const Ctx& C, const Tab64& X, const FieldP<double>& F64, int64_t j,
                                                  const PartDev& L, const PartDev& G, AppendState* A,
-                                                 qed_counters* ctr, unsigned long long* c, ExactQ* q = nullptr,
-                                                 int key = 0, bool net = false, float lnu = 0.0f) {
+                                                 qed_counters* ctr, unsigned long long* c, const ExactList* q = nullptr,
+                                                 long long word = 0, bool net = false, float lnu = 0.0f) {
     // The lepton's outcome (energy fraction, recoil, spin) and the photon's polarization for every event,
     // then the photon's slot reservation: an event whose photon does not fit is not applied.
     const uint32_t fl = C.S.flags;
@@ -865,16 +863,22 @@ static __device__ QED_EVENT_PASS void lepton_events(const Ctx& C, const Tab64& X
     }
     if (q != nullptr) {  // warp-uniform
         const unsigned m = __ballot_sync(0xffffffffu, queued);
-        if (queued) {
-            const int e = q->n + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
-            q->j[e] = j;
-            q->slot[e] = keep ? A->base[0] + ev : -1;
-            q->key[e] = key | (down ? (1 << 30) : 0);
-            q->lnu[e] = lnu;
+        if (m) {
+            const int lane = threadIdx.x & 31;
+            unsigned long long e = 0;
+            if (lane == 0) e = atomicAdd(q->n, (unsigned long long)__popc(m));
+            e = __shfl_sync(0xffffffffu, e, 0) + __popc(m & ((1u << lane) - 1u));
+            if (queued) {
+                const int64_t slot = keep ? A->base[0] + ev : -1;
+                if (e < q->cap) {
+                    q->item[3 * e] = word | (down ? 1ll << 62 : 0ll);
+                    q->item[3 * e + 1] = slot;
+                    q->item[3 * e + 2] = (long long)__float_as_uint(lnu);
+                } else {
+                    lepton_exact_one(C, X, F64, L, G, j, slot, down, net, lnu);
+                }
+            }
         }
-        __syncwarp();
-        if ((threadIdx.x & 31) == 0) q->n += __popc(m);
-        __syncwarp();
     }
 }
 
