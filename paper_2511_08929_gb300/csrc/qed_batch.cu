@@ -727,7 +727,7 @@ static void launch_batch_step(const qed_batch_s* b, cudaStream_t st, cudaEvent_t
         mlp_sample_listed(b->mlp, b->tables, b->d_mchi, b->d_mr, b->d_ms, b->capacity_total, &b->d_clk->n_events,
                           b->mlp_tol, b->d_mout, b->d_mfb, b->mlp_grid, st);
     }
-    const Tab64 X64{tab_params<double>(b->tables), b->tables->bes64};
+    const Tab64 X64{tab_params<double>(b->tables), b->tables->besp};
     batch_event_kernel<<<b->ev_grid, kEventThreads, 0, st>>>(b->d_inst, b->d_ctx, b->d_ev, b->capacity_total, b->d_clk,
                                                              X64, b->ctr, b->mlp ? b->d_mout : nullptr);
     batch_event64_kernel<<<b->ev64_grid, kEvent64Threads, 0, st>>>(b->d_inst, b->d_ctx, b->d_ev, b->capacity_total,

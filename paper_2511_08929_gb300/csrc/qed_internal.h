@@ -21,6 +21,7 @@ struct qed_tables_s {
     float* icdf32;
     float* icdf32lo;  // icdf64 - icdf32 rounded to float: the two floats hold an ICDF entry to ~1e-14
     double* bes64;  // [3][kBesN] scaled Bessel values
+    double* besp;   // [kBpN][3][kBpDeg + 1] the same functions as polynomials (the steps' FP64 events)
     float* bes32;
     double* amm64;  // [n_chi] ln a(chi_i), the field-dependent anomalous moment
     float* amm32;

@@ -157,7 +157,7 @@ void launch_lepton32(const qed_tables_s* t, const qed_field& f, const qed_step_d
     const void* k = (const void*)step32_kernel<false>;
     step32_kernel<false><<<blocks32(L->capacity, k, smem), kT32, smem, st>>>(
         tab_params<float>(t), t->bes32, field_params<float>(f), step_params(s, f), (float)L->charge, part_dev(L), g,
-        PartDev{}, G ? append_state(ctr) : nullptr, Tab64{tab_params<double>(t), t->bes64}, field_params<double>(f), ctr);
+        PartDev{}, G ? append_state(ctr) : nullptr, Tab64{tab_params<double>(t), t->besp}, field_params<double>(f), ctr);
 }
 
 void launch_photon32(const qed_tables_s* t, const qed_field& f, const qed_step_desc& s, const qed_particles* G,
@@ -172,5 +172,5 @@ void launch_photon32(const qed_tables_s* t, const qed_field& f, const qed_step_d
     const void* k = (const void*)step32_kernel<true>;
     step32_kernel<true><<<blocks32(G->capacity, k, smem), kT32, smem, st>>>(
         tab_params<float>(t), t->bes32, field_params<float>(f), step_params(s, f), 0.0f, part_dev(G), e, p,
-        (El && Po) ? append_state(ctr) : nullptr, Tab64{tab_params<double>(t), t->bes64}, field_params<double>(f), ctr);
+        (El && Po) ? append_state(ctr) : nullptr, Tab64{tab_params<double>(t), t->besp}, field_params<double>(f), ctr);
 }

@@ -9,6 +9,7 @@
 // which never changes k or w, writes two planes (one when the photon has no pair rate).
 #pragma once
 #include "qed_bessel.cuh"
+#include "qed_fp64.cuh"
 #include "qed_internal.h"
 #include "qed_steps.h"
 
@@ -523,8 +524,8 @@ __device__ __forceinline__ void store_photon32_step(const PartDev& G, int64_t j,
 // coefficients 1/(1 - lambda) - xi3/lambda and the like cancel), and the photon's Stokes vector and the
 // lepton's spin axis of the events whose FP32 forms cancel (|F| or |g| small against their terms).
 struct Tab64 {
-    TabP<double> T;     // FP64 rate and ICDF tables
-    const double* bes;  // FP64 scaled Bessel table [3][kBesN]
+    TabP<double> T;      // FP64 rate and ICDF tables
+    const double* besp;  // FP64 Bessel polynomials (bessel_poly)
 };
 
 __device__ __forceinline__ V3<double> wide(const F3& v) { return V3<double>{v.x, v.y, v.z}; }
@@ -604,80 +605,36 @@ static __device__ __noinline__ void lepton_event64(const Ctx& C, const Tab64& X,
                                                   bool net, float lnu, const uint4& w0, const uint4& w1,
                                                   const uint4& w2, F3& x_out,
                                                   F3& p_out, F3& s_out, F3& k_out, F3& P_out) {
-    using V = V3<double>;
     const uint32_t fl = C.S.flags;
-    const double dt = C.S.dt, q = (double)C.q;
-    V x{a.x, a.y, a.z}, p{a.w, b.x, b.y}, s{b.z, b.w, cc.x};
-    V E, B;
-    field_eval(F64, C.S.ph_hi, 0.0, x, E, B);
-    const V pold = p;
-    if (fl & QED_F_PUSH) p = boris(p, E, B, q, dt);
-    if (fl & QED_F_TBMT) {
-        const V pb = 0.5 * (pold + p);
-        s = rotate(s, tbmt_omega(pb, E, B, q, (fl & QED_F_TBMT_PAPER) != 0, tbmt_a(fl, X.T, F64.eta0, pb, E, B)), dt);
-    }
-    const double gam = sqrt(1.0 + dot(p, p));
-    if (fl & QED_F_MOVE) x = x + v3(p.x / gam * dt, p.y / gam * dt, p.z / gam * dt);
-    const double chi = chi_of(F64.eta0, gam, p, E, B);
-    const double pn = sqrt(dot(p, p));
-    const V khat = v3(p.x / pn, p.y / pn, p.z / pn);
-    V eps{0, 0, 0}, beta{0, 0, 0};
-    make_basis(E, B, v3(p.x / gam, p.y / gam, p.z / gam), khat, -q, eps, beta);
+    const V64 x{a.x, a.y, a.z}, p{a.w, b.x, b.y}, s{b.z, b.w, cc.x};
+    Lep64 st;
+    if (plane_wave(F64.kind)) lepton_classical64<true>(fl, X.T, F64, C.S.ph_hi, C.S.dt, 0.0, (double)C.q, x, p, s, st);
+    else lepton_classical64<false>(fl, X.T, F64, C.S.ph_hi, C.S.dt, 0.0, (double)C.q, x, p, s, st);
     const double r2 = uniform52(w1.x, w1.y), r3 = uniform52(w1.z, w1.w), r4 = uniform52(w2.x, w2.y);
-    double lam, one_m, up;
-    if (fl & QED_F_REJECT) {  // the accepted candidate lambda = r1^3
+    double lam, one_m, iom, u, up;  // iom = 1/(1 - lambda), u = lambda/(1 - lambda)
+    if (fl & QED_F_REJECT) {        // the accepted candidate lambda = r1^3
         const double r1 = uniform52(w0.x, w0.y);
         lam = r1 * r1 * r1;
         one_m = 1.0 - lam;
-        up = 2.0 * lam / (3.0 * chi * one_m);
-    } else if (net) {  // ln u' as the learned sampler drew it from the same uniform r2
-        up = exp((double)lnu);
-        lam = 3.0 * chi * up / (2.0 + 3.0 * chi * up);
-        one_m = 1.0 - lam;
-    } else {
-        up = exp(icdf_lookup(X.T, false, down ? 1 : 0, log(chi), log(r2) - log(1.0 - r2)));
-        lam = 3.0 * chi * up / (2.0 + 3.0 * chi * up);
-        one_m = 1.0 - lam;
+        iom = 1.0 / one_m;
+        u = lam * iom;
+        up = u / (1.5 * st.chi);
+    } else {  // ln u' as the learned sampler drew it from the same uniform r2, or the branch's ICDF row
+        up = exp(net ? (double)lnu : icdf_lookup64(X.T, false, down ? 1 : 0, log(st.chi), log(r2 / (1.0 - r2))));
+        u = 1.5 * st.chi * up;
+        iom = 1.0 + u;
+        one_m = 1.0 / iom;
+        lam = u * one_m;
     }
-    const V k = lam * p;
-    V pf = p, sf = s, sfu{0, 0, 0}, si{0, 0, 0};
-    if (fl & QED_F_RECOIL) pf = one_m * p;
-    if (fl & QED_F_RESOLVED) si = s;
-    double bb[3];
-    bessel64(X.bes, up, bb);
-    double xi[3] = {0.0, 0.0, 0.0};
-    double wv = 0.0;
-    V g{0, 0, 0};
-    if (fl & (QED_F_SPIN_EVENT | QED_F_POL_EVENT)) nlc_wg(lam, one_m, bb, si, beta, khat, wv, g);
-    if (fl & QED_F_SPIN_EVENT) {
-        const double gn = sqrt(dot(g, g));
-        if (fl & QED_F_BETA_BASIS) {  // resolved along +-beta (Sec. 8.3 comparison)
-            const double gb = dot(g, beta);
-            sf = (fl & QED_F_SPIN_COLLAPSE) ? (r3 < (wv - gb) / (2.0 * wv) ? -1.0 : 1.0) * beta : (gb / wv) * beta;
-        } else if (fl & QED_F_SPIN_COLLAPSE) {
-            const double sg = r3 < (wv - gn) / (2.0 * wv) ? -1.0 : 1.0;
-            sf = gn > 0.0 ? v3(sg * g.x / gn, sg * g.y / gn, sg * g.z / gn) : v3(0.0, 0.0, 0.0);
-        } else {
-            sf = v3(g.x / wv, g.y / wv, g.z / wv);
-        }
-        sfu = sf;
-    }
-    if (fl & QED_F_POL_EVENT) {
-        double Fv[4];
-        nlc_stokes(lam, one_m, bb, si, sfu, wv, g, eps, beta, khat, Fv);
-        const double Fn = sqrt(Fv[1] * Fv[1] + Fv[2] * Fv[2] + Fv[3] * Fv[3]);
-        if (fl & QED_F_POL_COLLAPSE) {
-            const double sg = r4 < (Fv[0] - Fn) / (2.0 * Fv[0]) ? -1.0 : 1.0;
-            for (int i = 0; i < 3; ++i) xi[i] = Fn > 0.0 ? sg * Fv[i + 1] / Fn : 0.0;
-        } else {
-            for (int i = 0; i < 3; ++i) xi[i] = Fv[i + 1] / Fv[0];
-        }
-    }
-    x_out = narrow(x);
-    p_out = narrow(pf);
+    const V64 si = (fl & QED_F_RESOLVED) ? st.s : V64{0.0, 0.0, 0.0};
+    V64 sf;
+    double xi[3];
+    nlc_event64(fl, X.besp, up, lam, u, iom + one_m, iom - one_m, st, si, r3, r4, sf, xi);
+    x_out = narrow(st.x);
+    p_out = narrow((fl & QED_F_RECOIL) ? one_m * st.p : st.p);
     s_out = narrow(sf);
-    k_out = narrow(k);
-    P_out = narrow(stokes_to_P(xi, eps, beta, khat));
+    k_out = narrow(lam * st.p);
+    P_out = narrow(stokes_to_P64(xi, st.eps, st.beta, st.khat));
 }
 
 // Events to be taken again in FP64, listed so that the FP64 code runs with every lane of a few warps busy (one
@@ -1028,59 +985,35 @@ static __device__ QED_EVENT_PASS void photon_events(const Ctx& C, const Tab64& X
         const bool low = m < half;  // u < 1/2: the positron takes the smaller fraction
         const uint64_t dm = low ? half - 1ull - m : m - half;
         const double rf = ((double)dm + 0.5) * 0x1.0p-51, rfc = ((double)((half - 1ull) - dm) + 0.5) * 0x1.0p-51;
-        const double chi = (double)st.chi;
-        double ut, lam, one_m;
-        if (rej) {  // the accepted candidate positron fraction lambda = r1 (Sec. 4.2)
+        const double chi = (double)st.chi, ichi = 1.0 / chi;
+        double ut, lam, one_m, Q;  // Q = 1/(lambda (1 - lambda)) = 3 chi u~'/2
+        if (rej) {                 // the accepted candidate positron fraction lambda = r1 (Sec. 4.2)
             lam = uniform52(w0.x, w0.y);
             one_m = 1.0 - lam;
-            ut = 2.0 / (3.0 * chi * lam * one_m);
+            Q = 1.0 / (lam * one_m);
+            ut = (2.0 / 3.0) * ichi * Q;
         } else {
-            const double xv = exp(icdf_lookup(X.T, true, minus ? 1 : 0, log(chi), log(rf) - log(rfc)));
-            const double umin = (8.0 / 3.0) / chi;
+            const double xv = exp(icdf_lookup64(X.T, true, minus ? 1 : 0, log(chi), log(rf / rfc)));
+            const double umin = (8.0 / 3.0) * ichi;
             ut = umin + xv;
             // mu (1 - mu) = q = 2/(3 chi u~'), so 1 - 4q = x/u~' exactly and mu = (1 - sqrt(x/u~'))/2
             // = u~'_min / (2 u~' (1 + sqrt(x/u~'))), free of cancellation near the centre
-            const double mu = 0.5 * (umin / ut) / (1.0 + sqrt(xv / ut));
+            const double iut = 1.0 / ut;
+            const double mu = 0.5 * umin * iut / (1.0 + sqrt(xv * iut));
             lam = low ? mu : 1.0 - mu;
             one_m = low ? 1.0 - mu : mu;
+            Q = 1.5 * chi * ut;
         }
-        const V3<double> k64 = wide(st.k);
+        const V64 k64 = wide(st.k);
         pp = narrow(lam * k64);
         pe = narrow(one_m * k64);
         if (fl & QED_F_SPIN_EVENT) {
-            double bb[3];
-            bessel64(X.bes, ut, bb);
             const double xi[3] = {st.xi[0], st.xi[1], st.xi[2]};
-            const V3<double> eps = wide(st.eps), beta = wide(st.beta), kh = wide(st.khat);
-            double w0v;
-            V3<double> je, jp;
-            nbw_j(lam, one_m, bb, xi, eps, beta, kh, w0v, je, jp);
-            if (fl & QED_F_SPIN_COLLAPSE) {
-                const double jen = sqrt(dot(je, je)), jpn = sqrt(dot(jp, jp));
-                V3<double> Se = jen > 0.0 ? (1.0 / jen) * je : V3<double>{0, 0, 0};
-                V3<double> Sp = jpn > 0.0 ? (1.0 / jpn) * jp : V3<double>{0, 0, 0};
-                if (fl & QED_F_BETA_BASIS) Se = Sp = beta;  // the G_ab sum to 4 w0 on any axes
-                // four correlated states, order (--, -+, +-, ++), first sign = positron
-                double cum = 0.0;
-                int chosen = 3;
-                for (int s4 = 0; s4 < 3; ++s4) {
-                    const double sa = (s4 & 2) ? 1.0 : -1.0, sbb = (s4 & 1) ? 1.0 : -1.0;
-                    cum += nbw_G(lam, one_m, bb, xi, sa * Sp, sbb * Se, eps, beta, kh) / (4.0 * w0v);
-                    if (r3 < cum) {
-                        chosen = s4;
-                        break;
-                    }
-                }
-                const double sa = (chosen & 2) ? 1.0 : -1.0, sbb = (chosen & 1) ? 1.0 : -1.0;
-                sp = narrow(sa * Sp);
-                se = narrow(sbb * Se);
-            } else if (fl & QED_F_BETA_BASIS) {
-                se = narrow((dot(je, beta) / w0v) * beta);
-                sp = narrow((dot(jp, beta) / w0v) * beta);
-            } else {
-                se = narrow((1.0 / w0v) * je);
-                sp = narrow((1.0 / w0v) * jp);
-            }
+            V64 e64, p64;
+            nbw_event64(fl, X.besp, ut, lam, one_m, one_m * Q, lam * Q, xi, r3, wide(st.eps), wide(st.beta),
+                        wide(st.khat), e64, p64);
+            se = narrow(e64);
+            sp = narrow(p64);
         }
         const uint4 wc = draw(id, C.S.seed, C.S.step, kSlotChild);
         ide = (uint64_t)wc.x | ((uint64_t)wc.y << 32);

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "qed_bessel.cuh"
+#include "qed_fp64.cuh"
 #include "qed_internal.h"
 
 namespace qed {
@@ -60,6 +61,51 @@ __global__ void bessel_table_kernel(double* tab64, float* tab32) {
     for (int f = 0; f < 3; ++f) {
         tab64[f * kBesN + j] = o[f];
         tab32[f * kBesN + j] = (float)o[f];
+    }
+}
+
+// The Bessel polynomials of the step kernels (bessel_poly): one warp per interval evaluates the functions at the
+// interval's 9 Chebyshev nodes, the lanes sharing the terms of the trapezoid sums (below 1e-4 the ascending series),
+// and turns the values into coefficients with the nodes' inverse Vandermonde matrix.
+__constant__ double c_vander[kBpDeg + 1][kBpDeg + 1];  // [power][node]
+__constant__ double c_cheb[kBpDeg + 1];
+
+__global__ void __launch_bounds__(128) bessel_poly_kernel(double* tab) {
+    __shared__ double val[4][3][kBpDeg + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * 4 + warp;
+    if (i >= kBpN) return;
+    const double centre = ldexp(1.0 + (i % kBpSub + 0.5) / kBpSub, kBpLoExp + i / kBpSub);
+    const double half = ldexp(0.5 / kBpSub, kBpLoExp + i / kBpSub);
+    for (int n = 0; n <= kBpDeg; ++n) {
+        const double x = fma(half, c_cheb[n], centre);
+        double o[3] = {0.0, 0.0, 0.0};
+        if (x < kBesLo) {
+            bessel_series<double>(x, o);
+        } else {
+            double T = acosh(1.0 + 46.0 / x);
+            T = acosh(1.0 + (46.0 + (2.0 / 3.0) * T) / x);
+            const double h = fmin(0.2, 0.6 * rsqrt(x));
+            const int steps = (int)ceil(T / h);
+            for (int m = 1 + lane; m <= steps; m += 32) {
+                const double t = m * h, sh = sinh(0.5 * t), e = exp(-x * (2.0 * sh * sh)), c3 = cosh(t / 3.0);
+                o[0] += e * c3;
+                o[1] += e * (2.0 * c3 * c3 - 1.0);
+                o[2] += e * c3 / cosh(t);
+            }
+            for (int f = 0; f < 3; ++f) {
+                for (int s = 16; s > 0; s >>= 1) o[f] += __shfl_xor_sync(0xffffffffu, o[f], s);
+                o[f] = (0.5 + o[f]) * h;
+            }
+        }
+        if (lane < 3) val[warp][lane][n] = lane == 0 ? o[0] : (lane == 1 ? o[1] : o[2]);
+    }
+    __syncwarp();
+    if (lane < kBpRow) {
+        const int f = lane / (kBpDeg + 1), k = lane % (kBpDeg + 1);
+        double v = 0.0;
+        for (int n = 0; n <= kBpDeg; ++n) v += c_vander[k][n] * val[warp][f][n];
+        tab[(size_t)i * kBpRow + lane] = v;
     }
 }
 
@@ -152,10 +198,10 @@ __global__ void __launch_bounds__(kNlcThreads) nlc_rows_kernel(const double* __r
 
 // NBW rows.  The densities in t at both signs sigma = +1, -1 (they share the Bessel functions and all but one
 // product)
-__device__ __forceinline__ void nbw_density(const double* __restrict__ bes, double chi, double t, double& dp, double& dm) {
+__device__ __forceinline__ void nbw_density(const double* __restrict__ besp, double chi, double t, double& dp, double& dm) {
     double b[3];
     const double ut = 8.0 / (3.0 * chi) + t * t;
-    bessel64(bes, ut, b);
+    bessel_poly(besp, ut, b);
     const double rho = 1.5 * chi * ut - 2.0;
     const double f = exp(-t * t) * 4.0 / (3.0 * chi * ut * sqrt(ut));
     const double w = b[2] + rho * b[1];
@@ -192,7 +238,7 @@ __device__ __forceinline__ void panel_cdf(const double* c, double d, double s, d
 // where the series has not converged; a Newton step on the series is ~100 fused multiply-adds.  A quadrature and a
 // density per step, with a stopping rule of one rounding unit that sent most entries through a bisection, took
 // 27 ms for 256 x 256 entries a sign; this kernel takes 0.69 ms (83 % of the FP64 pipe's cycles).
-__global__ void __launch_bounds__(256) nbw_rows_kernel(const double* __restrict__ bes, qed_table_desc d, double* rates,
+__global__ void __launch_bounds__(256) nbw_rows_kernel(const double* __restrict__ besp, qed_table_desc d, double* rates,
                                                        double* icdf) {
     __shared__ double coef[2][kNbwPanels][kGL];  // density at the nodes, then its Legendre coefficients
     __shared__ double cum[2][kNbwPanels + 1];
@@ -205,7 +251,7 @@ __global__ void __launch_bounds__(256) nbw_rows_kernel(const double* __restrict_
     for (int e = threadIdx.x; e < np * kGL; e += blockDim.x) {
         const int p = e / kGL, k = e % kGL;
         const double a = p * kPanel, b = fmin(tend, (p + 1) * kPanel);
-        nbw_density(bes, chi, 0.5 * (a + b) + 0.5 * (b - a) * c_gl_x[k], coef[0][p][k], coef[1][p][k]);
+        nbw_density(besp, chi, 0.5 * (a + b) + 0.5 * (b - a) * c_gl_x[k], coef[0][p][k], coef[1][p][k]);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < 2 * np; e += blockDim.x) {
@@ -273,10 +319,10 @@ __global__ void __launch_bounds__(256) nbw_rows_kernel(const double* __restrict_
             for (int it = 0; it < 4; ++it) {
                 double dens[2], sum = 0.0;
                 for (int k = 0; k < kGL; ++k) {
-                    nbw_density(bes, chi, 0.5 * (a + t) + 0.5 * (t - a) * c_gl_x[k], dens[0], dens[1]);
+                    nbw_density(besp, chi, 0.5 * (a + t) + 0.5 * (t - a) * c_gl_x[k], dens[0], dens[1]);
                     sum += c_gl_w[k] * (s ? dens[1] : dens[0]);
                 }
-                nbw_density(bes, chi, t, dens[0], dens[1]);
+                nbw_density(besp, chi, t, dens[0], dens[1]);
                 const double tn = t - (sum * 0.5 * (t - a) - T) / (s ? dens[1] : dens[0]);
                 if (!(tn >= a && tn <= a + w)) break;
                 const bool found = fabs(tn - t) <= 1e-9 * t;
@@ -420,11 +466,12 @@ extern "C" qed_status qed_tables_build(const qed_table_desc* desc, qed_tables_t*
         bytes += (n + 255) & ~size_t(255);
         return at;
     };
-    const size_t at[10] = {place(nr * sizeof(double)),        place(ni * sizeof(double)),
+    const size_t at[11] = {place(nr * sizeof(double)),        place(ni * sizeof(double)),
                            place(nr * sizeof(float)),         place(ni * sizeof(float)),
                            place(ni * sizeof(float)),         place(3 * kBesN * sizeof(double)),
                            place(3 * kBesN * sizeof(float)),  place(d.n_chi * sizeof(double)),
-                           place(d.n_chi * sizeof(float)),    place((size_t)G.panels * kGL * sizeof(double))};
+                           place(d.n_chi * sizeof(float)),    place((size_t)G.panels * kGL * sizeof(double)),
+                           place((size_t)kBpN * kBpRow * sizeof(double))};
     unsigned char* mem = nullptr;
     if (cudaMalloc(&mem, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -441,6 +488,7 @@ extern "C" qed_status qed_tables_build(const qed_table_desc* desc, qed_tables_t*
     t->amm64 = (double*)(mem + at[7]);
     t->amm32 = (float*)(mem + at[8]);
     double* gv = (double*)(mem + at[9]);
+    t->besp = (double*)(mem + at[10]);
     double glx[kGL], glw[kGL], leg[kGL][kGL];
     gauss_legendre(kGL, glx, glw);
     for (int i = 0; i < kGL; ++i) {
@@ -452,7 +500,23 @@ extern "C" qed_status qed_tables_build(const qed_table_desc* desc, qed_tables_t*
             p1 = p2;
         }
     }
-    if (cudaMemcpyToSymbolAsync(c_gl_x, glx, sizeof(glx), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+    // Chebyshev nodes, and their inverse Vandermonde matrix through the Chebyshev coefficients
+    double cheb[kBpDeg + 1], vander[kBpDeg + 1][kBpDeg + 1] = {};
+    {
+        constexpr int n = kBpDeg + 1;
+        double poly[n][n] = {};  // T_j's coefficients
+        poly[0][0] = poly[1][1] = 1.0;
+        for (int j = 2; j < n; ++j)
+            for (int k = 0; k < n; ++k) poly[j][k] = (k > 0 ? 2.0 * poly[j - 1][k - 1] : 0.0) - poly[j - 2][k];
+        for (int i = 0; i < n; ++i) cheb[i] = std::cos(kPi * (i + 0.5) / n);
+        for (int i = 0; i < n; ++i)
+            for (int j = 0; j < n; ++j)
+                for (int k = 0; k < n; ++k)
+                    vander[k][i] += (j == 0 ? 1.0 : 2.0) / n * std::cos(kPi * j * (i + 0.5) / n) * poly[j][k];
+    }
+    if (cudaMemcpyToSymbolAsync(c_cheb, cheb, sizeof(cheb), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(c_vander, vander, sizeof(vander), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(c_gl_x, glx, sizeof(glx), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(c_gl_w, glw, sizeof(glw), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(c_legendre, leg, sizeof(leg), 0, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         free_tables(t);
@@ -460,7 +524,8 @@ extern "C" qed_status qed_tables_build(const qed_table_desc* desc, qed_tables_t*
     }
     bessel_table_kernel<<<(kBesN + 127) / 128, 128, 0, st>>>(t->bes64, t->bes32);
     nlc_rows_kernel<<<2 * d.n_chi, kNlcThreads, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
-    nbw_rows_kernel<<<d.n_chi, 256, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
+    bessel_poly_kernel<<<(kBpN + 3) / 4, 128, 0, st>>>(t->besp);
+    nbw_rows_kernel<<<d.n_chi, 256, 0, st>>>(t->besp, d, t->rate64, t->icdf64);
     to_float_kernel<<<64, 256, 0, st>>>(t->rate64, t->rate32, nr);
     split_float_kernel<<<256, 256, 0, st>>>(t->icdf64, t->icdf32, t->icdf32lo, ni);
     amm_nodes_kernel<<<(G.panels * kGL + 3) / 4, 128, 0, st>>>(G, gv);
