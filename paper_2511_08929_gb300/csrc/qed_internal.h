@@ -144,7 +144,7 @@ inline bool valid_field(const qed_field* f) {
            (f->kind == QED_FIELD_CONST || f->n_cycles > 0.0);
 }
 
-inline int launch_blocks(int64_t work, int threads) {
+inline int launch_blocks(int64_t work, int threads, int per_sm = 8) {
     static int sms = 0;
     if (sms == 0) {
         int dev = 0;
@@ -153,7 +153,7 @@ inline int launch_blocks(int64_t work, int threads) {
         if (sms <= 0) sms = 1;
     }
     const int64_t need = (work + threads - 1) / threads;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * 8));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * per_sm));
 }
 
 // The learned sampler inside the batched step (defined with the network in qed_mlp.cu): the network's
