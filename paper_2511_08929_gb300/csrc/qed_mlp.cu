@@ -18,6 +18,7 @@
 #include <cuda_bf16.h>
 
 #include "qed_device.cuh"
+#include "qed_fp64.cuh"
 #include "qed_internal.h"
 
 namespace qed {
@@ -206,6 +207,167 @@ __device__ inline float xi3_at32(const float* __restrict__ bes32, float chi, flo
     return (b[1] + u * s * b[0]) / (-b[2] + kappa * b[1] + lam * s * b[0]);
 }
 
+// ---- the sampler's own solves ------------------------------------------------------------------------
+// The sampler's check and fallback take their roots on the float tables first and, where FP64 decides, finish them on
+// the FP64 tables by Newton's method: a step is two ICDF rows with their slopes, ~45 FP64 instructions a branch, and
+// two steps from the float root leave errors below 1e-13.  (The bracketing solvers above, which the training targets
+// use, take ~80 ICDF evaluations for a mixture quantile in FP64, 0.65 ms for one warp; this one takes ~0.03 ms.)
+
+// value and slope (in the logit) of branch b's ICDF at the logit y, rows (i, i + 1) blended with f; inside the grid,
+// and below it, where the row continues with slope 3
+template <class R>
+__device__ __forceinline__ void icdf_slope(const TabP<R>& T, int b, int i, R f, R y, R& q, R& dq) {
+    const R y0 = T.y_lo * T.inv_dy, tt = fma_(y, T.inv_dy, -y0);
+    if (!(tt > R(0))) {
+        const R* row = T.nlc_icdf + ((size_t)b * T.n_chi + i) * T.n_r;
+        q = fma_(R(3), y - T.y_lo, fma_(f, row[T.n_r] - row[0], row[0]));
+        dq = R(3);
+        return;
+    }
+    const int m = min(max((int)tt, 1), T.n_r - 3);
+    const R x = fma_(y, T.inv_dy, -y0 - R(m)), xm = x - R(1);
+    const R* row = T.nlc_icdf + ((size_t)b * T.n_chi + i) * T.n_r + m;
+    R v[2], d[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k, row += T.n_r) {
+        const R p0 = row[-1], p1 = row[0], p2 = row[1], p3 = row[2];
+        const R d1 = p2 - p1, d2 = R(0.5) * ((p0 - p1) + d1), d3 = fma_(R(-3), d1, p3 - p0) * R(1.0 / 6.0);
+        const R e = fma_(x + R(1), d3, d2), c = fma_(xm, e, d1);
+        v[k] = fma_(x, c, p1);
+        d[k] = fma_(x, fma_(xm, d3, e), c);
+    }
+    q = fma_(f, v[1] - v[0], v[0]);
+    dq = fma_(f, d[1] - d[0], d[0]) * T.inv_dy;
+}
+
+// Newton's method for the mixture quantile in (L, y_u, y_d): both branch ICDFs at their logits equal L and the blend
+// of the logits' CDFs equals r.  True when a step below `dy` was taken with every logit
+// below the grid's upper end.
+template <class R>
+__device__ inline bool mix_newton(const TabP<R>& T, int i, R f, R a, R r, int iters, R dy, R& L, R& yu, R& yd) {
+    const R yhi = T.y_lo + R(T.n_r - 1) / T.inv_dy;
+#pragma unroll 1
+    for (int it = 0; it < iters; ++it) {
+        if (!(yu < yhi && yd < yhi)) return false;
+        R qu, du, qd, dd;
+        icdf_slope(T, 0, i, f, yu, qu, du);
+        icdf_slope(T, 1, i, f, yd, qd, dd);
+        if (!(du > R(0) && dd > R(0))) return false;
+        const R iu = rcp_(du), id = rcp_(dd);
+        const R su = rcp_(R(1) + exp_(-yu)), sd = rcp_(R(1) + exp_(-yd));
+        const R wu = a * su * (R(1) - su) * iu, wd = (R(1) - a) * sd * (R(1) - sd) * id;
+        const R res = (r - a * su - (R(1) - a) * sd) - fma_(wu, L - qu, wd * (L - qd));
+        if (!(wu + wd > R(0))) return false;
+        L = L + div_(res, wu + wd);
+        const R eu = (L - qu) * iu, ed = (L - qd) * id;
+        yu += eu;
+        yd += ed;
+        if (fabs(eu) < dy && fabs(ed) < dy) return yu < yhi && yd < yhi;
+    }
+    return false;
+}
+
+// the logit at which branch b's ICDF row equals L, from a root y good to the float tables; false if it leaves the
+// grid upwards
+__device__ inline bool logit_newton64(const TabP<double>& T, int b, int i, double f, double L, double& y) {
+    const double yhi = T.y_lo + (T.n_r - 1) / T.inv_dy;
+#pragma unroll 1
+    for (int it = 0; it < 4; ++it) {
+        if (!(y < yhi)) return false;
+        double q, dq;
+        icdf_slope(T, b, i, f, y, q, dq);
+        if (!(dq > 0.0)) return false;
+        const double e = (L - q) / dq;
+        y += e;
+        if (fabs(e) < 1e-7) return y < yhi;
+    }
+    return false;
+}
+
+// branch_cdf on the float tables, returning the logit (infinite above the row's last entry)
+__device__ __noinline__ float branch_logit32(const TabP<float>& T, int b, float lnchi, float L, float yg, float qg) {
+    const float yhi = T.y_lo + (float)(T.n_r - 1) / T.inv_dy;
+    auto g = [&](float yy) { return icdf_lookup(T, false, b, lnchi, yy) - L; };
+    const float g0 = qg - L;
+    if (g0 == 0.0f) return yg;
+    const bool up = g0 < 0.0f;  // the root lies above yg
+    float x = yg, gx = g0;
+    float step = (L - qg) / 3.0f;
+    step = step < 0.0f ? -step : step;
+    if (step < 1e-5f) step = 1e-5f;
+    float a = x, ga = gx, c = x, gc = gx;
+    bool found = false;
+#pragma unroll 1
+    for (int k = 0; k < 26 && !found; ++k) {
+        float xn = up ? x + step : x - step;
+        const bool edge = up ? xn >= yhi : xn <= T.y_lo;
+        if (edge) xn = up ? yhi : T.y_lo;
+        const float gn = g(xn);
+        if (up ? gn >= 0.0f : gn <= 0.0f) {
+            a = up ? x : xn;
+            ga = up ? gx : gn;
+            c = up ? xn : x;
+            gc = up ? gn : gx;
+            found = true;
+        } else if (edge) {
+            if (up) return __int_as_float(0x7F800000);  // L above the row's last entry
+            return T.y_lo + (-gn) / 3.0f;               // below: y_lo + (L - bottom)/3
+        } else {
+            x = xn;
+            gx = gn;
+            step *= 2.0f;
+        }
+    }
+    if (!found) return x;  // not reached: 26 doublings span the grid
+    const float aL = L < 0.0f ? -L : L;
+    return illinois<30>(g, a, ga, c, gc, a - ga * (c - a) / (gc - ga), 1e-6f, 1e-7f * (aL > 1.0f ? aL : 1.0f));
+}
+
+// the mixture's CDF at L on the float tables, with the branches' logits
+__device__ inline float mix_cdf32(const TabP<float>& T, const MixPointT<float>& m, float L, float& yu, float& yd) {
+    yu = branch_logit32(T, 0, m.lnchi, L, m.y, m.qu);
+    yd = branch_logit32(T, 1, m.lnchi, L, m.y, m.qd);
+    return m.a * (1.0f / (1.0f + exp_(-yu))) + (1.0f - m.a) * (1.0f / (1.0f + exp_(-yd)));
+}
+
+// |C(L) - r| on the FP64 tables, from the float tables' logits (the bracketing solver where a logit lies above the
+// grid)
+__device__ __noinline__ double mix_error64(const TabP<double>& T, const MixPoint& m, double L, double r, float yu32,
+                                           float yd32) {
+    int i;
+    double f, yu = yu32, yd = yd32;
+    chi_coord(T, m.lnchi, i, f);
+    if (logit_newton64(T, 0, i, f, L, yu) && logit_newton64(T, 1, i, f, L, yd))
+        return fabs(m.a / (1.0 + exp(-yu)) + (1.0 - m.a) / (1.0 + exp(-yd)) - r);
+    return fabs(mix_cdf<30>(T, m, L) - r);
+}
+
+// the mixture quantile: Newton on the float tables from the blend of the branch quantiles, then on the FP64 tables;
+// the bracketing solver where that does not converge below the grid's upper end
+__device__ __noinline__ double mix_quantile_fast(const TabP<double>& T, const TabP<float>& T32, const MixPoint& m, double r) {
+    int i;
+    double f;
+    chi_coord(T, m.lnchi, i, f);
+    double L = mix_baseline(T, m), yu = m.y, yd = m.y;
+    float L32 = (float)L, yu32 = (float)m.y, yd32 = (float)m.y;
+    if (mix_newton<float>(T32, i, (float)f, (float)m.a, (float)r, 12, 1e-3f, L32, yu32, yd32)) {
+        L = L32;
+        yu = yu32;
+        yd = yd32;
+    }
+    if (mix_newton<double>(T, i, f, m.a, r, 8, 1e-7, L, yu, yd)) return L;
+    return mix_quantile<44, 32>(T, m, r);
+}
+
+// xi3 = F3 / F0 at u' = e^L from the Bessel polynomials (see xi3_at)
+__device__ inline double xi3_poly(const double* __restrict__ besp, double chi, double L, double s) {
+    if (!(L > -200.0 && L < 50.0)) return nan("");
+    const double up = exp(L), u = 1.5 * chi * up, iom = 1.0 + u, one_m = 1.0 / iom;
+    double b[3];
+    bessel_poly(besp, up, b);
+    return fma(u * s, b[0], b[1]) / (fma(iom + one_m, b[1], -b[2]) + u * one_m * s * b[0]);
+}
+
 __device__ inline void mlp_features(double chi, double r, double s, float x[3]) {
     const double y = fmin(kYClamp, fmax(-kYClamp, log(r) - log1p(-r)));
     x[0] = (float)((log(chi) - 0.5 * (kLnChiLo + kLnChiHi)) / (0.5 * (kLnChiHi - kLnChiLo)));
@@ -342,6 +504,11 @@ __global__ void mlp_adamw_kernel(float* P, float* Mm, float* Vv, const float* __
     P[k] -= lr * upd;
 }
 
+// Blocks per SM of the tensor-core kernels: 4 by registers (128 a thread; 39 KB of shared memory and 64 of the SM's 512
+// TMEM columns each leave room for more).  The occupancy query answers 1 for a kernel that allocates TMEM; a grid of
+// one block per SM took 4.0 ms for 1e6 checked samples, one of four 2.8.
+constexpr int kTcPerSm = 4;
+
 // ---- fused inference on the 5th-generation tensor cores ---------------------------------------------
 // A block of 128 threads takes 128 samples at a time, one per thread and one per TMEM lane.  Layer 1
 // (K = 3) runs in FP32 on the CUDA cores; each thread writes its 64 SiLU outputs as BF16 into the A
@@ -363,8 +530,6 @@ struct TcShared {
     alignas(1024) unsigned char w4[kTN4 * kH * 2];  // W4 padded to 16 rows
     float w1[kOffW2];                               // W1, b1 (FP32)
     float b2[kH], b3[kH], b4[4];
-    int64_t queue[2 * kTR];  // sampler: indices of samples waiting for the table path
-    int queued;
     uint64_t bar;            // MMA completion
     uint32_t tmem;           // TMEM base address of the accumulator
 };
@@ -653,16 +818,16 @@ __global__ void __launch_bounds__(kTR) mlp_forward_kernel(const float* __restric
 constexpr int kLnUpOnly = 4;
 
 // the table path for sample i (the exact mixture quantile, and xi3 there unless ln_up_only)
-__device__ void table_path(const TabP<double>& T, const double* __restrict__ bes_tab, const double* __restrict__ chi_in,
-                           const double* __restrict__ r_in, const double* __restrict__ s_in, int64_t i,
-                           float* __restrict__ out4, bool ln_up_only) {
+__device__ __noinline__ void table_path(const TabP<double>& T, const TabP<float>& T32, const double* __restrict__ besp,
+                                        const double* __restrict__ chi_in, const double* __restrict__ r_in,
+                                        const double* __restrict__ s_in, int64_t i, float* __restrict__ out4, bool ln_up_only) {
     const double chi = chi_in[i], r = r_in[i], s = s_in[i];
     const MixPoint m = mix_point(T, chi, r, s);
-    const double L = mix_quantile<44, 32>(T, m, r);
+    const double L = mix_quantile_fast(T, T32, m, r);
     out4[4 * i] = (float)L;
     out4[4 * i + 1] = 0.0f;
     out4[4 * i + 2] = 0.0f;
-    out4[4 * i + 3] = ln_up_only ? 0.0f : (float)xi3_at(bes_tab, chi, L, s);
+    out4[4 * i + 3] = ln_up_only ? 0.0f : (float)xi3_poly(besp, chi, L, s);
 }
 
 // The check of a network sample, first on the float tables: the FP32 CDF and xi3 errors are within ~1e-6
@@ -671,99 +836,156 @@ __device__ void table_path(const TabP<double>& T, const double* __restrict__ bes
 // the FP64 tables (the FP64 pipe of this GPU runs at 1/64 of the FP32 rate).
 constexpr float kMargin32 = 1e-5f;
 
-// the sampler: network, CDF check; samples that fail it (or all, flags bit 0) wait in a block-wide queue
-// and take the table path 128 at a time, one per thread, so that the block never waits on a few slow
-// threads (the tiles of the network keep the block in step)
-__global__ void __launch_bounds__(kTR) mlp_sample_kernel(const float* __restrict__ P, TabP<double> T,
-                                                         TabP<float> T32, const float* __restrict__ bes32,
-                                                         const double* __restrict__ bes_tab,
-                                                         const double* __restrict__ chi_in, const double* __restrict__ r_in,
-                                                         const double* __restrict__ s_in, int64_t n, double tol,
-                                                         int flags, float* __restrict__ out4, uint8_t* __restrict__ fell,
-                                                         float* __restrict__ err_out, unsigned long long* n_fallback,
-                                                         const unsigned long long* __restrict__ n_dev = nullptr) {
+// The sampler is two kernels.  The first runs the network and leaves its raw outputs in out4; the second checks
+// them.  In one kernel the check's warps, which differ in their solves, met at the eight barriers of every 128-sample
+// tile of the network, and the two codes together missed the instruction cache (barrier and no-instruction stalls
+// were 23 of 33 cycles between issues).  1e6 checked samples of a trained network, 1.1 % of them from the tables: 4.0 ms
+// in one kernel with one block per SM, 2.8 ms with four, 0.69 ms in two kernels with the solves above.
+constexpr uint32_t kNoNet = 0x7FC0BAD0u;  // o[0] of a tile the tensor cores did not answer for (a NaN of its own)
+
+__global__ void __launch_bounds__(kTR, kTcPerSm) mlp_net_kernel(const float* __restrict__ P,
+                                                                const double* __restrict__ chi_in,
+                                                                const double* __restrict__ r_in,
+                                                                const double* __restrict__ s_in, int64_t n,
+                                                                float* __restrict__ out4,
+                                                                const unsigned long long* __restrict__ n_dev) {
     __shared__ TcShared S;
     if (n_dev) {  // a count the previous kernel of the stream left on the device
         const int64_t nd = (int64_t)*n_dev;
         if (nd < n) n = nd;
     }
-    if (threadIdx.x == 0) S.queued = 0;
     tc_setup(S, P);
-    unsigned long long nf = 0;  // thread 0: fallbacks of this block
     uint32_t phase = 0;
-    bool broken = false;  // a wait gave up: the remaining tiles take the table path (the same in every thread)
-    const bool table_only = (flags & 1) != 0;
-    const bool ln_up_only = (flags & kLnUpOnly) != 0;
+    bool broken = false;  // a wait gave up: the remaining tiles skip the network (the same in every thread)
     for (int64_t base = (int64_t)blockIdx.x * kTR; base < n; base += (int64_t)gridDim.x * kTR) {
         const int64_t i = base + threadIdx.x;
         float x[3] = {0.0f, 0.0f, 0.0f}, o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         if (i < n) mlp_features(chi_in[i], r_in[i], s_in[i], x);
-        bool net = false;  // the network ran for this tile
-        if (!table_only && !broken) {
-            net = tc_infer(S, x, phase, o);
-            broken = !net;
+        if (!broken) broken = !tc_infer(S, x, phase, o);
+        if (broken) o[0] = __uint_as_float(kNoNet);
+        if (i < n)
+            for (int j = 0; j < 4; ++j) out4[4 * i + j] = o[j];  // (the caller's array need not be aligned to 16 bytes)
+    }
+    tc_teardown(S.tmem);
+}
+
+// The check: samples that pass on the float tables are done; the others wait in a block-wide queue, and a full block
+// of them at a time goes through FP64 (the check again for those within kMargin32 of the bound, the table path for
+// those that fail it, and for all of them with flags bit 0).  One block of 1024 threads per SM: the queue's last,
+// partly filled pass then runs in a few warps of every SM.
+constexpr int kCheckThreads = 1024;
+
+struct CheckItem {
+    int64_t i;
+    float L, o3, yu, yd;  // the sample and its logits, where the FP64 check decides (yu NaN: the table path)
+};
+
+__global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double> T, TabP<float> T32,
+                                                                     const float* __restrict__ bes32,
+                                                                     const double* __restrict__ besp,
+                                                                     const double* __restrict__ chi_in,
+                                                                     const double* __restrict__ r_in,
+                                                                     const double* __restrict__ s_in, int64_t n, double tol,
+                                                                     int flags, float* __restrict__ out4,
+                                                                     uint8_t* __restrict__ fell, float* __restrict__ err_out,
+                                                                     unsigned long long* n_fallback,
+                                                                     const unsigned long long* __restrict__ n_dev) {
+    extern __shared__ __align__(16) unsigned char check_smem[];
+    CheckItem* queue = reinterpret_cast<CheckItem*>(check_smem);  // [2 kCheckThreads]
+    __shared__ int queued;
+    if (n_dev) {
+        const int64_t nd = (int64_t)*n_dev;
+        if (nd < n) n = nd;
+    }
+    if (threadIdx.x == 0) queued = 0;
+    __syncthreads();
+    const bool table_only = (flags & 1) != 0, ln_up_only = (flags & kLnUpOnly) != 0;
+    const float ftol = (float)tol;
+    unsigned nf = 0;  // this thread's fallbacks
+    // a queued sample: the FP64 check decides, then the table path
+    auto finish = [&](const CheckItem& q) {
+        bool fb = true;
+        if (!isnan(q.yu)) {
+            const double chi = chi_in[q.i], r = r_in[q.i], s = s_in[q.i];
+            const MixPoint m = mix_point(T, chi, r, s);
+            const double e64 = mix_error64(T, m, (double)q.L, r, q.yu, q.yd);
+            double d64 = 0.0;
+            if (!ln_up_only)
+                d64 = fabs(xi3_poly(besp, chi, mix_baseline(T, m), s) + (double)q.o3 / kOutScale -
+                           xi3_poly(besp, chi, (double)q.L, s));
+            if (err_out) err_out[q.i] = (float)e64;
+            fb = !(e64 <= tol) || !(d64 <= tol);
         }
+        if (fell) fell[q.i] = fb ? 1 : 0;
+        if (fb) {
+            table_path(T, T32, besp, chi_in, r_in, s_in, q.i, out4, ln_up_only);
+            ++nf;
+        }
+    };
+    for (int64_t base = (int64_t)blockIdx.x * kCheckThreads; base < n; base += (int64_t)gridDim.x * kCheckThreads) {
+        const int64_t i = base + threadIdx.x;
         if (i < n) {
-            bool fb = !net;
-            if (!fb) {
-                const double chi = chi_in[i], r = r_in[i], s = s_in[i];
-                // the sample on the float tables: baseline, correction, CDF error (and xi3's)
-                const MixPointT<float> m32 = mix_point32(T32, chi, r, s);
-                const float Lb = mix_baseline(T32, m32);
-                const float L = Lb + o[0] / (float)kOutScale;
-                float xi1 = 0.0f, xi2 = 0.0f, xi3 = 0.0f, dxi3 = 0.0f;
-                if (!ln_up_only) {
-                    xi1 = o[1] / (float)kOutScale;
-                    xi2 = o[2] / (float)kOutScale;
-                    xi3 = xi3_at32(bes32, (float)chi, Lb, (float)s) + o[3] / (float)kOutScale;
-                    dxi3 = fabsf(xi3 - xi3_at32(bes32, (float)chi, L, (float)s));
+            CheckItem q{i, 0.0f, 0.0f, __int_as_float(0x7FC00000), 0.0f};
+            bool done = false;
+            if (table_only) {
+                if (err_out) err_out[i] = -1.0f;
+            } else {
+                const float4 o = make_float4(out4[4 * i], out4[4 * i + 1], out4[4 * i + 2], out4[4 * i + 3]);
+                if (__float_as_uint(o.x) == kNoNet) {
+                    if (err_out) err_out[i] = -1.0f;
+                } else {
+                    const double chi = chi_in[i], r = r_in[i], s = s_in[i];
+                    // the sample on the float tables: baseline, correction, CDF error (and xi3's)
+                    const MixPointT<float> m32 = mix_point32(T32, chi, r, s);
+                    const float Lb = mix_baseline(T32, m32);
+                    const float L = Lb + o.x / (float)kOutScale;
+                    float xi1 = 0.0f, xi2 = 0.0f, xi3 = 0.0f, dxi3 = 0.0f;
+                    if (!ln_up_only) {
+                        xi1 = o.y / (float)kOutScale;
+                        xi2 = o.z / (float)kOutScale;
+                        xi3 = xi3_at32(bes32, (float)chi, Lb, (float)s) + o.w / (float)kOutScale;
+                        dxi3 = fabsf(xi3 - xi3_at32(bes32, (float)chi, L, (float)s));
+                    }
+                    float yu, yd;
+                    const float err_q = fabsf(mix_cdf32(T32, m32, L, yu, yd) - (float)r);  // the CDF check
+                    const bool stokes_ok = fabsf(xi1) <= ftol && fabsf(xi2) <= ftol;
+                    const bool pass32 = err_q <= ftol - kMargin32 && dxi3 <= ftol - kMargin32 && stokes_ok;
+                    const bool fail32 = !(err_q <= ftol + kMargin32) || !(dxi3 <= ftol + kMargin32) || !stokes_ok;
+                    if (err_out) err_out[i] = err_q;
+                    done = pass32;
+                    if (!fail32) {  // (one that fails leaves its row to the table path)
+                        out4[4 * i] = L;
+                        out4[4 * i + 1] = xi1;
+                        out4[4 * i + 2] = xi2;
+                        out4[4 * i + 3] = xi3;
+                        if (!pass32) {  // the band around tol: the FP64 check decides
+                            q.L = L;
+                            q.o3 = o.w;
+                            q.yu = yu;
+                            q.yd = yd;
+                        }
+                    }
                 }
-                const float ftol = (float)tol;
-                float err_q = fabsf(mix_cdf<30>(T32, m32, L) - (float)r);  // the CDF check
-                const bool stokes_ok = fabsf(xi1) <= ftol && fabsf(xi2) <= ftol;
-                const bool pass32 = err_q <= ftol - kMargin32 && dxi3 <= ftol - kMargin32 && stokes_ok;
-                const bool fail32 = !(err_q <= ftol + kMargin32) || !(dxi3 <= ftol + kMargin32) || !stokes_ok;
-                fb = !pass32;
-                if (!pass32 && !fail32) {  // the band around tol: the FP64 check decides
-                    const MixPoint m = mix_point(T, chi, r, s);
-                    const double e64 = fabs(mix_cdf<30>(T, m, (double)L) - r);
-                    double d64 = 0.0;
-                    if (!ln_up_only)
-                        d64 = fabs(xi3_at(bes_tab, chi, mix_baseline(T, m), s) + (double)o[3] / kOutScale -
-                                   xi3_at(bes_tab, chi, (double)L, s));
-                    err_q = (float)e64;
-                    fb = !(e64 <= tol) || !(d64 <= tol);
-                }
-                if (err_out) err_out[i] = err_q;
-                if (!fb) {
-                    out4[4 * i] = L;
-                    out4[4 * i + 1] = xi1;
-                    out4[4 * i + 2] = xi2;
-                    out4[4 * i + 3] = xi3;
-                }
-            } else if (err_out) {
-                err_out[i] = -1.0f;
             }
-            if (fell) fell[i] = fb ? 1 : 0;
-            if (fb) S.queue[atomicAdd(&S.queued, 1)] = i;  // at most 2 kTR - 1 entries
+            if (done) {
+                if (fell) fell[i] = 0;
+            } else {
+                queue[atomicAdd(&queued, 1)] = q;  // at most 2 kCheckThreads - 1 entries
+            }
         }
         __syncthreads();
-        const int qn = S.queued;  // the same in every thread
-        if (qn >= kTR) {
-            table_path(T, bes_tab, chi_in, r_in, s_in, S.queue[qn - kTR + threadIdx.x], out4, ln_up_only);
+        const int qn = queued;  // the same in every thread
+        if (qn >= kCheckThreads) {
+            finish(queue[qn - kCheckThreads + threadIdx.x]);
             __syncthreads();
-            if (threadIdx.x == 0) {
-                S.queued = qn - kTR;
-                nf += kTR;
-            }
+            if (threadIdx.x == 0) queued = qn - kCheckThreads;
             __syncthreads();
         }
     }
     __syncthreads();
-    const int qn = S.queued;
-    if ((int)threadIdx.x < qn) table_path(T, bes_tab, chi_in, r_in, s_in, S.queue[threadIdx.x], out4, ln_up_only);
-    if (threadIdx.x == 0 && n_fallback && nf + (unsigned long long)qn) atomicAdd(n_fallback, nf + (unsigned long long)qn);
-    tc_teardown(S.tmem);
+    if ((int)threadIdx.x < queued) finish(queue[threadIdx.x]);
+    nf = __reduce_add_sync(0xffffffffu, nf);
+    if ((threadIdx.x & 31) == 0 && n_fallback && nf) atomicAdd(n_fallback, (unsigned long long)nf);
 }
 
 // The method the network would replace, as the step's event pass runs it (Sec. 5.1): the spin branch
@@ -970,23 +1192,36 @@ extern "C" qed_status qed_mlp_train(qed_mlp_t m, qed_tables_t t, int64_t steps, 
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
 }
 
-// persistent grid for the tensor-core kernels: one resident wave of 128-thread blocks, at most 4 per SM
-// (each holds 64 TMEM columns of the SM's 512, and its 38 KB of shared memory)
-static int tc_blocks(int64_t n, const void* kern) {
-    int dev = 0, sms = 1, per_sm = 1;
+// persistent grid for the tensor-core kernels: one resident wave of 128-thread blocks
+static int tc_blocks(int64_t n) {
+    int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTR, 0);
-    const int64_t resident = (int64_t)sms * std::max(1, std::min(per_sm, 4));
-    return (int)std::max<int64_t>(1, std::min<int64_t>((n + kTR - 1) / kTR, resident));
+    return (int)std::max<int64_t>(1, std::min<int64_t>((n + kTR - 1) / kTR, (int64_t)sms * kTcPerSm));
 }
 
 extern "C" qed_status qed_mlp_forward(qed_mlp_t m, const float* x_dev, int64_t n, float* out_dev, void* stream) {
     if (!valid_mlp(m)) return QED_ERR_STATE;
     if (n < 0 || (n > 0 && (!x_dev || !out_dev))) return QED_ERR_ARG;
     if (n == 0) return QED_OK;
-    mlp_forward_kernel<<<tc_blocks(n, (const void*)mlp_forward_kernel), kTR, 0, (cudaStream_t)stream>>>(m->P, x_dev, n,
+    mlp_forward_kernel<<<tc_blocks(n), kTR, 0, (cudaStream_t)stream>>>(m->P, x_dev, n,
                                                                                                    out_dev);
+    return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
+}
+
+// network (unless flags bit 0) and check of the first min(n, *n_dev) samples; grid: the network kernel's
+static qed_status mlp_sample_launch(qed_mlp_t m, const qed_tables_s* t, const double* chi, const double* r, const double* s,
+                                    int64_t n, const unsigned long long* n_dev, double tol, int flags, float* out4,
+                                    uint8_t* fell_back, float* err_out, unsigned long long* n_fallback, int grid,
+                                    cudaStream_t st) {
+    const size_t smem = 2 * kCheckThreads * sizeof(CheckItem);
+    if (cudaFuncSetAttribute(mlp_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return QED_ERR_CUDA;
+    if (!(flags & QED_MLP_ALWAYS_TABLE))
+        mlp_net_kernel<<<grid, kTR, 0, st>>>(m->P, chi, r, s, n, out4, n_dev);
+    const int blocks = (int)std::min<int64_t>((n + kCheckThreads - 1) / kCheckThreads, (grid + kTcPerSm - 1) / kTcPerSm);
+    mlp_check_kernel<<<blocks, kCheckThreads, smem, st>>>(tab_params<double>(t), tab_params<float>(t), t->bes32, t->besp, chi,
+                                                          r, s, n, tol, flags, out4, fell_back, err_out, n_fallback, n_dev);
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
 }
 
@@ -1006,26 +1241,18 @@ extern "C" qed_status qed_mlp_sample(qed_mlp_t m, qed_tables_t t, const double* 
                                                                           t->bes32, chi, r, s, n, out4);
         return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
     }
-    // persistent grid (one resident wave): each warp streams many 32-sample rows, so its fallback queue
-    // drains full
-    const int blocks = tc_blocks(n, (const void*)mlp_sample_kernel);
-    mlp_sample_kernel<<<blocks, kTR, 0, (cudaStream_t)stream>>>(m->P, tab_params<double>(t), tab_params<float>(t),
-                                                                t->bes32, t->bes64, chi, r, s, n, tol, flags, out4,
-                                                                fell_back, err_out, n_fallback);
-    return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
+    return mlp_sample_launch(m, t, chi, r, s, n, nullptr, tol, flags, out4, fell_back, err_out, n_fallback, tc_blocks(n),
+                             (cudaStream_t)stream);
 }
 
 // ---- the sampler inside the batched step (qed_batch.cu) ------------------------------------------------
 
 bool mlp_valid(qed_mlp_t m) { return valid_mlp(m); }
 
-int mlp_listed_grid(int64_t n_max) { return tc_blocks(n_max, (const void*)mlp_sample_kernel); }
+int mlp_listed_grid(int64_t n_max) { return tc_blocks(n_max); }
 
 qed_status mlp_sample_listed(qed_mlp_t m, const qed_tables_s* t, const double* chi, const double* r, const double* s,
                              int64_t n_max, const unsigned long long* n_dev, double tol, float* out4,
                              unsigned long long* n_fallback, int grid, cudaStream_t st) {
-    mlp_sample_kernel<<<grid, kTR, 0, st>>>(m->P, tab_params<double>(t), tab_params<float>(t), t->bes32, t->bes64,
-                                            chi, r, s, n_max, tol, kLnUpOnly, out4, nullptr, nullptr, n_fallback,
-                                            n_dev);
-    return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
+    return mlp_sample_launch(m, t, chi, r, s, n_max, n_dev, tol, kLnUpOnly, out4, nullptr, nullptr, n_fallback, grid, st);
 }
