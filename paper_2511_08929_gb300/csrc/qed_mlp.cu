@@ -8,11 +8,10 @@
 // predicts the correction to the rate-weighted blend of the two branch quantiles (and of xi3 there),
 // scaled by 100.
 //
-// Kernels: target generation (FP64), a BF16 GEMM on the tensor cores (tcgen05.mma, FP32 accumulator in
-// TMEM; split-K for the weight gradients), FP32 elementwise / first-layer / reduction / AdamW kernels for
-// training, and a fused inference kernel (layers 2-4 as tcgen05.mma on 128-sample tiles, bias and SiLU
-// between them applied on the way from TMEM back to shared memory), followed by the CDF check and the
-// table fallback.
+// Kernels: target generation (FP64); one training kernel (forward, backward and weight gradients of 128-sample
+// tiles on the tensor cores: tcgen05.mma with BF16 operands and FP32 accumulators in TMEM) and AdamW; inference
+// (layers 2-4 as tcgen05.mma on 128-sample tiles, bias and SiLU between them applied on the way from TMEM back to
+// shared memory), and the CDF check with the table fallback.
 #include <cstring>
 
 #include <cuda_bf16.h>
@@ -407,90 +406,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// ---- training kernels (FP32) ------------------------------------------------------------------------
-// layer 1: Z1 = X W1^T + b1, H1 = silu(Z1)
-__global__ void mlp_layer1_kernel(const float* __restrict__ P, const float* __restrict__ X, int64_t n, float* Z,
-                                  float* H) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * kH; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = e / kH;
-        const int j = (int)(e % kH);
-        const float* w = P + kOffW1 + 3 * j;
-        const float z = fmaf(w[0], X[3 * b], fmaf(w[1], X[3 * b + 1], fmaf(w[2], X[3 * b + 2], P[kOffB1 + j])));
-        Z[e] = z;
-        H[e] = silu_f(z);
-    }
-}
-
-// Z += bias (in place), H = silu(Z)
-__global__ void mlp_bias_silu_kernel(const float* __restrict__ bias, int64_t n, float* Z, float* H) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * kH; e += (int64_t)gridDim.x * blockDim.x) {
-        const float z = Z[e] + bias[e % kH];
-        Z[e] = z;
-        H[e] = silu_f(z);
-    }
-}
-
-// O += b4; dO = 2 (O - T) / n; loss += sum (O - T)^2 / n
-__global__ void mlp_out_loss_kernel(const float* __restrict__ P, const float* __restrict__ Tg, int64_t n, float* O,
-                                    float* dO, float* loss) {
-    float acc = 0.0f;
-    const float inv = 1.0f / (float)n;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * 4; e += (int64_t)gridDim.x * blockDim.x) {
-        const float o = O[e] + P[kOffB4 + (e & 3)];
-        O[e] = o;
-        const float d = o - Tg[e];
-        dO[e] = 2.0f * d * inv;
-        acc = fmaf(d * inv, d, acc);
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, acc);
-}
-
-// dZ = dH * silu'(Z) (in place on dH)
-__global__ void mlp_silu_back_kernel(const float* __restrict__ Z, int64_t n, float* dH) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * kH; e += (int64_t)gridDim.x * blockDim.x)
-        dH[e] *= dsilu_f(Z[e]);
-}
-
-// column sums of D[n][w] into out[w] (one block per column; deterministic order)
-__global__ void mlp_colsum_kernel(const float* __restrict__ D, int64_t n, int w, float* out) {
-    __shared__ float red[32];
-    const int col = blockIdx.x;
-    float acc = 0.0f;
-    for (int64_t b = threadIdx.x; b < n; b += blockDim.x) acc += D[b * w + col];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        acc = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (threadIdx.x == 0) out[col] = acc;
-    }
-}
-
-// dW1[j][i] = sum_b dZ1[b][j] X[b][i] (one block per entry, FP32)
-__global__ void mlp_dw1_kernel(const float* __restrict__ dZ, const float* __restrict__ X, int64_t n, float* g) {
-    __shared__ float red[32];
-    const int j = blockIdx.x / 3, i = blockIdx.x % 3;
-    float acc = 0.0f;
-    for (int64_t b = threadIdx.x; b < n; b += blockDim.x) acc = fmaf(dZ[b * kH + j], X[3 * b + i], acc);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        acc = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (threadIdx.x == 0) g[kOffW1 + 3 * j + i] = acc;
-    }
-}
-
+// ---- AdamW ----------------------------------------------------------------------------------------
 __device__ __forceinline__ bool is_weight(int k) {
     return k < kOffB1 || (k >= kOffW2 && k < kOffB2) || (k >= kOffW3 && k < kOffB3) || (k >= kOffW4 && k < kOffB4);
 }
 
-// AdamW (decoupled weight decay on weights only); t = step count after this update
-__global__ void mlp_adamw_kernel(float* P, float* Mm, float* Vv, const float* __restrict__ G, float lr, float wd,
-                                 float b1t, float b2t) {
+// AdamW (decoupled weight decay on weights only); t = step count after this update.  zero (may be NULL): the gradient
+// array to clear for the next step's sums (the same as G in the training loop)
+__global__ void mlp_adamw_kernel(float* P, float* Mm, float* Vv, const float* G, float lr, float wd, float b1t, float b2t,
+                                 float* zero) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= kParams) return;
     const float g = G[k];
@@ -502,6 +426,7 @@ __global__ void mlp_adamw_kernel(float* P, float* Mm, float* Vv, const float* __
     float upd = mh / (sqrtf(vh) + 1e-8f);
     if (is_weight(k)) upd += wd * P[k];
     P[k] -= lr * upd;
+    if (zero) zero[k] = 0.0f;
 }
 
 // Blocks per SM of the tensor-core kernels: 4 by registers (128 a thread; 39 KB of shared memory and 64 of the SM's 512
@@ -688,108 +613,330 @@ __device__ void tc_teardown(uint32_t tmem) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-// ---- BF16 GEMM on the tensor cores for training (FP32 in global memory, rounded to BF16 when staged;
-// FP32 accumulation in TMEM) ----------------------------------------------------------------------------
-// C(m, n) (+)= sum_k A(m, k) B(k, n); A(m, k) = A[m sam + k sak], B(k, n) = B[k sbk + n sbn]; C row-major
-// with leading dimension ldc.  A block of 128 threads computes a 128 x 64 tile of C, staging 64-wide K
-// slices of A and B (any strides) as K-major BF16 operands and accumulating with tcgen05.mma.
-// grid = (ceil(N/64), ceil(M/128), ksplit); with ksplit > 1 the partial sums are added atomically (C
-// zeroed by the caller).  If the tensor cores do not answer within the wait limit the tile is NaN.
-struct GemmShared {
-    alignas(1024) unsigned char a[kTR * kH * 2];  // A slice: 128 rows x 64 K
-    alignas(1024) unsigned char b[kH * kH * 2];   // B slice: 64 columns of C x 64 K
+// ---- training: forward, backward and weight gradients of a tile of 128 samples in one kernel ------------
+// A block keeps 128 samples, one per TMEM lane, through the whole pass: nothing of the network's 64-wide activations goes
+// to global memory.  Layers 2-4 forward and the input gradients of layers 3 and 2 are
+// tcgen05.mma of the sample-major tile (M = samples) with the weights or their transposes; the weight gradients of
+// layers 2 and 3 are tcgen05.mma over K = 128 samples (M = output units in the lower 64 rows, the upper 64 zero;
+// N = input units) that stay in TMEM over the block's tiles.  As in a GEMM of its own, every operand is rounded to
+// BF16 and sums are FP32; biases, layer 1 and the 4-wide layer's gradient are FP32 sums over the warp's lanes.
+// TMEM columns: Z2, Z3, a scratch accumulator, dW3, dW2.
+// Nine GEMM launches that staged their operands from FP32 arrays in global memory (13-80 us each on 32 blocks) and
+// ten elementwise and column-sum launches took 0.34 ms for a batch of 4096; this pass takes 25 us.
+constexpr uint32_t kTrainCols = 512;
+constexpr uint32_t kColZ2 = 0, kColZ3 = 64, kColT = 128, kColW3 = 192, kColW2 = 256;
+
+struct TrainShared {
+    alignas(1024) unsigned char a[kTR * kH * 2];        // A operand: 128 samples x 64
+    alignas(1024) unsigned char w2[kH * kH * 2];        // B operands: W2, W3 (N = output units)
+    alignas(1024) unsigned char w3[kH * kH * 2];
+    alignas(1024) unsigned char w2t[kH * kH * 2];       // their transposes (N = input units)
+    alignas(1024) unsigned char w3t[kH * kH * 2];
+    alignas(1024) unsigned char w4[kTN4 * kH * 2];      // W4 padded to 16 rows
+    alignas(1024) unsigned char h1t[kH * kTR * 2];      // B operands: H1^T, H2^T (64 units x 128 samples)
+    alignas(1024) unsigned char h2t[kH * kTR * 2];
+    alignas(1024) unsigned char dzt[kTR * kTR * 2];     // A operand: dZ^T (64 units x 128 samples, upper 64 rows zero)
+    float w1[kOffW2];                                   // W1, b1 (FP32)
+    float b2[kH], b3[kH], b4[4];
+    float w4r[4][kH];                                   // W4 rounded to BF16
     uint64_t bar;
     uint32_t tmem;
 };
 
-__global__ void __launch_bounds__(kTR) gemm_bf16_kernel(int M, int N, int K, const float* __restrict__ A, int64_t sam,
-                                                         int64_t sak, const float* __restrict__ B, int64_t sbk,
-                                                         int64_t sbn, float* __restrict__ C, int64_t ldc, int ksplit) {
-    __shared__ GemmShared S;
-    const int tid = threadIdx.x;
+// byte offset of (row r, column k) in a K-major tile with K = 128
+__device__ __forceinline__ uint32_t kmaj128(int r, int k) {
+    return (uint32_t)((r >> 3) * 2048 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
+}
+
+__device__ __forceinline__ float bf16_round(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+
+// one thread: D (+)= A B^T over ks steps of K = 16; group strides in bytes
+__device__ __forceinline__ void tc_issue(uint32_t d, uint32_t a, uint32_t asbo, uint32_t b, uint32_t bsbo, int ks, uint32_t id,
+                                         bool acc) {
+    for (int k = 0; k < ks; ++k) {
+        const uint64_t da = (tc_desc(a + 256 * k) & ~((uint64_t)0x3FFF << 32)) | ((uint64_t)(asbo >> 4) << 32);
+        const uint64_t db = (tc_desc(b + 256 * k) & ~((uint64_t)0x3FFF << 32)) | ((uint64_t)(bsbo >> 4) << 32);
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+            "l"(da), "l"(db), "r"(id), "r"((uint32_t)(acc || k > 0))
+            : "memory");
+    }
+}
+
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sm_u32(bar)) : "memory");
+}
+
+// every thread: the shared-memory operands written so far, to the MMA
+__device__ __forceinline__ void tc_publish() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+}
+
+// every thread: wait for the committed MMAs (bounded); false in every thread if the wait gave up
+__device__ __forceinline__ bool tc_await(uint64_t* bar, uint32_t& phase) {
+    bool done = false;
+    for (int i = 0; i < kTcWaitLimit && !done; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(sm_u32(bar)), "r"(phase)
+            : "memory");
+        done = ok != 0;
+    }
+    phase ^= 1u;
+    tc_fence_after();
+    return __syncthreads_and(done) != 0;
+}
+
+// Four threads share a sample, 16 units each (a warp reads the TMEM lanes of its index modulo 4): the elementwise work
+// and the column sums are what a pass costs, and one thread per sample left a single warp on each scheduler (61 us a
+// pass of 32 tiles against 25).
+constexpr int kTrainThreads = 4 * kTR;
+constexpr int kTU = 16;  // units per thread
+
+// this thread's 16 values as BF16: its part of its row of the sample-major A tile, and of its column of a unit-major
+// tile
+__device__ __forceinline__ void train_row(unsigned char* a, int c0, const float v[kTU]) {
+#pragma unroll
+    for (int c = 0; c < kTU / 8; ++c) {
+        uint4 q;
+        q.x = pack_bf16(v[8 * c], v[8 * c + 1]);
+        q.y = pack_bf16(v[8 * c + 2], v[8 * c + 3]);
+        q.z = pack_bf16(v[8 * c + 4], v[8 * c + 5]);
+        q.w = pack_bf16(v[8 * c + 6], v[8 * c + 7]);
+        *reinterpret_cast<uint4*>(a + kmaj(threadIdx.x & (kTR - 1), c0 + 8 * c)) = q;
+    }
+}
+__device__ __forceinline__ void train_column(unsigned char* t, int c0, const float v[kTU]) {
+#pragma unroll
+    for (int j = 0; j < kTU; ++j)
+        *reinterpret_cast<__nv_bfloat16*>(t + kmaj128(c0 + j, threadIdx.x & (kTR - 1))) = __float2bfloat16_rn(v[j]);
+}
+
+// sums of 16 columns over the warp's lanes: lanes 2 c and 2 c + 1 get column c's, added to s (v is used up).  At each
+// step a lane keeps the half of its columns that its lane bit names and gets its partner's sums of that half: 16
+// shuffles for 16 columns.
+template <int W>
+__device__ __forceinline__ void column_fold(float v[kTU]) {
+    const bool upper = threadIdx.x & (2 * W);
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const float send = upper ? v[i] : v[i + W], keep = upper ? v[i + W] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * W);
+    }
+}
+__device__ __forceinline__ void column_sums(float v[kTU], float& s) {
+    column_fold<8>(v);
+    column_fold<4>(v);
+    column_fold<2>(v);
+    column_fold<1>(v);
+    s += v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// grad (zeroed by the caller) += dL/dparameters, loss (may be NULL) += L of the n samples (X, Tg)
+__global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(const float* __restrict__ P, const float* __restrict__ X,
+                                                           const float* __restrict__ Tg, int64_t n, float* __restrict__ grad,
+                                                           float* __restrict__ loss) {
+    extern __shared__ __align__(1024) unsigned char train_smem[];
+    TrainShared& S = *reinterpret_cast<TrainShared*>(train_smem);
+    const int tid = threadIdx.x, lane = tid & 31, c0 = (tid / kTR) * kTU;  // this thread's units c0 .. c0 + 15
+    for (int i = tid; i < kOffW2; i += kTrainThreads) S.w1[i] = P[i];
+    for (int i = tid; i < kH; i += kTrainThreads) {
+        S.b2[i] = P[kOffB2 + i];
+        S.b3[i] = P[kOffB3 + i];
+    }
+    if (tid < 4) S.b4[tid] = P[kOffB4 + tid];
+    for (int i = tid; i < kH * kH; i += kTrainThreads) {
+        const int r = i / kH, k = i % kH;
+        const __nv_bfloat16 a = __float2bfloat16_rn(P[kOffW2 + i]), b = __float2bfloat16_rn(P[kOffW3 + i]);
+        *reinterpret_cast<__nv_bfloat16*>(S.w2 + kmaj(r, k)) = a;
+        *reinterpret_cast<__nv_bfloat16*>(S.w3 + kmaj(r, k)) = b;
+        *reinterpret_cast<__nv_bfloat16*>(S.w2t + kmaj(k, r)) = a;
+        *reinterpret_cast<__nv_bfloat16*>(S.w3t + kmaj(k, r)) = b;
+    }
+    for (int i = tid; i < kTN4 * kH; i += kTrainThreads) {
+        const int r = i / kH, k = i % kH;
+        const float w = r < 4 ? bf16_round(P[kOffW4 + i]) : 0.0f;
+        *reinterpret_cast<__nv_bfloat16*>(S.w4 + kmaj(r, k)) = __float2bfloat16_rn(w);
+        if (r < 4) S.w4r[r][k] = w;
+    }
+    for (int i = tid; i < (int)(sizeof(S.dzt) / 16); i += kTrainThreads) reinterpret_cast<uint4*>(S.dzt)[i] = make_uint4(0, 0, 0, 0);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sm_u32(&S.bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm_u32(&S.tmem)),
-                     "r"(kTmemCols)
+                     "r"(kTrainCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const int m0 = blockIdx.y * kTR, n0 = blockIdx.x * kH;
-    const int kchunk = ((K + ksplit - 1) / ksplit + kH - 1) / kH * kH;
-    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
-    const uint32_t id = tc_idesc(kH);
+    const uint32_t tm = S.tmem, row = tm + ((uint32_t)(tid & (kTR - 1) & ~31) << 16);
+    const uint32_t id64 = tc_idesc(kH), id16 = tc_idesc(kTN4);
+    const float inv = 1.0f / (float)n;
     uint32_t phase = 0;
     bool ok = true;
-    for (int k0 = kb; k0 < ke && ok; k0 += kH) {
-        for (int e = tid; e < kTR * kH; e += kTR) {
-            const int mm = e / kH, kk = e % kH, m = m0 + mm, k = k0 + kk;
-            *reinterpret_cast<__nv_bfloat16*>(S.a + kmaj(mm, kk)) =
-                __float2bfloat16_rn(m < M && k < ke ? A[m * sam + k * sak] : 0.0f);
+    float lsum = 0.0f, sb4[4] = {0, 0, 0, 0}, sb3 = 0.0f, sb2 = 0.0f, sb1 = 0.0f, sw4[4] = {}, sw1[3] = {};
+    bool first = true;
+    for (int64_t base = (int64_t)blockIdx.x * kTR; base < n && ok; base += (int64_t)gridDim.x * kTR, first = false) {
+        const int64_t i = base + (tid & (kTR - 1));
+        const bool have = i < n;
+        float x[3] = {0.0f, 0.0f, 0.0f}, v[kTU];
+        if (have)
+            for (int q = 0; q < 3; ++q) x[q] = X[3 * i + q];
+        // forward
+#pragma unroll
+        for (int k = 0; k < kTU; ++k) {
+            const float* w = S.w1 + 3 * (c0 + k);
+            v[k] = silu_f(fmaf(w[0], x[0], fmaf(w[1], x[1], fmaf(w[2], x[2], S.w1[kOffB1 + c0 + k]))));
         }
-        for (int e = tid; e < kH * kH; e += kTR) {
-            const int nn = e / kH, kk = e % kH, n = n0 + nn, k = k0 + kk;
-            *reinterpret_cast<__nv_bfloat16*>(S.b + kmaj(nn, kk)) =
-                __float2bfloat16_rn(n < N && k < ke ? B[k * sbk + n * sbn] : 0.0f);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
+        train_row(S.a, c0, v);
+        train_column(S.h1t, c0, v);
+        tc_publish();
         if (tid == 0) {
+            tc_issue(tm + kColZ2, sm_u32(S.a), 1024, sm_u32(S.w2), 1024, kH / 16, id64, false);
+            tc_commit(&S.bar);
+        }
+        if (!(ok = tc_await(&S.bar, phase))) break;
+        tc_ld16(row + kColZ2 + c0, v);
 #pragma unroll
-            for (int ks = 0; ks < kH / 16; ++ks) {
-                const uint64_t da = tc_desc(sm_u32(S.a) + 256 * ks), db = tc_desc(sm_u32(S.b) + 256 * ks);
-                const uint32_t acc = (k0 > kb || ks > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(S.tmem),
-                    "l"(da), "l"(db), "r"(id), "r"(acc)
-                    : "memory");
+        for (int k = 0; k < kTU; ++k) v[k] = silu_f(v[k] + S.b2[c0 + k]);
+        train_row(S.a, c0, v);
+        train_column(S.h2t, c0, v);
+        tc_publish();
+        if (tid == 0) {
+            tc_issue(tm + kColZ3, sm_u32(S.a), 1024, sm_u32(S.w3), 1024, kH / 16, id64, false);
+            tc_commit(&S.bar);
+        }
+        if (!(ok = tc_await(&S.bar, phase))) break;
+        tc_ld16(row + kColZ3 + c0, v);
+#pragma unroll
+        for (int k = 0; k < kTU; ++k) v[k] = silu_f(v[k] + S.b3[c0 + k]);
+        train_row(S.a, c0, v);
+        tc_publish();
+        if (tid == 0) {
+            tc_issue(tm + kColT, sm_u32(S.a), 1024, sm_u32(S.w4), 1024, kH / 16, id16, false);
+            tc_commit(&S.bar);
+        }
+        if (!(ok = tc_await(&S.bar, phase))) break;
+        // outputs, loss and their gradient
+        float u[16], d[4];
+        tc_ld16(row + kColT, u);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float e = have ? u[q] + S.b4[q] - Tg[4 * i + q] : 0.0f;
+            lsum = fmaf(e * inv, e, lsum);
+            d[q] = 2.0f * e * inv;
+            sb4[q] += d[q];
+            d[q] = bf16_round(d[q]);
+        }
+        // layer 4: dW4 (v still holds H3), then dZ3 = (dO W4) silu'(Z3)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float t[kTU];
+#pragma unroll
+            for (int k = 0; k < kTU; ++k) t[k] = d[q] * bf16_round(v[k]);
+            column_sums(t, sw4[q]);
+        }
+        tc_ld16(row + kColZ3 + c0, v);
+#pragma unroll
+        for (int k = 0; k < kTU; ++k)
+            v[k] = fmaf(d[3], S.w4r[3][c0 + k], fmaf(d[2], S.w4r[2][c0 + k], fmaf(d[1], S.w4r[1][c0 + k], d[0] * S.w4r[0][c0 + k]))) *
+                   dsilu_f(v[k] + S.b3[c0 + k]);
+        train_row(S.a, c0, v);
+        train_column(S.dzt, c0, v);
+        tc_publish();
+        if (tid == 0) {
+            tc_issue(tm + kColT, sm_u32(S.a), 1024, sm_u32(S.w3t), 1024, kH / 16, id64, false);
+            tc_issue(tm + kColW3, sm_u32(S.dzt), 2048, sm_u32(S.h2t), 2048, kTR / 16, id64, !first);
+            tc_commit(&S.bar);
+        }
+        column_sums(v, sb3);
+        if (!(ok = tc_await(&S.bar, phase))) break;
+        // layer 3 -> dZ2
+        {
+            float z[kTU];
+            tc_ld16(row + kColT + c0, v);
+            tc_ld16(row + kColZ2 + c0, z);
+#pragma unroll
+            for (int k = 0; k < kTU; ++k) v[k] *= dsilu_f(z[k] + S.b2[c0 + k]);
+        }
+        train_row(S.a, c0, v);
+        train_column(S.dzt, c0, v);
+        tc_publish();
+        if (tid == 0) {
+            tc_issue(tm + kColT, sm_u32(S.a), 1024, sm_u32(S.w2t), 1024, kH / 16, id64, false);
+            tc_issue(tm + kColW2, sm_u32(S.dzt), 2048, sm_u32(S.h1t), 2048, kTR / 16, id64, !first);
+            tc_commit(&S.bar);
+        }
+        column_sums(v, sb2);
+        if (!(ok = tc_await(&S.bar, phase))) break;
+        // layer 2 -> dZ1, layer 1 (FP32)
+        tc_ld16(row + kColT + c0, v);
+#pragma unroll
+        for (int k = 0; k < kTU; ++k) {
+            const float* w = S.w1 + 3 * (c0 + k);
+            v[k] *= dsilu_f(fmaf(w[0], x[0], fmaf(w[1], x[1], fmaf(w[2], x[2], S.w1[kOffB1 + c0 + k]))));
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            float t[kTU];
+#pragma unroll
+            for (int k = 0; k < kTU; ++k) t[k] = v[k] * x[q];
+            column_sums(t, sw1[q]);
+        }
+        column_sums(v, sb1);
+    }
+    // the block's sums to the gradient
+    const float bad = __int_as_float(0x7FC00000);
+    if (!first || !ok) {
+        const int u0 = tid & (kTR - 1);
+        if (u0 < kH) {  // (whole warps: the accumulator loads are collective)
+            float a[kTU], b[kTU];
+            tc_ld16(row + kColW3 + c0, a);
+            tc_ld16(row + kColW2 + c0, b);
+#pragma unroll
+            for (int q = 0; q < kTU; ++q) {
+                atomicAdd(&grad[kOffW3 + u0 * kH + c0 + q], ok ? a[q] : bad);
+                atomicAdd(&grad[kOffW2 + u0 * kH + c0 + q], ok ? b[q] : bad);
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             sm_u32(&S.bar))
-                         : "memory");
         }
-        bool done = false;
-        for (int i = 0; i < kTcWaitLimit && !done; ++i) {
-            uint32_t r;
-            asm volatile(
-                "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-                : "=r"(r)
-                : "r"(sm_u32(&S.bar)), "r"(phase)
-                : "memory");
-            done = r != 0;
-        }
-        phase ^= 1u;
-        tc_fence_after();
-        ok = __syncthreads_and(done) != 0;  // also: the slices may be restaged
-    }
-    if (kb < ke) {
-        const int m = m0 + tid;
-        const uint32_t lane_addr = S.tmem + ((uint32_t)(tid & ~31) << 16);
-#pragma unroll 1
-        for (int c0 = 0; c0 < kH; c0 += 16) {
-            float v[16];
-            tc_ld16(lane_addr + (uint32_t)c0, v);
-            if (m < M)
+        if (!(lane & 1)) {
+            const int j = c0 + (lane >> 1);
+            atomicAdd(&grad[kOffB3 + j], ok ? sb3 : bad);
+            atomicAdd(&grad[kOffB2 + j], ok ? sb2 : bad);
+            atomicAdd(&grad[kOffB1 + j], ok ? sb1 : bad);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int n = n0 + c0 + j;
-                    if (n < N) {
-                        const float x = ok ? v[j] : __int_as_float(0x7FC00000);
-                        if (ksplit > 1) atomicAdd(&C[m * ldc + n], x);
-                        else C[m * ldc + n] = x;
-                    }
-                }
+            for (int q = 0; q < 4; ++q) atomicAdd(&grad[kOffW4 + q * kH + j], ok ? sw4[q] : bad);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) atomicAdd(&grad[kOffW1 + 3 * j + q], ok ? sw1[q] : bad);
+        }
+        if (c0 == 0) {  // one of a sample's four threads
+            for (int o = 16; o > 0; o >>= 1) {
+                lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) sb4[q] += __shfl_down_sync(0xffffffffu, sb4[q], o);
+            }
+            if (lane == 0) {
+                if (loss) atomicAdd(loss, ok ? lsum : bad);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) atomicAdd(&grad[kOffB4 + q], ok ? sb4[q] : bad);
+            }
         }
     }
-    tc_teardown(S.tmem);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (tid < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(kTrainCols) : "memory");
 }
 
 // raw network outputs for feature rows X[n][3] (NaN where the tensor cores did not answer)
@@ -1037,8 +1184,9 @@ struct qed_mlp_s {
     uint32_t magic;
     int64_t max_batch;
     float *P, *M, *V, *G;  // parameters, Adam moments, gradients
-    float *X, *T, *Z1, *H1, *Z2, *H2, *Z3, *H3, *O, *dO, *dA, *dB, *loss;
-    int64_t steps;         // AdamW steps taken
+    float *X, *T;          // training samples of several steps (sample_room of them)
+    int64_t sample_room;
+    int64_t steps;  // AdamW steps taken
 };
 
 static bool valid_mlp(const qed_mlp_s* m) { return m && m->magic == kMlpMagic; }
@@ -1047,17 +1195,14 @@ static int grid_for(int64_t work, int threads) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((work + threads - 1) / threads, 152 * 16));
 }
 
-static void gemm(int M, int N, int K, const float* A, int64_t sam, int64_t sak, const float* B, int64_t sbk,
-                 int64_t sbn, float* C, int64_t ldc, int ksplit, cudaStream_t st) {
-    const dim3 grid((N + kH - 1) / kH, (M + kTR - 1) / kTR, ksplit);
-    gemm_bf16_kernel<<<grid, kTR, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, ksplit);
-}
+// Samples generated ahead per launch of the training loop.  A batch of 4096 is 128 warps on 608 schedulers, each a
+// chain of ~12000 FP64 instructions (0.4 ms however few they are); 65536 samples fill the FP64 pipes (1.36 ms, 0.085
+// a batch).
+constexpr int64_t kTargetsAhead = 65536;
 
 extern "C" void qed_mlp_destroy(qed_mlp_t m) {
     if (!valid_mlp(m)) return;
-    for (float* p : {m->P, m->M, m->V, m->G, m->X, m->T, m->Z1, m->H1, m->Z2, m->H2, m->Z3, m->H3, m->O, m->dO, m->dA,
-                     m->dB, m->loss})
-        cudaFree(p);
+    for (float* p : {m->P, m->M, m->V, m->G, m->X, m->T}) cudaFree(p);
     m->magic = 0;
     delete m;
 }
@@ -1068,14 +1213,11 @@ extern "C" qed_status qed_mlp_create(int64_t max_batch, const float* init_params
     qed_mlp_s* m = new qed_mlp_s();
     m->magic = kMlpMagic;
     m->max_batch = max_batch;
-    const size_t np = sizeof(float) * kParams, nb = (size_t)max_batch;
-    bool ok = cudaMalloc(&m->P, np) == cudaSuccess && cudaMalloc(&m->M, np) == cudaSuccess &&
+    m->sample_room = std::max(max_batch, kTargetsAhead);
+    const size_t np = sizeof(float) * kParams, ns = (size_t)m->sample_room;
+    const bool ok = cudaMalloc(&m->P, np) == cudaSuccess && cudaMalloc(&m->M, np) == cudaSuccess &&
               cudaMalloc(&m->V, np) == cudaSuccess && cudaMalloc(&m->G, np) == cudaSuccess &&
-              cudaMalloc(&m->X, 3 * nb * 4) == cudaSuccess && cudaMalloc(&m->T, 4 * nb * 4) == cudaSuccess;
-    for (float** p : {&m->Z1, &m->H1, &m->Z2, &m->H2, &m->Z3, &m->H3, &m->dA, &m->dB})
-        ok = ok && cudaMalloc(p, kH * nb * 4) == cudaSuccess;
-    ok = ok && cudaMalloc(&m->O, 4 * nb * 4) == cudaSuccess && cudaMalloc(&m->dO, 4 * nb * 4) == cudaSuccess &&
-         cudaMalloc(&m->loss, 4) == cudaSuccess;
+              cudaMalloc(&m->X, 3 * ns * 4) == cudaSuccess && cudaMalloc(&m->T, 4 * ns * 4) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         qed_mlp_destroy(m);
@@ -1118,56 +1260,42 @@ extern "C" qed_status qed_mlp_targets(qed_tables_t t, int64_t n, uint64_t seed, 
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
 }
 
-// forward and backward of one batch (features x, targets y); gradients into grad (kParams floats)
-static void mlp_grad_launch(qed_mlp_s* m, const float* x, const float* y, int64_t n, float* grad, float* loss,
-                            cudaStream_t st) {
-    const float* P = m->P;
-    const int eg = grid_for(n * kH, 256);
-    const int ks = (int)std::min<int64_t>(64, std::max<int64_t>(1, n / 512));
-    mlp_layer1_kernel<<<eg, 256, 0, st>>>(P, x, n, m->Z1, m->H1);
-    gemm((int)n, kH, kH, m->H1, kH, 1, P + kOffW2, 1, kH, m->Z2, kH, 1, st);
-    mlp_bias_silu_kernel<<<eg, 256, 0, st>>>(P + kOffB2, n, m->Z2, m->H2);
-    gemm((int)n, kH, kH, m->H2, kH, 1, P + kOffW3, 1, kH, m->Z3, kH, 1, st);
-    mlp_bias_silu_kernel<<<eg, 256, 0, st>>>(P + kOffB3, n, m->Z3, m->H3);
-    gemm((int)n, 4, kH, m->H3, kH, 1, P + kOffW4, 1, kH, m->O, 4, 1, st);
-    if (loss) cudaMemsetAsync(loss, 0, sizeof(float), st);
-    mlp_out_loss_kernel<<<grid_for(n * 4, 256), 256, 0, st>>>(P, y, n, m->O, m->dO, loss);
-    cudaMemsetAsync(grad, 0, sizeof(float) * kParams, st);
-    // layer 4
-    gemm(4, kH, (int)n, m->dO, 1, 4, m->H3, kH, 1, grad + kOffW4, kH, ks, st);
-    mlp_colsum_kernel<<<4, 256, 0, st>>>(m->dO, n, 4, grad + kOffB4);
-    gemm((int)n, kH, 4, m->dO, 4, 1, P + kOffW4, kH, 1, m->dA, kH, 1, st);
-    mlp_silu_back_kernel<<<eg, 256, 0, st>>>(m->Z3, n, m->dA);
-    // layer 3
-    gemm(kH, kH, (int)n, m->dA, 1, kH, m->H2, kH, 1, grad + kOffW3, kH, ks, st);
-    mlp_colsum_kernel<<<kH, 256, 0, st>>>(m->dA, n, kH, grad + kOffB3);
-    gemm((int)n, kH, kH, m->dA, kH, 1, P + kOffW3, kH, 1, m->dB, kH, 1, st);
-    mlp_silu_back_kernel<<<eg, 256, 0, st>>>(m->Z2, n, m->dB);
-    // layer 2
-    gemm(kH, kH, (int)n, m->dB, 1, kH, m->H1, kH, 1, grad + kOffW2, kH, ks, st);
-    mlp_colsum_kernel<<<kH, 256, 0, st>>>(m->dB, n, kH, grad + kOffB2);
-    gemm((int)n, kH, kH, m->dB, kH, 1, P + kOffW2, kH, 1, m->dA, kH, 1, st);
-    mlp_silu_back_kernel<<<eg, 256, 0, st>>>(m->Z1, n, m->dA);
-    // layer 1 (FP32)
-    mlp_dw1_kernel<<<3 * kH, 256, 0, st>>>(m->dA, x, n, grad);
-    mlp_colsum_kernel<<<kH, 256, 0, st>>>(m->dA, n, kH, grad + kOffB1);
+// forward and backward of one batch (features x, targets y), added to grad (kParams floats) and loss
+static qed_status mlp_grad_launch(qed_mlp_s* m, const float* x, const float* y, int64_t n, float* grad, float* loss,
+                                  cudaStream_t st) {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainShared)) !=
+        cudaSuccess)
+        return QED_ERR_CUDA;
+    const int blocks = (int)std::min<int64_t>((n + kTR - 1) / kTR, sms);
+    mlp_train_kernel<<<blocks, kTrainThreads, sizeof(TrainShared), st>>>(m->P, x, y, n, grad, loss);
+    return QED_OK;
 }
 
 extern "C" qed_status qed_mlp_grad(qed_mlp_t m, const float* x_dev, const float* y_dev, int64_t n, float* grad_dev,
                                    float* loss_dev, void* stream) {
     if (!valid_mlp(m)) return QED_ERR_STATE;
     if (n < 1 || n > m->max_batch || !x_dev || !y_dev || !grad_dev) return QED_ERR_ARG;
-    mlp_grad_launch(m, x_dev, y_dev, n, grad_dev, loss_dev, (cudaStream_t)stream);
+    cudaStream_t st = (cudaStream_t)stream;
+    cudaMemsetAsync(grad_dev, 0, sizeof(float) * kParams, st);
+    if (loss_dev) cudaMemsetAsync(loss_dev, 0, sizeof(float), st);
+    const qed_status s = mlp_grad_launch(m, x_dev, y_dev, n, grad_dev, loss_dev, st);
+    if (s != QED_OK) return s;
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
+}
+
+static void adamw_launch(qed_mlp_s* m, const float* grad, float lr, float weight_decay, float* zero, cudaStream_t st) {
+    m->steps += 1;
+    const float b1t = (float)std::pow(0.9, (double)m->steps), b2t = (float)std::pow(0.999, (double)m->steps);
+    mlp_adamw_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(m->P, m->M, m->V, grad, lr, weight_decay, b1t, b2t, zero);
 }
 
 extern "C" qed_status qed_mlp_adamw(qed_mlp_t m, const float* grad_dev, float lr, float weight_decay, void* stream) {
     if (!valid_mlp(m)) return QED_ERR_STATE;
     if (!grad_dev || !(lr >= 0.0f) || !(weight_decay >= 0.0f)) return QED_ERR_ARG;
-    m->steps += 1;
-    const float b1t = (float)std::pow(0.9, (double)m->steps), b2t = (float)std::pow(0.999, (double)m->steps);
-    mlp_adamw_kernel<<<(kParams + 255) / 256, 256, 0, (cudaStream_t)stream>>>(m->P, m->M, m->V, grad_dev, lr,
-                                                                               weight_decay, b1t, b2t);
+    adamw_launch(m, grad_dev, lr, weight_decay, nullptr, (cudaStream_t)stream);
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
 }
 
@@ -1178,16 +1306,25 @@ extern "C" qed_status qed_mlp_train(qed_mlp_t m, qed_tables_t t, int64_t steps, 
     if (!valid_tables(t)) return QED_ERR_STATE;
     if (steps < 0 || batch < 1 || batch > m->max_batch || first_index < 0 || !(lr >= 0.0f) || !(lr_final >= 0.0f))
         return QED_ERR_ARG;
+    if (!(weight_decay >= 0.0f) && steps > 0) return QED_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
+    const int64_t ahead = m->sample_room / batch;  // whole batches generated per launch
+    cudaMemsetAsync(m->G, 0, sizeof(float) * kParams, st);
+    if (loss_per_step_dev) cudaMemsetAsync(loss_per_step_dev, 0, sizeof(float) * (size_t)steps, st);
     for (int64_t k = 0; k < steps; ++k) {
         // cosine decay from lr to lr_final
         const double c = steps > 1 ? 0.5 * (1.0 + std::cos(3.141592653589793 * (double)k / (double)(steps - 1))) : 1.0;
         const float lrk = (float)(lr_final + (lr - lr_final) * c);
-        qed_status s = qed_mlp_targets(t, batch, seed, first_index + k * batch, m->X, m->T, nullptr, stream);
+        const int64_t at = k % ahead;
+        if (at == 0) {
+            const qed_status s = qed_mlp_targets(t, std::min(ahead, steps - k) * batch, seed, first_index + k * batch, m->X,
+                                                 m->T, nullptr, stream);
+            if (s != QED_OK) return s;
+        }
+        const qed_status s = mlp_grad_launch(m, m->X + 3 * at * batch, m->T + 4 * at * batch, batch, m->G,
+                                             loss_per_step_dev ? loss_per_step_dev + k : nullptr, st);
         if (s != QED_OK) return s;
-        mlp_grad_launch(m, m->X, m->T, batch, m->G, loss_per_step_dev ? loss_per_step_dev + k : nullptr, st);
-        s = qed_mlp_adamw(m, m->G, lrk, weight_decay, stream);
-        if (s != QED_OK) return s;
+        adamw_launch(m, m->G, lrk, weight_decay, m->G, st);
     }
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
 }
