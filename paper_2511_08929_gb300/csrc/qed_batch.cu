@@ -230,16 +230,25 @@ struct WarpSeg {
     int t0, t1, n;  // its tile range and particle count
 };
 
+// Photons that may have a pair rate, queued per warp by the plane-wave kernels: the ten state words of the step (x, P_x;
+// P_y, P_z, tau; k) and the index, a column per photon.
+constexpr int kRateQ = 64;  // drained 32 at a time
+struct RateQ {
+    float v[11][kRateQ];
+    int j[kRateQ];
+};
+
 // shared memory of the batched kernel: the 1-D rate tables (the Bessel table, read only by the event
 // kernel, stays in global memory behind L1), the tile list, the per-warp segment state, the tiles, the
-// event queues and the chunk rings
-__host__ __device__ inline size_t batch_smem_bytes(int warps, int stages, int n_chi, int n_seg) {
+// event queues, the chunk rings and (plane-wave kernels) the rate queues
+__host__ __device__ inline size_t batch_smem_bytes(int warps, int stages, int n_chi, int n_seg, bool rate_queue) {
     size_t off = align128((size_t)4 * n_chi * 4);
     off += align128((size_t)(n_seg + 1) * 4);
     off += align128((size_t)warps * sizeof(WarpSeg));
     off += (size_t)warps * stages * sizeof(Tile);
     off += (size_t)warps * kWQ * 8;
     off += (size_t)warps * kChunkRing * 8;
+    if (rate_queue) off += (size_t)warps * sizeof(RateQ);
     return off;
 }
 
@@ -266,6 +275,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     sh.queue = (int64_t*)(smem + off);
     off += (size_t)WARPS * kWQ * 8;
     int2* s_chunks = (int2*)(smem + off);
+    off += (size_t)WARPS * kChunkRing * 8;
+    RateQ* s_rq = (RateQ*)(smem + off);  // plane-wave kernels only
+    constexpr bool PW = plane_waves_only<FIX>();
 
     for (int i = threadIdx.x; i < 2 * T.n_chi; i += blockDim.x) {
         sh.rates[i] = T.nlc_rate[i];
@@ -338,7 +350,47 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     int cur = -1;  // current segment
     int sp = 0, ii = 0;
     int st = 0;  // stage of the current tile
-    while (t < te) {
+    RateQ& rq = s_rq[warp];
+    int rn = 0;  // queued photons of the current segment (warp-uniform)
+    float chi_z = 0.0f;
+    if (PW) {
+        float m = -1e30f;
+        for (int i = lane; i < 2 * T.n_chi; i += 32) m = fmaxf(m, Tl.nbw_rate[i]);
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        chi_z = no_rate_chi(T, m);
+    }
+    // the events of a pass to the warp's queue, and from there to the list
+    auto list = [&](bool event, int j) {
+        const unsigned m = __ballot_sync(0xffffffffu, event);
+        if (event) wq[qn + __popc(m & ((1u << lane) - 1u))] = ((long long)cur << 32) | (long long)j;
+        qn += __popc(m);
+        __syncwarp();
+        if (qn >= 32) {  // 32 entries to the step's event list with one atomic add
+            qn -= 32;
+            flush(qn, 32, sp == 2);
+        }
+    };
+    while (true) {
+        const bool more = t < te;
+        // photons that may have a pair rate, 32 at a time (or what is left of a segment, whose context goes)
+        if (PW && (rn >= 32 || (rn > 0 && (!more || t >= WS.t1)))) {
+            const int cnt = min(rn, 32);
+            rn -= cnt;
+            bool event = false;
+            int j = 0;
+            if (lane < cnt) {
+                const int e = rn + lane;
+                j = rq.j[e];
+                const float4 a = make_float4(rq.v[0][e], rq.v[1][e], rq.v[2][e], rq.v[3][e]);
+                const float4 b = make_float4(rq.v[4][e], rq.v[5][e], rq.v[6][e], rq.v[7][e]);
+                const float4 cc = make_float4(rq.v[8][e], rq.v[9][e], rq.v[10][e], 0.0f);
+                event = photon_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl);
+            }
+            __syncwarp();
+            list(event, j);
+            continue;
+        }
+        if (!more) break;
         cp_async_wait<STAGES - 1>();  // this lane's copies of the current tile have landed
         if (t >= WS.t1) {  // the tile lies in a later segment
             do ++cur;
@@ -408,16 +460,23 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
         }
         if (++st == STAGES) st = 0;
         bool event = false;
-        if (valid)
-            event = sp == 2 ? photon_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl)
-                            : lepton_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl);
-        const unsigned m = __ballot_sync(0xffffffffu, event);
-        if (event) wq[qn + __popc(m & ((1u << lane) - 1u))] = ((long long)cur << 32) | (long long)j;
-        qn += __popc(m);
-        __syncwarp();
-        if (qn >= 32) {  // 32 entries to the step's event list with one atomic add
-            qn -= 32;
-            flush(qn, 32, sp == 2);
+        if (PW && sp == 2) {
+            const bool rate = valid && photon_needs_rate<FIX ? FIX : QED_F_FULL>(C, WS.L, j, a, b, cc, chi_z, ctr, c);
+            const unsigned m = __ballot_sync(0xffffffffu, rate);
+            if (rate) {
+                const int e = rn + __popc(m & ((1u << lane) - 1u));
+                rq.v[0][e] = a.x; rq.v[1][e] = a.y; rq.v[2][e] = a.z; rq.v[3][e] = a.w;
+                rq.v[4][e] = b.x; rq.v[5][e] = b.y; rq.v[6][e] = b.z; rq.v[7][e] = b.w;
+                rq.v[8][e] = cc.x; rq.v[9][e] = cc.y; rq.v[10][e] = cc.z;
+                rq.j[e] = j;
+            }
+            rn += __popc(m);
+            __syncwarp();
+        } else {
+            if (valid)
+                event = !PW && sp == 2 ? photon_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl)
+                                       : lepton_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl);
+            list(event, j);
         }
         if (++t == te) {  // the chunk is done: the next one (its entry was written when its copies began)
             ch = ring[rk++ & (kChunkRing - 1)];
@@ -666,7 +725,7 @@ struct qed_batch_s {
 template <int WARPS, int STAGES, int MINB, uint32_t FIX>
 static void launch_variant(const qed_batch_s* b, int grid, cudaStream_t st) {
     const qed_tables_s* t = b->tables;
-    const size_t smem = batch_smem_bytes(WARPS, STAGES, t->desc.n_chi, kSpecies * b->n_inst);
+    const size_t smem = batch_smem_bytes(WARPS, STAGES, t->desc.n_chi, kSpecies * b->n_inst, plane_waves_only<FIX>());
     BatchP P;
     P.flags = b->desc.flags;
     P.dt_f = (float)b->desc.dt;
@@ -687,12 +746,13 @@ static void launch_variant(const qed_batch_s* b, int grid, cudaStream_t st) {
 // [0]: flags read at run time; [1]: built for QED_F_FULL (every flag test of the streaming pass folded)
 static const BatchVariant kVariants[2][QED_BATCH_VARIANTS] = {QED_VARIANTS(0u), QED_VARIANTS(QED_F_FULL)};
 
-static const BatchVariant& variant_of(const qed_batch_s* b, int v) {
-    return kVariants[b->desc.flags == QED_F_FULL && b->plane_waves ? 1 : 0][v];
-}
+static bool fixed_kernel(const qed_batch_s* b) { return b->desc.flags == QED_F_FULL && b->plane_waves; }
+
+static const BatchVariant& variant_of(const qed_batch_s* b, int v) { return kVariants[fixed_kernel(b) ? 1 : 0][v]; }
 
 static size_t variant_smem(const qed_batch_s* b, int v) {
-    return batch_smem_bytes(variant_of(b, v).warps, variant_of(b, v).stages, b->tables->desc.n_chi, kSpecies * b->n_inst);
+    return batch_smem_bytes(variant_of(b, v).warps, variant_of(b, v).stages, b->tables->desc.n_chi, kSpecies * b->n_inst,
+                            fixed_kernel(b));
 }
 
 // resident blocks per SM of variant v for this batch (0 if it does not fit)

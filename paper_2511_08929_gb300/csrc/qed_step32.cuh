@@ -899,6 +899,24 @@ struct PState {
     float chi, lnchi, xi[3], Wp, Wm, Wmp, Wx;
 };
 
+// |k| and k-hat of a photon; returns |k|^2 (nonzero exactly when k is)
+__device__ __forceinline__ float photon_direction(const F3& k, float& en, F3& khat) {
+    float en2 = dot(k, k);
+    if (en2 < 0x1.0p-100f) {
+        // |k|^2 near or below the float range (photons of ~1e-15 mc^2 and softer, a few per 1e8 emissions
+        // in the NLC spectrum's lambda^(1/3) tail): the components scaled by 2^100 keep k-hat's precision
+        const F3 ks = 0x1.0p+100f * k;
+        const float e2s = dot(ks, ks);
+        en = sqrt_(e2s) * 0x1.0p-100f;
+        khat = e2s > 0.0f ? rsqrtf(e2s) * ks : F3{0, 0, 0};
+        en2 = e2s > 0.0f ? fmaxf(en2, 0x1.0p-149f) : 0.0f;
+    } else {
+        en = sqrt_(en2);
+        khat = rsqrtf(en2) * k;
+    }
+    return en2;
+}
+
 template <uint32_t FIX = 0, bool ACC = false>
 __device__ __forceinline__ void photon_classical(const Ctx& C, const float4& a, const float4& b, const float4& cc, PState& st,
                                                  unsigned long long* c,
@@ -910,19 +928,7 @@ __device__ __forceinline__ void photon_classical(const Ctx& C, const float4& a, 
     st.w = cc.w;
     constexpr bool PW = plane_waves_only<FIX>();
     field_eval<float, ACC, PW>(C.F, C.S.ph_hi_f, C.S.ph_lo_f, xold, st.E, st.B);
-    float en2 = dot(st.k, st.k);
-    if (en2 < 0x1.0p-100f) {
-        // |k|^2 near or below the float range (photons of ~1e-15 mc^2 and softer, a few per 1e8 emissions
-        // in the NLC spectrum's lambda^(1/3) tail): the components scaled by 2^100 keep k-hat's precision
-        const F3 ks = 0x1.0p+100f * st.k;
-        const float e2s = dot(ks, ks);
-        st.en = sqrt_(e2s) * 0x1.0p-100f;
-        st.khat = e2s > 0.0f ? rsqrtf(e2s) * ks : F3{0, 0, 0};
-        en2 = e2s > 0.0f ? fmaxf(en2, 0x1.0p-149f) : 0.0f;  // nonzero exactly when k is
-    } else {
-        st.en = sqrt_(en2);
-        st.khat = rsqrtf(en2) * st.k;
-    }
+    const float en2 = photon_direction(st.k, st.en, st.khat);
     st.x = xold;
     if (flags_of<FIX>(C) & QED_F_MOVE) st.x = axpy(C.S.dt_f, st.khat, xold);
     st.qed = false;
@@ -1101,6 +1107,40 @@ __device__ __forceinline__ bool photon_stream_one(const Ctx& C, const PartDev& G
     }
     store_photon32_step(G, j, st.x, Pf, tauf);
     c[C_RATE_STEPS]++;
+    return false;
+}
+
+// Below this chi both pair rates are zero in FP32: J = exp(ln(J e^{8/(3 chi)}) - 8/(3 chi)) leaves the normal float
+// range (e^-88 is half its smallest number; results below it are flushed) whatever the table's entry, at most m, adds.
+__device__ __forceinline__ float no_rate_chi(const TabP<float>& T, float m) {
+    return fmaxf(T.chi_min, (float)(8.0 / 3.0) / (88.0f + fmaxf(m, 0.0f)));
+}
+
+// The first part of a photon's step in a plane wave: most photons are too soft, or outside the pulse, for a pair rate
+// in the float range, and only move.  chi <= eta0 (e + max(-k_z, 0)) |a| with a the wave's amplitude at the photon, the
+// number field_eval forms; where that bound, raised by more than its rounding, lies below chi_z (no_rate_chi) the full
+// step would find no rate and write the same position, which is written here.  Returns true for the others (nothing
+// written).
+template <uint32_t FIX>
+__device__ __forceinline__ bool photon_needs_rate(const Ctx& C, const PartDev& G, int64_t j, const float4& a, const float4& b,
+                                                  const float4& cc, float chi_z, qed_counters* ctr, unsigned long long* c) {
+    static_assert(plane_waves_only<FIX>(), "the bound is that of a single plane wave");
+    if (!finite_photon(a, b, cc)) {
+        c[C_NONFINITE]++;
+        record_error(ctr, QED_ERR_NAN, j);
+        return false;
+    }
+    const F3 x{a.x, a.y, a.z}, k{cc.x, cc.y, cc.z};
+    float en;
+    F3 khat;
+    photon_direction(k, en, khat);
+    float e1;
+    const float ps = two_sum(C.S.ph_hi_f, -x.z, e1);
+    const float amp = C.F.a0 * envelope(ps + (e1 + C.S.ph_lo_f), C.F);
+    const float bound = C.F.eta0 * (en + fmaxf(-k.z, 0.0f)) * fabsf(amp) * 1.0001f;
+    if (!(bound < chi_z)) return true;
+    const F3 xn = (FIX & QED_F_MOVE) ? axpy(C.S.dt_f, khat, x) : x;
+    G.q0[j] = make_float4(xn.x, xn.y, xn.z, a.w);
     return false;
 }
 
