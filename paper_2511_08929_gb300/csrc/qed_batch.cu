@@ -2,10 +2,7 @@
 // time step, the step index and time on the device (so a CUDA graph of whole steps replays unchanged),
 // and an autotuner for the launch shape.
 //
-// One time step of the batch is eight launches on one stream:
-//   plan      alive counts at step start (counts clamped to capacity), the tile list over all segments
-//             (segment = one species of one instance, species-major), each segment's step context,
-//             particle-step accounting;
+// One time step of the batch is four launches on one stream:
 //   step      the persistent kernel: every warp takes runs of consecutive tiles from a work counter
 //             (guided: long runs first, short ones at the end, at most `chunk` tiles) and streams them
 //             through shared memory with per-lane asynchronous copies, running the per-particle
@@ -16,8 +13,11 @@
 //             the persistent kernel, whose registers then hold only the streaming pass: no calls, no
 //             spills): one kernel for the lepton events in FP32, one for what is FP64 (the photon events,
 //             and the lepton events whose FP32 spectra cancel);
-//   compact   head / classify / tail / move of every instance's photons (converted photons leave,
-//             Sec. 4.3), the last one also advancing the device step counter.
+//   finish    per instance the daughters' counts, the compaction of its photons (converted photons leave,
+//             Sec. 4.3) and the plan of the next step: alive counts at its start, each segment's step
+//             context (segment = one species of one instance), the tile list over all segments
+//             (species-major); then the device step counter and the particle-step accounting.
+// A plan kernel makes the first step's plan of every call.
 // Daughters appended during a step sit beyond the counts taken by `plan`, so they are first stepped in
 // the next step (the begin snapshot of the single-buffer path).
 #include <cstdio>
@@ -43,7 +43,7 @@ struct InstDev {
     int64_t* holes;  // photon compaction scratch of this instance
     int64_t* live;
     uint8_t* mark;
-    int64_t* hdr;  // [0] n, [1] D, [2] holes found, [3] live found
+    int64_t* hdr;  // [0] holes found, [1] live found (zero between steps)
     AppendState* app;  // daughter reservations of the step: [0] photons (lepton events), [1] pairs
 };
 
@@ -58,10 +58,14 @@ struct ClockDev {
     unsigned long long psteps;
     unsigned long long species_steps[kSpecies];
     long long alive[kSpecies];
-    int next_tile;  // the persistent kernel's work counter (tiles handed out), reset by the plan kernel
-    unsigned long long n_list[2];  // the step's listed events (leptons, photons), reset by the plan kernel
-    unsigned long long n_exact;    // lepton events to be taken again in FP64, reset by the plan kernel
-    unsigned long long n_events;   // events of the last step (both kinds)
+    // of the step in flight, set by its plan: particles to process, the persistent kernel's work counter (tiles handed
+    // out), the listed events (leptons, photons), the lepton events to be taken again in FP64
+    unsigned long long planned[kSpecies];
+    int next_tile;
+    unsigned int finished;  // instances the finish kernel is done with
+    unsigned long long n_list[2];
+    unsigned long long n_exact;
+    unsigned long long n_events;  // events of the last step (both kinds)
 };
 
 struct BatchP {
@@ -70,44 +74,94 @@ struct BatchP {
     double store_min, chi_floor;
 };
 
-// The step context of one segment (one species of one instance), written by the plan kernel every
-// step for the event kernel: its lanes take events of several segments at once.
+// The step context of one segment (one species of one instance) for the event kernels, whose lanes take events of
+// several segments at once: made when the batch is created, its step index and phase rewritten by every plan.
 struct SegCtx {
     Ctx C;       // tables (global memory), field, step parameters and charge
     int ii, sp;  // instance and species
 };
 
 // ------------------------------------------------------------------------------------------------
-// plan: one block of kPlanThreads threads, each owning up to 3 consecutive segments
+// plan of a step: per instance its particle counts (clamped to capacity), contexts and daughter reservations; then
+// the tile list over all segments.  A plan kernel makes it when the caller asks for steps (it may have changed its
+// buffers since the last one); within a call the finish kernel of each step plans the next.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPlanThreads = 1024;
 
-__global__ void __launch_bounds__(kPlanThreads)
-    batch_plan_kernel(const InstDev* __restrict__ inst, int n_inst, SegDev* seg, int64_t* tile0, ClockDev* clk,
-                      SegCtx* ctx, TabP<float> T, const float* bes, BatchP P) {
+// once per batch: what no step changes
+__global__ void batch_init_kernel(const InstDev* __restrict__ inst, int n_inst, SegDev* seg, SegCtx* ctx, const ClockDev* clk,
+                                  TabP<float> T, const float* bes, BatchP P) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= kSpecies * n_inst) return;
+    const int sp = s / n_inst, i = s - sp * n_inst;
+    const InstDev& I = inst[i];
+    seg[s] = SegDev{I.sp[sp].q0, I.sp[sp].q1, I.sp[sp].q2, 0};
+    SegCtx& X = ctx[s];
+    X.ii = i;
+    X.sp = sp;
+    X.C.T = T;
+    X.C.bes = bes;
+    X.C.F = I.F;
+    X.C.q = sp == 0 ? -1.0f : (sp == 1 ? 1.0f : 0.0f);
+    StepP& S = X.C.S;
+    S.dt = clk->dt;
+    S.dt_f = P.dt_f;
+    S.flags = P.flags;
+    S.seed = I.seed;
+    S.store_min = P.store_min;
+    S.chi_floor = P.chi_floor;
+    S.store_min_f = (float)P.store_min;
+    S.chi_floor_f = (float)P.chi_floor;
+}
+
+// one thread per species: segment (instance i, species sp) of step `step` with n particles
+__device__ __forceinline__ void plan_segment(const InstDev& I, int i, int sp, int64_t n, int n_inst, uint64_t step,
+                                             const ClockDev* clk, SegDev* seg, SegCtx* ctx) {
+    const int s = sp * n_inst + i;
+    seg[s].n = n;
+    // time of this step: a product then a sum, each rounded (no contraction)
+    const double t_now = __dadd_rn(clk->t0, __dmul_rn((double)(step - clk->step0), clk->dt));
+    StepP& S = ctx[s].C.S;
+    const double ph = __dadd_rn(t_now, I.phase);
+    S.ph_hi = ph;
+    S.ph_hi_f = (float)ph;
+    S.ph_lo_f = (float)(ph - (double)(float)ph);
+    S.step = step;
+}
+
+// the instance's daughter reservations from its (clamped) counts at step start
+__device__ __forceinline__ void plan_appends(const InstDev& I, int64_t ne, int64_t np, int64_t ng) {
+    I.app[0] = AppendState{{ng, 0}, I.sp[2].capacity - ng, 0ull};
+    I.app[1] = AppendState{{ne, np}, min(I.sp[0].capacity - ne, I.sp[1].capacity - np), 0ull};
+}
+
+// one block: the tile list from the segments' counts (species-major), the particles per species, the step's counters
+__device__ void plan_tiles(int n_inst, const SegDev* seg, int64_t* tile0, ClockDev* clk) {
     __shared__ long long wsum[32];
     __shared__ unsigned long long tot[kSpecies];
     const int n_seg = kSpecies * n_inst;
-    const int per = (n_seg + kPlanThreads - 1) / kPlanThreads;  // <= 3
-    const int s0 = threadIdx.x * per;
+    const int per = (n_seg + blockDim.x - 1) / blockDim.x;
+    const int s0 = threadIdx.x * per, s1 = min(s0 + per, n_seg);
     if (threadIdx.x < kSpecies) tot[threadIdx.x] = 0;
     __syncthreads();
-    long long loc[3] = {0, 0, 0}, mine = 0;
-    for (int k = 0; k < per; ++k) {
-        const int s = s0 + k;
-        if (s >= n_seg) break;
-        const int sp = s / n_inst, i = s - sp * n_inst;
-        const PartDev& Pd = inst[i].sp[sp];
-        const int64_t c = *Pd.count;
-        const int64_t n = c < 0 ? 0 : (c > Pd.capacity ? Pd.capacity : c);
-        if (c != n) *Pd.count = n;  // reservations that did not fit
-        seg[s] = SegDev{Pd.q0, Pd.q1, Pd.q2, n};
-        loc[k] = (n + 31) / 32;
-        mine += loc[k];
-        atomicAdd(&tot[sp], (unsigned long long)n);
+    constexpr int kHeld = 4;  // counts held in registers (96 instances: 2 a thread of 256)
+    int64_t held[kHeld];
+#pragma unroll
+    for (int k = 0; k < kHeld; ++k) held[k] = s0 + k < s1 ? __ldcg(&seg[s0 + k].n) : 0;
+    long long mine = 0;
+    unsigned long long sum[kSpecies] = {0, 0, 0};
+    for (int s = s0; s < s1; ++s) {
+        const int64_t n = s - s0 < kHeld ? held[0] : __ldcg(&seg[s].n);
+#pragma unroll
+        for (int k = 0; k + 1 < kHeld; ++k) held[k] = held[k + 1];
+        mine += (n + 31) / 32;
+        const int sp = s / n_inst;
+        sum[0] += sp == 0 ? n : 0;
+        sum[1] += sp == 1 ? n : 0;
+        sum[2] += sp == 2 ? n : 0;
     }
     // block-wide exclusive scan of the per-thread tile counts
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
     long long incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -115,9 +169,13 @@ __global__ void __launch_bounds__(kPlanThreads)
         if (lane >= o) incl += v;
     }
     if (lane == 31) wsum[wid] = incl;
+    for (int k = 0; k < kSpecies; ++k) {
+        const unsigned long long v = warp_sum(sum[k]);
+        if (lane == 0 && v) atomicAdd(&tot[k], v);
+    }
     __syncthreads();
     if (wid == 0) {
-        long long v = wsum[lane], x = v;
+        long long v = lane < warps ? wsum[lane] : 0, x = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const long long u = __shfl_up_sync(0xffffffffu, x, o);
@@ -128,52 +186,35 @@ __global__ void __launch_bounds__(kPlanThreads)
     }
     __syncthreads();
     long long ex = wsum[wid] + incl - mine;
-    const uint64_t step = clk->step;
-    // time of this step: a product then a sum, each rounded (no contraction)
-    const double t_now = __dadd_rn(clk->t0, __dmul_rn((double)(step - clk->step0), clk->dt));
-    for (int k = 0; k < per; ++k) {
-        const int s = s0 + k;
-        if (s >= n_seg) break;
+    for (int s = s0; s < s1; ++s) {
         tile0[s] = ex;
-        ex += loc[k];
-        const int sp = s / n_inst, i = s - sp * n_inst;
-        const InstDev& I = inst[i];
-        SegCtx& X = ctx[s];
-        X.ii = i;
-        X.sp = sp;
-        X.C.T = T;
-        X.C.bes = bes;
-        X.C.F = I.F;
-        X.C.q = sp == 0 ? -1.0f : (sp == 1 ? 1.0f : 0.0f);
-        StepP& S = X.C.S;
-        S.dt = clk->dt;
-        S.ph_hi = __dadd_rn(t_now, I.phase);
-        S.ph_hi_f = (float)S.ph_hi;
-        S.ph_lo_f = (float)(S.ph_hi - (double)S.ph_hi_f);
-        S.dt_f = P.dt_f;
-        S.flags = P.flags;
-        S.step = step;
-        S.seed = I.seed;
-        S.store_min = P.store_min;
-        S.chi_floor = P.chi_floor;
-        S.store_min_f = (float)P.store_min;
-        S.chi_floor_f = (float)P.chi_floor;
+        if (s + 1 < s1) ex += (__ldcg(&seg[s].n) + 31) / 32;
     }
-    // open every instance's daughter reservations from the counts at step start (clamped above)
-    for (int i = threadIdx.x; i < n_inst; i += blockDim.x) {
-        const InstDev& I = inst[i];
-        append_open(&I.app[0], I.sp[2].count, I.sp[2].capacity, nullptr, 0);
-        append_open(&I.app[1], I.sp[0].count, I.sp[0].capacity, I.sp[1].count, I.sp[1].capacity);
-    }
+    if (threadIdx.x < kSpecies) clk->planned[threadIdx.x] = tot[threadIdx.x];
     if (threadIdx.x == 0) {
         clk->next_tile = 0;
+        clk->finished = 0;
         clk->n_list[0] = clk->n_list[1] = clk->n_exact = 0;
-        clk->psteps += tot[0] + tot[1] + tot[2];
-        for (int k = 0; k < kSpecies; ++k) {
-            clk->species_steps[k] += tot[k];
-            clk->alive[k] = (long long)tot[k];
-        }
     }
+}
+
+__global__ void __launch_bounds__(kPlanThreads)
+    batch_plan_kernel(const InstDev* __restrict__ inst, int n_inst, SegDev* seg, int64_t* tile0, ClockDev* clk, SegCtx* ctx) {
+    const uint64_t step = clk->step;
+    for (int i = threadIdx.x; i < n_inst; i += kPlanThreads) {
+        const InstDev& I = inst[i];
+        int64_t n[kSpecies];
+        for (int sp = 0; sp < kSpecies; ++sp) {
+            const PartDev& Pd = I.sp[sp];
+            const int64_t c = *Pd.count;
+            n[sp] = c < 0 ? 0 : (c > Pd.capacity ? Pd.capacity : c);
+            if (c != n[sp]) *Pd.count = n[sp];  // a count its caller left outside the buffer
+            plan_segment(I, i, sp, n[sp], n_inst, step, clk, seg, ctx);
+        }
+        plan_appends(I, n[0], n[1], n[2]);
+    }
+    __syncthreads();
+    plan_tiles(n_inst, seg, tile0, clk);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -606,65 +647,83 @@ __global__ void __launch_bounds__(256) batch_mlp_prep_kernel(const InstDev* __re
 }
 
 // ------------------------------------------------------------------------------------------------
-// photon compaction of every instance (grid.y = instance); the same hole filling as qed_compact
+// the end of a step, one cluster of 8 blocks per instance: its daughters' counts, the compaction of its photons
+// (grid-stride over the dead list; the same hole filling as qed_compact), the plan of its next step; the last
+// instance's first block then makes the tile list and advances the device clock.  The compaction's phases meet at
+// cluster barriers: as four launches, with the plan a fifth, they took 20 us a step for 8 small instances, 34 for 96 and
+// 35 for a cascade's one; this kernel takes 12, 15 and 21.
 // ------------------------------------------------------------------------------------------------
-constexpr int kCompactBlocks = 8;  // blocks per instance (grid-stride over the dead list)
+constexpr int kFinishCluster = 8;
 
-__global__ void batch_compact_head(const InstDev* __restrict__ inst, int n_inst) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_inst) return;
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(kFinishCluster, 1, 1)
+    batch_finish_kernel(const InstDev* __restrict__ inst, int n_inst, SegDev* seg, int64_t* tile0, ClockDev* clk, SegCtx* ctx) {
+    __shared__ bool last;
+    const int i = blockIdx.y;
     const InstDev& I = inst[i];
     const PartDev& G = I.sp[2];
-    // close the step's daughter reservations: the counts after this step's appends
-    append_close(&I.app[0], G.count, nullptr);
-    append_close(&I.app[1], I.sp[0].count, I.sp[1].count);
-    const int64_t n = max((int64_t)0, min(*G.count, G.capacity));
-    I.hdr[0] = n;
-    I.hdr[1] = max((int64_t)0, min(*G.n_dead, n));
-    I.hdr[2] = 0;
-    I.hdr[3] = 0;
-}
-
-__global__ void batch_compact_classify(const InstDev* __restrict__ inst) {
-    const InstDev& I = inst[blockIdx.y];
-    const int64_t n = I.hdr[0], D = I.hdr[1], lim = n - D;
-    const int64_t* dead = I.sp[2].dead;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < D; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t d = dead[k];
-        if (d < 0 || d >= n) continue;
-        if (d >= lim) I.mark[d - lim] = 1;
-        else I.holes[atomicAdd((unsigned long long*)&I.hdr[2], 1ull)] = d;
-    }
-}
-
-__global__ void batch_compact_tail(const InstDev* __restrict__ inst) {
-    const InstDev& I = inst[blockIdx.y];
-    const int64_t n = I.hdr[0], D = I.hdr[1], lim = n - D;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < D; k += (int64_t)gridDim.x * blockDim.x) {
-        if (I.mark[k]) I.mark[k] = 0;
-        else I.live[atomicAdd((unsigned long long*)&I.hdr[3], 1ull)] = lim + k;
-    }
-}
-
-__global__ void batch_compact_move(const InstDev* __restrict__ inst, ClockDev* clk) {
-    const InstDev& I = inst[blockIdx.y];
-    const PartDev& G = I.sp[2];
-    const int64_t nh = min(I.hdr[2], I.hdr[3]);
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nh; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t src = I.live[k], dst = I.holes[k];
-        G.q0[dst] = G.q0[src];
-        G.q1[dst] = G.q1[src];
-        G.q2[dst] = G.q2[src];
-        G.id[dst] = G.id[src];
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *G.count = I.hdr[0] - I.hdr[1];
-        *G.n_dead = 0;
-        if (blockIdx.y == 0) {
-            clk->step += 1;  // the step is complete: advance the device clock
-            clk->n_events = clk->n_list[0] + clk->n_list[1];
+    // the counts after this step's appends (reservations beyond a budget were refused)
+    const AppendState A0 = I.app[0], A1 = I.app[1];
+    const int64_t n = A0.base[0] + min((int64_t)A0.next, A0.budget), pairs = min((int64_t)A1.next, A1.budget);
+    const int64_t D = max((int64_t)0, min(*G.n_dead, n)), lim = n - D;
+    const uint64_t step = clk->step + 1;
+    const int64_t k0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)kFinishCluster * blockDim.x;
+    if (D > 0) {  // (the same in every block of the cluster)
+        for (int64_t k = k0; k < D; k += stride) {
+            const int64_t d = G.dead[k];
+            if (d < 0 || d >= n) continue;
+            if (d >= lim) I.mark[d - lim] = 1;
+            else I.holes[atomicAdd((unsigned long long*)&I.hdr[0], 1ull)] = d;
+        }
+        cluster_sync();
+        for (int64_t k = k0; k < D; k += stride) {
+            if (__ldcg(&I.mark[k])) I.mark[k] = 0;
+            else I.live[atomicAdd((unsigned long long*)&I.hdr[1], 1ull)] = lim + k;
+        }
+        cluster_sync();
+        const int64_t nh = min(__ldcg(&I.hdr[0]), __ldcg(&I.hdr[1]));
+        for (int64_t k = k0; k < nh; k += stride) {
+            const int64_t src = __ldcg(&I.live[k]), dst = __ldcg(&I.holes[k]);
+            G.q0[dst] = G.q0[src];
+            G.q1[dst] = G.q1[src];
+            G.q2[dst] = G.q2[src];
+            G.id[dst] = G.id[src];
         }
     }
+    cluster_sync();  // every block has read the instance's counts and list lengths
+    if (blockIdx.x != 0) return;
+    if (threadIdx.x < kSpecies) {
+        const int sp = threadIdx.x;
+        const int64_t c = sp == 2 ? lim : A1.base[sp] + pairs;
+        *I.sp[sp].count = c;
+        plan_segment(I, i, sp, c, n_inst, step, clk, seg, ctx);
+        __threadfence();
+    }
+    __syncwarp();
+    if (threadIdx.x == 0) {
+        *G.n_dead = 0;
+        I.hdr[0] = I.hdr[1] = 0;
+        plan_appends(I, A1.base[0] + pairs, A1.base[1] + pairs, lim);
+        __threadfence();
+        last = atomicAdd(&clk->finished, 1u) == (unsigned)n_inst - 1u;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x == 0) {  // the step is complete
+        clk->step = step;
+        clk->n_events = clk->n_list[0] + clk->n_list[1];
+        for (int k = 0; k < kSpecies; ++k) {
+            clk->psteps += clk->planned[k];
+            clk->species_steps[k] += clk->planned[k];
+            clk->alive[k] = (long long)clk->planned[k];
+        }
+    }
+    __syncthreads();
+    plan_tiles(n_inst, seg, tile0, clk);
 }
 
 }  // namespace qed
@@ -772,13 +831,6 @@ static bool valid_batch(const qed_batch_s* b) { return b != nullptr && b->magic 
 static void launch_batch_step(const qed_batch_s* b, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1,
                               bool capturing = false) {
     const unsigned rec = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
-    BatchP P;
-    P.flags = b->desc.flags;
-    P.dt_f = (float)b->desc.dt;
-    P.store_min = b->desc.photon_store_min;
-    P.chi_floor = b->desc.chi_floor;
-    batch_plan_kernel<<<1, kPlanThreads, 0, st>>>(b->d_inst, b->n_inst, b->d_seg, b->d_tile0, b->d_clk, b->d_ctx,
-                                                  tab_params<float>(b->tables), b->tables->bes32, P);
     if (e0) cudaEventRecordWithFlags(e0, st, rec);
     variant_of(b, b->tuning.variant).launch(b, b->grid, st);
     if (b->mlp) {  // the learned sampler draws every listed emission's energy fraction
@@ -793,11 +845,15 @@ static void launch_batch_step(const qed_batch_s* b, cudaStream_t st, cudaEvent_t
     batch_event64_kernel<<<b->ev64_grid, kEvent64Threads, 0, st>>>(b->d_inst, b->d_ctx, b->d_ev, b->capacity_total,
                                                                    b->d_clk, X64, b->ctr, b->mlp != nullptr);
     if (e1) cudaEventRecordWithFlags(e1, st, rec);
-    batch_compact_head<<<(b->n_inst + 255) / 256, 256, 0, st>>>(b->d_inst, b->n_inst);
-    const dim3 g(kCompactBlocks, b->n_inst);
-    batch_compact_classify<<<g, 256, 0, st>>>(b->d_inst);
-    batch_compact_tail<<<g, 256, 0, st>>>(b->d_inst);
-    batch_compact_move<<<g, 256, 0, st>>>(b->d_inst, b->d_clk);
+    // (a single large instance has as many converted photons as 8 blocks of 256 threads take several rounds for)
+    const int threads = b->n_inst <= 32 ? 1024 : 256;
+    batch_finish_kernel<<<dim3(kFinishCluster, b->n_inst), threads, 0, st>>>(b->d_inst, b->n_inst, b->d_seg, b->d_tile0,
+                                                                             b->d_clk, b->d_ctx);
+}
+
+// the plan of the next step from the buffers as they are (before the first step of a call)
+static void launch_plan(const qed_batch_s* b, cudaStream_t st) {
+    batch_plan_kernel<<<1, kPlanThreads, 0, st>>>(b->d_inst, b->n_inst, b->d_seg, b->d_tile0, b->d_clk, b->d_ctx);
 }
 
 // the caller's event pair k (modulo their number), or none
@@ -962,6 +1018,17 @@ extern "C" qed_status qed_batch_create(qed_tables_t t, const qed_instance* insta
         qed_batch_destroy(b);
         return QED_ERR_CUDA;
     }
+    BatchP P;
+    P.flags = desc->flags;
+    P.dt_f = (float)desc->dt;
+    P.store_min = desc->photon_store_min;
+    P.chi_floor = desc->chi_floor;
+    batch_init_kernel<<<(n_seg + 255) / 256, 256>>>(b->d_inst, n_inst, b->d_seg, b->d_ctx, b->d_clk, tab_params<float>(t),
+                                                    t->bes32, P);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) {
+        qed_batch_destroy(b);
+        return QED_ERR_CUDA;
+    }
     int ev_per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ev_per_sm, batch_event_kernel, kEventThreads, 0);
     b->ev_grid = b->sms * std::max(1, ev_per_sm);
@@ -1006,8 +1073,11 @@ extern "C" qed_status qed_batch_step(qed_batch_t b, int32_t n_steps, void* strea
             }
             b->exec_steps = G;
         }
+        if (n_steps > 0) launch_plan(b, st);
         for (; done + G <= n_steps; done += G)
             if (cudaGraphLaunch(b->exec, st) != cudaSuccess) return QED_ERR_CUDA;
+    } else if (n_steps > 0) {
+        launch_plan(b, st);
     }
     for (; done < n_steps; ++done) {
         cudaEvent_t e0, e1;
@@ -1187,6 +1257,7 @@ extern "C" qed_status qed_batch_tune(qed_batch_t b, int32_t steps_per_candidate,
                 break;
             }
             double ms = 0.0;
+            launch_plan(b, st);
             for (int r = 0; r < steps_per_candidate; ++r) {
                 launch_batch_step(b, st, e0, e1);
                 float x = 0.0f;
