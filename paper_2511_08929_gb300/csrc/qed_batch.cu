@@ -271,13 +271,7 @@ struct WarpSeg {
     int t0, t1, n;  // its tile range and particle count
 };
 
-// Photons that may have a pair rate, queued per warp by the plane-wave kernels: the ten state words of the step (x, P_x;
-// P_y, P_z, tau; k) and the index, a column per photon.
-constexpr int kRateQ = 64;  // drained 32 at a time
-struct RateQ {
-    float v[11][kRateQ];
-    int j[kRateQ];
-};
+using BatchRateQ = RateQT<int>;  // (a batch's buffers hold at most INT32_MAX particles)
 
 // shared memory of the batched kernel: the 1-D rate tables (the Bessel table, read only by the event
 // kernel, stays in global memory behind L1), the tile list, the per-warp segment state, the tiles, the
@@ -289,7 +283,7 @@ __host__ __device__ inline size_t batch_smem_bytes(int warps, int stages, int n_
     off += (size_t)warps * stages * sizeof(Tile);
     off += (size_t)warps * kWQ * 8;
     off += (size_t)warps * kChunkRing * 8;
-    if (rate_queue) off += (size_t)warps * sizeof(RateQ);
+    if (rate_queue) off += (size_t)warps * sizeof(BatchRateQ);
     return off;
 }
 
@@ -317,7 +311,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     off += (size_t)WARPS * kWQ * 8;
     int2* s_chunks = (int2*)(smem + off);
     off += (size_t)WARPS * kChunkRing * 8;
-    RateQ* s_rq = (RateQ*)(smem + off);  // plane-wave kernels only
+    BatchRateQ* s_rq = (BatchRateQ*)(smem + off);  // plane-wave kernels only (the offset so far is a multiple of 8)
     constexpr bool PW = plane_waves_only<FIX>();
 
     for (int i = threadIdx.x; i < 2 * T.n_chi; i += blockDim.x) {
@@ -391,15 +385,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     int cur = -1;  // current segment
     int sp = 0, ii = 0;
     int st = 0;  // stage of the current tile
-    RateQ& rq = s_rq[warp];
+    BatchRateQ& rq = s_rq[warp];
     int rn = 0;  // queued photons of the current segment (warp-uniform)
     float chi_z = 0.0f;
-    if (PW) {
-        float m = -1e30f;
-        for (int i = lane; i < 2 * T.n_chi; i += 32) m = fmaxf(m, Tl.nbw_rate[i]);
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        chi_z = no_rate_chi(T, m);
-    }
+    if (PW) chi_z = no_rate_chi(T, Tl.nbw_rate);
     // the events of a pass to the warp's queue, and from there to the list
     auto list = [&](bool event, int j) {
         const unsigned m = __ballot_sync(0xffffffffu, event);
@@ -420,11 +409,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
             bool event = false;
             int j = 0;
             if (lane < cnt) {
-                const int e = rn + lane;
-                j = rq.j[e];
-                const float4 a = make_float4(rq.v[0][e], rq.v[1][e], rq.v[2][e], rq.v[3][e]);
-                const float4 b = make_float4(rq.v[4][e], rq.v[5][e], rq.v[6][e], rq.v[7][e]);
-                const float4 cc = make_float4(rq.v[8][e], rq.v[9][e], rq.v[10][e], 0.0f);
+                float4 a, b, cc;
+                j = rq.get(rn + lane, a, b, cc);
                 event = photon_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl);
             }
             __syncwarp();
@@ -504,13 +490,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
         if (PW && sp == 2) {
             const bool rate = valid && photon_needs_rate<FIX ? FIX : QED_F_FULL>(C, WS.L, j, a, b, cc, chi_z, ctr, c);
             const unsigned m = __ballot_sync(0xffffffffu, rate);
-            if (rate) {
-                const int e = rn + __popc(m & ((1u << lane) - 1u));
-                rq.v[0][e] = a.x; rq.v[1][e] = a.y; rq.v[2][e] = a.z; rq.v[3][e] = a.w;
-                rq.v[4][e] = b.x; rq.v[5][e] = b.y; rq.v[6][e] = b.z; rq.v[7][e] = b.w;
-                rq.v[8][e] = cc.x; rq.v[9][e] = cc.y; rq.v[10][e] = cc.z;
-                rq.j[e] = j;
-            }
+            if (rate) rq.put(rn + __popc(m & ((1u << lane) - 1u)), j, a, b, cc);
             rn += __popc(m);
             __syncwarp();
         } else {

@@ -185,26 +185,54 @@ struct Shared32 {
 
 __host__ __device__ inline size_t align128(size_t b) { return (b + 127) & ~size_t(127); }
 
-__host__ __device__ inline size_t smem32_bytes(int n_chi) {
-    return align128((size_t)3 * kBesN * 4 + (size_t)4 * n_chi * 4) + (size_t)kWarps32 * kStages * sizeof(Tile) +
-           (size_t)kWarps32 * kStages * 8 + (size_t)kWarps32 * kWQ * 8;
+// Photons that may have a pair rate, queued per warp by the plane-wave kernels (photon_needs_rate): the state words of
+// the step (x, P_x; P_y, P_z, tau; k) and the index, a column per photon.
+constexpr int kRateQ = 64;  // drained 32 at a time
+template <class J>  // the index type
+struct RateQT {
+    float v[11][kRateQ];
+    J j[kRateQ];
+    __device__ __forceinline__ void put(int e, J index, const float4& a, const float4& b, const float4& cc) {
+        v[0][e] = a.x; v[1][e] = a.y; v[2][e] = a.z; v[3][e] = a.w;
+        v[4][e] = b.x; v[5][e] = b.y; v[6][e] = b.z; v[7][e] = b.w;
+        v[8][e] = cc.x; v[9][e] = cc.y; v[10][e] = cc.z;
+        j[e] = index;
+    }
+    __device__ __forceinline__ J get(int e, float4& a, float4& b, float4& cc) const {
+        a = make_float4(v[0][e], v[1][e], v[2][e], v[3][e]);
+        b = make_float4(v[4][e], v[5][e], v[6][e], v[7][e]);
+        cc = make_float4(v[8][e], v[9][e], v[10][e], 0.0f);
+        return j[e];
+    }
+};
+using RateQ = RateQT<int64_t>;
+
+// the single-buffer kernels' shared memory; bes: the Bessel table is staged too (the plane-wave kernels, which read it
+// at events only, leave it in global memory); rate_queue: a RateQ per warp at the end
+__host__ __device__ inline size_t smem32_bytes(int n_chi, bool bes, bool rate_queue) {
+    return align128((size_t)(bes ? 3 * kBesN * 4 : 0) + (size_t)4 * n_chi * 4) + (size_t)kWarps32 * kStages * sizeof(Tile) +
+           (size_t)kWarps32 * kStages * 8 + (size_t)kWarps32 * kWQ * 8 + (rate_queue ? kWarps32 * sizeof(RateQ) : 0);
 }
 
-__device__ __forceinline__ Shared32 carve32(unsigned char* smem, int n_chi) {
+__device__ __forceinline__ Shared32 carve32(unsigned char* smem, int n_chi, bool bes, RateQ** rq) {
     Shared32 s;
     s.bes = (float*)smem;
-    s.rates = s.bes + 3 * kBesN;
-    size_t off = align128((size_t)3 * kBesN * 4 + (size_t)4 * n_chi * 4);
+    s.rates = s.bes + (bes ? 3 * kBesN : 0);
+    size_t off = align128((size_t)(bes ? 3 * kBesN * 4 : 0) + (size_t)4 * n_chi * 4);
     s.tiles = (Tile*)(smem + off);
     off += (size_t)kWarps32 * kStages * sizeof(Tile);
     s.bars = (uint64_t*)(smem + off);
     off += (size_t)kWarps32 * kStages * 8;
     s.queue = (int64_t*)(smem + off);
+    off += (size_t)kWarps32 * kWQ * 8;
+    *rq = (RateQ*)(smem + off);
     return s;
 }
 
-__device__ __forceinline__ void load_tables32(const Shared32& sh, const float* __restrict__ bes_g, const TabP<float>& T) {
-    for (int i = threadIdx.x; i < 3 * kBesN; i += blockDim.x) sh.bes[i] = bes_g[i];
+__device__ __forceinline__ void load_tables32(const Shared32& sh, const float* __restrict__ bes_g, const TabP<float>& T,
+                                              bool bes) {
+    if (bes)
+        for (int i = threadIdx.x; i < 3 * kBesN; i += blockDim.x) sh.bes[i] = bes_g[i];
     for (int i = threadIdx.x; i < 2 * T.n_chi; i += blockDim.x) {
         sh.rates[i] = T.nlc_rate[i];
         sh.rates[2 * T.n_chi + i] = T.nbw_rate[i];
@@ -1112,8 +1140,12 @@ __device__ __forceinline__ bool photon_stream_one(const Ctx& C, const PartDev& G
 
 // Below this chi both pair rates are zero in FP32: J = exp(ln(J e^{8/(3 chi)}) - 8/(3 chi)) leaves the normal float
 // range (e^-88 is half its smallest number; results below it are flushed) whatever the table's entry, at most m, adds.
-__device__ __forceinline__ float no_rate_chi(const TabP<float>& T, float m) {
-    return fmaxf(T.chi_min, (float)(8.0 / 3.0) / (88.0f + fmaxf(m, 0.0f)));
+// (all lanes of a warp; nbw: the rate rows)
+__device__ __forceinline__ float no_rate_chi(const TabP<float>& T, const float* nbw) {
+    float m = 0.0f;
+    for (int i = threadIdx.x & 31; i < 2 * T.n_chi; i += 32) m = fmaxf(m, nbw[i]);
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    return fmaxf(T.chi_min, (float)(8.0 / 3.0) / (88.0f + m));
 }
 
 // The first part of a photon's step in a plane wave: most photons are too soft, or outside the pulse, for a pair rate
