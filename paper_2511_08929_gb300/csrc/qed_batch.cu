@@ -264,12 +264,15 @@ __device__ __forceinline__ void batch_issue(Tile* tile, const int* tile0, const 
     cp_async_commit();
 }
 
-// per-warp state of the current segment, in shared memory (written by lane 0 at a segment change)
+// per-warp state of the current segment, in shared memory (written at a segment change: the context and the buffer
+// copied by all lanes, 8 bytes each; copied and computed by one lane they took 1-2 us)
 struct WarpSeg {
-    Ctx C;      // tables, field, step parameters and charge of the segment's instance and species
+    Ctx C;      // field, step parameters and charge of the segment's instance and species (the plan's)
     PartDev L;  // the segment's buffer (planes, ids, count) for the streaming pass
     int t0, t1, n;  // its tile range and particle count
 };
+static_assert(sizeof(Ctx) % 8 == 0 && sizeof(PartDev) % 8 == 0 && alignof(Ctx) == 8 && alignof(PartDev) == 8,
+              "copied in words of 8 bytes");
 
 using BatchRateQ = RateQT<int>;  // (a batch's buffers hold at most INT32_MAX particles)
 
@@ -291,8 +294,8 @@ __host__ __device__ inline size_t batch_smem_bytes(int warps, int stages, int n_
 template <int WARPS, int STAGES, int MINB, uint32_t FIX>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
     batch_step_kernel(TabP<float> T, float* bes_g, const InstDev* __restrict__ inst,
-                      const SegDev* __restrict__ seg, const int64_t* __restrict__ tile0_g, int n_inst,
-                      const ClockDev* __restrict__ clk, BatchP P, int chunk, int* work, long long* ev,
+                      const SegDev* __restrict__ seg, const SegCtx* __restrict__ ctx,
+                      const int64_t* __restrict__ tile0_g, int n_inst, int chunk, int* work, long long* ev,
                       long long ev_cap, unsigned long long* n_ev, qed_counters* ctr) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int n_seg = kSpecies * n_inst;
@@ -333,7 +336,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     Tl.nlc_rate = sh.rates;
     Tl.nbw_rate = sh.rates + 2 * T.n_chi;
     const int W2 = 2 * gridDim.x * WARPS;
-    unsigned long long c[C_N] = {};
+    unsigned c[C_N] = {};
     int2* ring = s_chunks + warp * kChunkRing;
     // the copy walk (warp-uniform): tile pt of a chunk ending at pe, the chunks put in the ring (pk), the
     // prefetched take (ns, nsz; lane 0 adds, the warp shares the result)
@@ -429,35 +432,17 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
             sp = cur / n_inst;
             ii = cur - sp * n_inst;
             __syncwarp();
+            const SegCtx& X = ctx[cur];
+            const uint64_t* src = reinterpret_cast<const uint64_t*>(&X.C);
+            uint64_t* dst = reinterpret_cast<uint64_t*>(&C);
+            for (int k = lane; k < (int)(sizeof(Ctx) / 8); k += 32) dst[k] = src[k];
+            src = reinterpret_cast<const uint64_t*>(&inst[ii].sp[sp]);
+            dst = reinterpret_cast<uint64_t*>(&WS.L);
+            for (int k = lane; k < (int)(sizeof(PartDev) / 8); k += 32) dst[k] = src[k];
             if (lane == 0) {
-                const InstDev& I = inst[ii];
-                const uint64_t step = clk->step;
-                // time of this step: a product then a sum, each rounded (no contraction)
-                const double t_now = __dadd_rn(clk->t0, __dmul_rn((double)(step - clk->step0), clk->dt));
                 WS.t0 = s_tile0[cur];
                 WS.t1 = s_tile0[cur + 1];
                 WS.n = (int)seg[cur].n;
-                WS.L = I.sp[sp];
-                C.T = T;
-                C.T.nlc_rate = sh.rates;
-                C.T.nbw_rate = sh.rates + 2 * T.n_chi;
-                C.bes = sh.bes;
-                C.F = I.F;
-                C.q = sp == 0 ? -1.0f : (sp == 1 ? 1.0f : 0.0f);
-                StepP S;
-                S.dt = clk->dt;
-                S.ph_hi = __dadd_rn(t_now, I.phase);
-                S.ph_hi_f = (float)S.ph_hi;
-                S.ph_lo_f = (float)(S.ph_hi - (double)S.ph_hi_f);
-                S.dt_f = P.dt_f;
-                S.flags = P.flags;
-                S.step = step;
-                S.seed = I.seed;
-                S.store_min = P.store_min;
-                S.chi_floor = P.chi_floor;
-                S.store_min_f = (float)P.store_min;
-                S.chi_floor_f = (float)P.chi_floor;
-                C.S = S;
             }
             __syncwarp();
         }
@@ -541,7 +526,7 @@ __global__ void __launch_bounds__(kEventThreads, 2) batch_event_kernel(const Ins
                                                                    const float* __restrict__ lnup = nullptr) {
     const unsigned long long n = clk->n_list[0];
     const ExactList q = exact_list(ev, ev_cap, clk);
-    unsigned long long c[C_N] = {};
+    unsigned c[C_N] = {};
     const int lane = threadIdx.x & 31;
     const unsigned long long warps = (unsigned long long)gridDim.x * (kEventThreads / 32);
     for (unsigned long long k = first_chunk() * 32; k < n; k += warps * 32) {
@@ -564,7 +549,7 @@ __global__ void __launch_bounds__(kEvent64Threads) batch_event64_kernel(const In
     const unsigned long long n = clk->n_list[1], nc = (n + 31) / 32;
     const ExactList q = exact_list(ev, ev_cap, clk);
     const unsigned long long nx = min(*q.n, q.cap), xc = (nx + 31) / 32;
-    unsigned long long c[C_N] = {};
+    unsigned c[C_N] = {};
     const int lane = threadIdx.x & 31;
     const unsigned long long warps = (unsigned long long)gridDim.x * (kEvent64Threads / 32);
     for (unsigned long long k = first_chunk(); k < nc + xc; k += warps) {
@@ -765,13 +750,8 @@ template <int WARPS, int STAGES, int MINB, uint32_t FIX>
 static void launch_variant(const qed_batch_s* b, int grid, cudaStream_t st) {
     const qed_tables_s* t = b->tables;
     const size_t smem = batch_smem_bytes(WARPS, STAGES, t->desc.n_chi, kSpecies * b->n_inst, plane_waves_only<FIX>());
-    BatchP P;
-    P.flags = b->desc.flags;
-    P.dt_f = (float)b->desc.dt;
-    P.store_min = b->desc.photon_store_min;
-    P.chi_floor = b->desc.chi_floor;
     batch_step_kernel<WARPS, STAGES, MINB, FIX><<<grid, WARPS * 32, smem, st>>>(
-        tab_params<float>(t), t->bes32, b->d_inst, b->d_seg, b->d_tile0, b->n_inst, b->d_clk, P, b->tuning.chunk,
+        tab_params<float>(t), t->bes32, b->d_inst, b->d_seg, b->d_ctx, b->d_tile0, b->n_inst, b->tuning.chunk,
         &b->d_clk->next_tile, b->d_ev, b->capacity_total, b->d_clk->n_list, b->ctr);
 }
 

@@ -241,12 +241,14 @@ __device__ __forceinline__ void load_tables32(const Shared32& sh, const float* _
 
 enum { C_EVENTS, C_STORED, C_DROPPED, C_CLAMPED, C_RENORM, C_BELOW, C_NONFINITE, C_RATE_STEPS, C_BOUND, C_N };
 
-// per-warp counter flush (no block barrier: warps finish at different times)
-__device__ __forceinline__ void flush_warp(unsigned long long (&c)[C_N], qed_counters* ctr) {
+// per-warp counter flush (no block barrier: warps finish at different times).  A lane's counts fit 32 bits (a buffer's
+// particles over the lanes of at least one warp); the lanes' halves are summed by two warp reductions.
+__device__ __forceinline__ void flush_warp(unsigned (&c)[C_N], qed_counters* ctr) {
 #pragma unroll
     for (int i = 0; i < C_N; ++i) {
-        const unsigned long long v = warp_sum(c[i]);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&ctr->events + i, v);
+        if (!__any_sync(0xffffffffu, c[i] != 0)) continue;
+        const unsigned lo = __reduce_add_sync(0xffffffffu, c[i] & 0xFFFFu), hi = __reduce_add_sync(0xffffffffu, c[i] >> 16);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&ctr->events + i, ((unsigned long long)hi << 16) + lo);
     }
 }
 
@@ -465,7 +467,7 @@ struct LState {
 // ACC: fields from the accurate sine and cosine (the event passes), else the fast ones
 template <uint32_t FIX = 0, bool ACC = false>
 __device__ __forceinline__ void lepton_classical(const Ctx& C, const float4& a, const float4& b, const float4& cc, LState& st,
-                                                 unsigned long long* c,
+                                                 unsigned* c,
                                                  const TabP<float>* Tp = nullptr) {
     const TabP<float>& T = Tp ? *Tp : C.T;  // the caller may hand the tables over from its parameters
     const uint32_t fl = flags_of<FIX>(C);
@@ -600,7 +602,7 @@ __device__ __forceinline__ float nlc_stokes_scale(float lam, float one_m, const 
 // the density is below the float range.  A step whose acceptance exceeds 1 is counted (the method needs
 // it below 1).
 __device__ __forceinline__ bool reject_nlc(const Ctx& C, const uint4& w0, float chi, float gam, float sb,
-                                           unsigned long long* c) {
+                                           unsigned* c) {
     const float r1 = u52f(w0.x, w0.y), r2 = u52f(w0.z, w0.w);
     const float lc = r1 * r1 * r1, om = 1.0f - lc;
     const float up = div_(2.0f * lc, 3.0f * chi * om);
@@ -614,7 +616,7 @@ __device__ __forceinline__ bool reject_nlc(const Ctx& C, const uint4& w0, float 
 }
 
 __device__ __forceinline__ bool reject_nbw(const Ctx& C, const uint4& w0, float chi, float en, float xi3,
-                                           unsigned long long* c) {
+                                           unsigned* c) {
     const float r1 = u52f(w0.x, w0.y), r2 = u52f(w0.z, w0.w);
     const float om = 1.0f - r1;
     const float ut = div_(2.0f, 3.0f * chi * r1 * om);
@@ -707,7 +709,7 @@ static __device__ __noinline__ void lepton_exact_one(const Ctx& C, const Tab64& 
 // the branch's ICDF row.
 static __device__ QED_EVENT_PASS void lepton_events(const Ctx& C, const Tab64& X, const FieldP<double>& F64, int64_t j,
                                                  const PartDev& L, const PartDev& G, AppendState* A,
-                                                 qed_counters* ctr, unsigned long long* c, const ExactList* q = nullptr,
+                                                 qed_counters* ctr, unsigned* c, const ExactList* q = nullptr,
                                                  long long word = 0, bool net = false, float lnu = 0.0f) {
     // The lepton's outcome (energy fraction, recoil, spin) and the photon's polarization for every event,
     // then the photon's slot reservation: an event whose photon does not fit is not applied.
@@ -722,8 +724,8 @@ static __device__ QED_EVENT_PASS void lepton_events(const Ctx& C, const Tab64& X
     bool down = false;
     if (j >= 0) {
         const float4 a = __ldcg(L.q0 + j), b = __ldcg(L.q1 + j), cc = __ldcg(L.q2 + j);
-        lepton_classical<0, true>(C, a, b, cc, st, nullptr);  // the streaming pass's step, accurate fields
         id = L.id[j];
+        lepton_classical<0, true>(C, a, b, cc, st, nullptr);  // the streaming pass's step, accurate fields
         pf = st.p;
         sf = st.s;
         // the optical depth as the streaming pass left it (spent), kept if the event is not applied
@@ -871,7 +873,7 @@ static __device__ QED_EVENT_PASS void lepton_events(const Ctx& C, const Tab64& X
 // particle's optical depth ran out (it is then left untouched for the event pass)
 template <uint32_t FIX = 0>
 __device__ __forceinline__ bool lepton_stream_one(const Ctx& C, const PartDev& L, int64_t j, const float4& a, const float4& b,
-                                                  const float4& cc, qed_counters* ctr, unsigned long long* c, const TabP<float>* Tp = nullptr) {
+                                                  const float4& cc, qed_counters* ctr, unsigned* c, const TabP<float>* Tp = nullptr) {
     const uint32_t fl = flags_of<FIX>(C);
     const float dt = C.S.dt_f;
     if (!finite_state(a, b, cc)) {
@@ -947,7 +949,7 @@ __device__ __forceinline__ float photon_direction(const F3& k, float& en, F3& kh
 
 template <uint32_t FIX = 0, bool ACC = false>
 __device__ __forceinline__ void photon_classical(const Ctx& C, const float4& a, const float4& b, const float4& cc, PState& st,
-                                                 unsigned long long* c,
+                                                 unsigned* c,
                                                  const TabP<float>* Tp = nullptr) {
     const TabP<float>& T = Tp ? *Tp : C.T;  // the caller may hand the tables over from its parameters
     const F3 xold{a.x, a.y, a.z};
@@ -986,7 +988,7 @@ __device__ __forceinline__ void photon_classical(const Ctx& C, const float4& a, 
 // decision is FP64 (pairs are rare; their spin coefficients cancel).
 static __device__ QED_EVENT_PASS void photon_events(const Ctx& C, const Tab64& X, int64_t j, const PartDev& G,
                                                  const PartDev& El, const PartDev& Po, AppendState* A,
-                                                 qed_counters* ctr, unsigned long long* c) {
+                                                 qed_counters* ctr, unsigned* c) {
     const uint32_t fl = C.S.flags;
     const bool have = A != nullptr;
     bool want = false;
@@ -996,6 +998,7 @@ static __device__ QED_EVENT_PASS void photon_events(const Ctx& C, const Tab64& X
     uint64_t ide = 0, idp = 0;
     if (j >= 0) {
         const float4 a = __ldcg(G.q0 + j), b = __ldcg(G.q1 + j), cc = __ldcg(G.q2 + j);
+        const uint64_t id = G.id[j];
         PState st;
         photon_classical<0, true>(C, a, b, cc, st, nullptr);
         x = st.x;
@@ -1005,7 +1008,6 @@ static __device__ QED_EVENT_PASS void photon_events(const Ctx& C, const Tab64& X
         tauf = tau_join(b.z, b.w);
         const bool rej = (fl & QED_F_REJECT) != 0;
         if ((fl & QED_F_TAU) && !rej) tauf -= widen_pos(st.Wx * C.S.dt_f);
-        const uint64_t id = G.id[j];
         const uint4 w0 = draw(id, C.S.seed, C.S.step, kSlotTauBranch);
         bool minus;
         if (fl & QED_F_TAU) minus = u52f(w0.z, w0.w) * st.Wx < st.Wmp;
@@ -1085,7 +1087,7 @@ static __device__ QED_EVENT_PASS void photon_events(const Ctx& C, const Tab64& X
 
 template <uint32_t FIX = 0>
 __device__ __forceinline__ bool photon_stream_one(const Ctx& C, const PartDev& G, int64_t j, const float4& a, const float4& b,
-                                                  const float4& cc, qed_counters* ctr, unsigned long long* c, const TabP<float>* Tp = nullptr) {
+                                                  const float4& cc, qed_counters* ctr, unsigned* c, const TabP<float>* Tp = nullptr) {
     const uint32_t fl = flags_of<FIX>(C);
     const float dt = C.S.dt_f;
     if (!finite_photon(a, b, cc)) {
@@ -1155,7 +1157,7 @@ __device__ __forceinline__ float no_rate_chi(const TabP<float>& T, const float* 
 // written).
 template <uint32_t FIX>
 __device__ __forceinline__ bool photon_needs_rate(const Ctx& C, const PartDev& G, int64_t j, const float4& a, const float4& b,
-                                                  const float4& cc, float chi_z, qed_counters* ctr, unsigned long long* c) {
+                                                  const float4& cc, float chi_z, qed_counters* ctr, unsigned* c) {
     static_assert(plane_waves_only<FIX>(), "the bound is that of a single plane wave");
     if (!finite_photon(a, b, cc)) {
         c[C_NONFINITE]++;
