@@ -321,13 +321,14 @@ qed_status qed_compact_noalloc(qed_particles *photons, void *stream);
 
 /* ---- Batched collisions: many independent instances stepped together ----
  * A batch is a set of independent collision instances (each its own laser, seed and three FP32 species
- * buffers) advanced in lockstep.  One time step of the whole batch is: a planning kernel (alive counts
- * at step start, the tile list over all instances and species, each one's step context), one
- * persistent kernel that streams every tile of 32 particles of every instance (the lepton step of
- * Sec. 5.1 for electrons and positrons, the photon step of Sec. 5.2 for photons, each as qed_push_step /
- * qed_pair_step do) and lists the particles whose optical depth ran out, an event kernel that runs the
- * emission / pair branch for the listed particles, and the photon compaction of every instance.  The step index and time live in device memory and advance on the
- * device, so a captured CUDA graph of one or more steps is replayed unchanged.  Results are the ones
+ * buffers) advanced in lockstep.  One time step of the whole batch is: one persistent kernel that streams
+ * every tile of 32 particles of every instance (the lepton step of Sec. 5.1 for electrons and positrons,
+ * the photon step of Sec. 5.2 for photons, each as qed_push_step / qed_pair_step do) and lists the
+ * particles whose optical depth ran out, two event kernels that run the emission / pair branch for the
+ * listed particles (FP32, and what is FP64), and one that ends the step: the photon compaction of every
+ * instance and the plan of the next step (alive counts at its start, the tile list over all instances and
+ * species, each one's step context; a plan kernel makes the first of a call).  The step index and time live in
+ * device memory and advance on the device, so a captured CUDA graph of one or more steps is replayed unchanged.  Results are the ones
  * qed_push_step, qed_pair_step and qed_compact give per instance with begin snapshots (the same
  * arithmetic and random draws; appended daughters may sit in another order), whatever the tuning. */
 #define QED_BATCH_MAX_INSTANCES 1024

@@ -765,19 +765,22 @@ static void launch_variant(const qed_batch_s* b, int grid, cudaStream_t st) {
 // [0]: flags read at run time; [1]: built for QED_F_FULL (every flag test of the streaming pass folded)
 static const BatchVariant kVariants[2][QED_BATCH_VARIANTS] = {QED_VARIANTS(0u), QED_VARIANTS(QED_F_FULL)};
 
-static bool fixed_kernel(const qed_batch_s* b) { return b->desc.flags == QED_F_FULL && b->plane_waves; }
-
-static const BatchVariant& variant_of(const qed_batch_s* b, int v) { return kVariants[fixed_kernel(b) ? 1 : 0][v]; }
-
-static size_t variant_smem(const qed_batch_s* b, int v) {
-    return batch_smem_bytes(variant_of(b, v).warps, variant_of(b, v).stages, b->tables->desc.n_chi, kSpecies * b->n_inst,
-                            fixed_kernel(b));
+static size_t variant_smem(const qed_batch_s* b, int v, bool fixed) {
+    return batch_smem_bytes(kVariants[fixed][v].warps, kVariants[fixed][v].stages, b->tables->desc.n_chi,
+                            kSpecies * b->n_inst, fixed);
 }
+
+// the kernel built for the full flag set, where the batch is plane waves and its rate queues fit beside the tables
+static bool fixed_kernel(const qed_batch_s* b, int v) {
+    return b->desc.flags == QED_F_FULL && b->plane_waves && variant_smem(b, v, true) <= kMaxBlockSmem;
+}
+
+static const BatchVariant& variant_of(const qed_batch_s* b, int v) { return kVariants[fixed_kernel(b, v) ? 1 : 0][v]; }
 
 // resident blocks per SM of variant v for this batch (0 if it does not fit)
 static int variant_occupancy(const qed_batch_s* b, int v) {
     int per_sm = 0;
-    const size_t smem = variant_smem(b, v);
+    const size_t smem = variant_smem(b, v, fixed_kernel(b, v));
     const BatchVariant& k = variant_of(b, v);
     if (cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.kern, k.warps * 32, smem) != cudaSuccess) return 0;

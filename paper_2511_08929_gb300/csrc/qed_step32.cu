@@ -183,14 +183,14 @@ static int blocks32(int64_t capacity, const void* kern, size_t smem) {
 // The full flag set in a single plane wave takes the kernels built for it (the batched kernels' arithmetic, bit for
 // bit).  With the kernels that read the flags, 64 steps of 1e4 electrons took 3.06 ms, 48 steps of 1e6 electrons with
 // 1e7 photons 31.9 ms; with these 2.94 and 30.5.
-static bool fixed_flags32(const qed_field& f, const qed_step_desc& s) {
-    return s.flags == QED_F_FULL && (f.kind == QED_FIELD_LP || f.kind == QED_FIELD_CP);
+static bool fixed_flags32(const qed_field& f, const qed_step_desc& s, size_t smem) {
+    return s.flags == QED_F_FULL && (f.kind == QED_FIELD_LP || f.kind == QED_FIELD_CP) && smem <= qed::kMaxBlockSmem;
 }
 
 void launch_lepton32(const qed_tables_s* t, const qed_field& f, const qed_step_desc& s, const qed_particles* L,
                      const qed_particles* G, qed_counters* ctr, cudaStream_t st) {
     using namespace qed;
-    const bool fixed = fixed_flags32(f, s);
+    const bool fixed = fixed_flags32(f, s, smem32_bytes(t->desc.n_chi, false, false));
     const size_t smem = smem32_bytes(t->desc.n_chi, !fixed, false);
     PartDev g{};
     if (G) g = part_dev(G);
@@ -203,7 +203,7 @@ void launch_lepton32(const qed_tables_s* t, const qed_field& f, const qed_step_d
 void launch_photon32(const qed_tables_s* t, const qed_field& f, const qed_step_desc& s, const qed_particles* G,
                      const qed_particles* El, const qed_particles* Po, qed_counters* ctr, cudaStream_t st) {
     using namespace qed;
-    const bool fixed = fixed_flags32(f, s);
+    const bool fixed = fixed_flags32(f, s, smem32_bytes(t->desc.n_chi, false, true));
     const size_t smem = smem32_bytes(t->desc.n_chi, !fixed, fixed);
     PartDev e{}, p{};
     if (El && Po) {

@@ -207,6 +207,10 @@ struct RateQT {
 };
 using RateQ = RateQT<int64_t>;
 
+// dynamic shared memory a block can have; the plane-wave kernels, whose rate queues come on top of the rate tables, run
+// only where their tables leave room (n_chi up to ~9000), else the kernels that read the flags do
+constexpr size_t kMaxBlockSmem = 227 * 1024;
+
 // the single-buffer kernels' shared memory; bes: the Bessel table is staged too (the plane-wave kernels, which read it
 // at events only, leave it in global memory); rate_queue: a RateQ per warp at the end
 __host__ __device__ inline size_t smem32_bytes(int n_chi, bool bes, bool rate_queue) {
