@@ -606,7 +606,7 @@ def native_batch(args):
     if tr is not None:  # ncu DRAM bytes per particle-step of a smaller capture, scaled to this launch
         traffic = tr["dram_bytes_per_particle_step"] * psteps / K
     # the timed span of a step: the persistent streaming kernel and the event kernel that follows it
-    roof = {"kernel": "batch_step_kernel+batch_event_kernel", "bound": "hbm", "achieved": None, "peak": peak, "unit": "GB/s",
+    roof = {"kernel": "batch_step_kernel+batch_event_kernel+batch_event64_kernel", "bound": "hbm", "achieved": None, "peak": peak, "unit": "GB/s",
             "frac": None, "traffic": traffic, "peak_source": peak_kind,
             "algorithmic_bytes_per_launch": alg / K, "design_bytes_per_launch": alg_design / K}
     if tr is not None:
@@ -646,7 +646,7 @@ def native_batch(args):
                    "l2": "state > L2 (no flush needed)", "tables": "256 chi x 256 r, FP64-built"},
         "roofline": roof,
         "clocks": clocks,
-        "gpu_launches": 7 * K,  # plan, persistent kernel, event kernel, four compaction kernels per step
+        "gpu_launches": 4 * K + 1,  # persistent kernel, two event kernels, step end; one plan kernel per call
         "particles_at_start": {"electrons": int(s0.alive[0]), "positrons": int(s0.alive[1]),
                                "photons": int(s0.alive[2])},
         "particle_steps_timed": {"electrons": d_sp[0], "positrons": d_sp[1], "photons": d_sp[2]},
@@ -778,7 +778,7 @@ def native_cascade(args):
     alg = unit_bytes(d_sp[0] + d_sp[1], d_sp[2], tot["stored"])
     alg_design = design_bytes(d_sp[0] + d_sp[1], d_sp[2], tot["rate_steps"], tot["events"], tot["stored"])
     full = steps // SEG * SEG  # steps whose kernels were event-timed (whole graph launches)
-    roof = {"kernel": "batch_step_kernel+batch_event_kernel", "bound": "hbm", "peak": peak, "unit": "GB/s",
+    roof = {"kernel": "batch_step_kernel+batch_event_kernel+batch_event64_kernel", "bound": "hbm", "peak": peak, "unit": "GB/s",
             "peak_source": peak_kind, "traffic": None,
             "algorithmic_bytes_per_launch": alg / steps, "design_bytes_per_launch": alg_design / steps}
     if tk > 0:
@@ -800,7 +800,7 @@ def native_cascade(args):
                    "load_s": round(t_load, 1), "tables": "256 chi x 256 r, FP64-built"},
         "roofline": roof,
         "clocks": summarize_clocks(clock_lines),
-        "gpu_launches": 7 * steps,
+        "gpu_launches": 4 * steps + -(-steps // SEG),
         "growth": growth,
         "particle_steps_timed": {"electrons": d_sp[0], "positrons": d_sp[1], "photons": d_sp[2]},
         "counters": tot,
@@ -902,7 +902,7 @@ def native_helicity(args):
                       "electrons": [x["n"] for x in insts], "sizing": sizing,
                       "timed": f"all {steps} steps of the crossing, graph launches of {SEG} steps",
                       "launch": {"variant": v, "blocks_per_sm": bps, "chunk": ch}},
-           "clocks": summarize_clocks(clock_lines), "gpu_launches": 7 * steps,
+           "clocks": summarize_clocks(clock_lines), "gpu_launches": 4 * steps + 1,
            "counters": {k: int(x) for k, x in c.as_dict().items()},
            "particles_at_end": {"electrons": [int(bt.buffers()[k][0].count()) for k in range(2)],
                                 "positrons": [int(bt.buffers()[k][1].count()) for k in range(2)],
@@ -1039,7 +1039,7 @@ def mlp_leg(args, tables, torch, bt=None, stream=0):
             "eval_events": total, "samples_per_s": net_rate, "fallback_fraction": n_fb / total,
             "network_cdf_error_hist": {k: float(v / total) for k, v in zip(labels, hist)},
             "table_path_samples_per_s": tab_rate, "table_path_events": n_tab,
-            "table_path": "the checked sampler's own fallback: the exact mixture quantile, regula falsi on the tables' mixture CDF",
+            "table_path": "the checked sampler's own fallback: the exact mixture quantile of the tables",
             "gain_over_table_path": net_rate / tab_rate,
             "branch_table_samples_per_s": br_rate,
             "branch_table": "the step's sampler: spin branch by W_down(1-s)/(2W_s), one float-float ICDF row",

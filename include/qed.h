@@ -385,7 +385,7 @@ qed_status qed_batch_get_tuning(qed_batch_t b, qed_batch_tuning *out);
  * instantiation can be kept out of a timed region. */
 qed_status qed_batch_step(qed_batch_t b, int32_t n_steps, void *stream);
 /* Kernel timing: events[2k], events[2k+1] (cudaEvent_t, created by the caller with timing enabled) are
- * recorded before the persistent kernel and after the event kernel of the k-th step (k modulo n_pairs)
+ * recorded before the persistent kernel and after the event kernels of the k-th step (k modulo n_pairs)
  * of every CUDA graph captured from now on (step k of the graph) and of directly launched steps (counted
  * from this call).  n_pairs = 0 switches it off.  Discards any captured graph. */
 qed_status qed_batch_set_kernel_events(qed_batch_t b, void *const *events, int32_t n_pairs);
@@ -418,7 +418,8 @@ void qed_batch_destroy(qed_batch_t b);
 typedef struct qed_mlp_s *qed_mlp_t;
 
 /* A network with the given initial parameters (host array of QED_MLP_PARAMS floats) and device scratch
- * for training batches of up to max_batch samples.  Errors: QED_ERR_ARG, QED_ERR_NOMEM, QED_ERR_CUDA. */
+ * for training batches of up to max_batch samples (28 B each, of 65536 samples at least: qed_mlp_train generates
+ * several batches' samples at a time).  Errors: QED_ERR_ARG, QED_ERR_NOMEM, QED_ERR_CUDA. */
 qed_status qed_mlp_create(int64_t max_batch, const float *init_params, qed_mlp_t *out);
 void qed_mlp_destroy(qed_mlp_t m);
 /* Copy the parameters to / from host memory (setting resets the optimiser state).  Synchronous. */
@@ -467,7 +468,7 @@ qed_status qed_mlp_sample(qed_mlp_t m, qed_tables_t t, const double *chi, const 
  * (0, 1), or the batch's flags hold QED_F_REJECT), QED_ERR_NOMEM. */
 qed_status qed_batch_set_mlp(qed_batch_t b, qed_mlp_t m, double tol);
 /* For tests of the sampler on the event path: the last step's gathered inputs and samples, the first
- * n_max events (host arrays of n_max doubles each for chi, r, s_beta, n_max x 4 floats for out4, n_max
+ * n_max events, the lepton events before the pair events (host arrays of n_max doubles each for chi, r, s_beta, n_max x 4 floats for out4, n_max
  * bytes for is_lepton; any may be NULL); *n_out = the number of events of that step; pair events carry
  * placeholder inputs (chi 1, r 1/2, s_beta 0) and is_lepton 0; *n_fallback_total = the samples (pair
  * placeholders included) that took the tables since the network was last set.  Synchronous. */
