@@ -122,7 +122,8 @@ def summarize_clocks(lines):
     return {"sm_mhz": float(np.median(sm)), "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
 
 
-KERNEL_SOURCES = ("qed_batch.cu", "qed_step32.cuh", "qed_device.cuh", "qed_bessel.cuh", "qed_steps.h", "qed_internal.h")
+KERNEL_SOURCES = ("qed_batch.cu", "qed_step32.cuh", "qed_device.cuh", "qed_bessel.cuh", "qed_fp64.cuh", "qed_steps.h",
+                  "qed_internal.h")
 
 
 def kernel_source_hash() -> str:
