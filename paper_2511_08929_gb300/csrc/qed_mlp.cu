@@ -342,20 +342,21 @@ __device__ __noinline__ double mix_error64(const TabP<double>& T, const MixPoint
 }
 
 // the mixture quantile: Newton on the float tables from the blend of the branch quantiles, then on the FP64 tables;
-// the bracketing solver where that does not converge below the grid's upper end
-__device__ __noinline__ double mix_quantile_fast(const TabP<double>& T, const TabP<float>& T32, const MixPoint& m, double r) {
+// false where that does not converge below the grid's upper end (there the bracketing solver, mix_quantile, finds it)
+__device__ __noinline__ bool mix_quantile_fast(const TabP<double>& T, const TabP<float>& T32, const MixPoint& m, double r,
+                                               double& L) {
     int i;
     double f;
     chi_coord(T, m.lnchi, i, f);
-    double L = mix_baseline(T, m), yu = m.y, yd = m.y;
+    L = mix_baseline(T, m);
+    double yu = m.y, yd = m.y;
     float L32 = (float)L, yu32 = (float)m.y, yd32 = (float)m.y;
     if (mix_newton<float>(T32, i, (float)f, (float)m.a, (float)r, 12, 1e-3f, L32, yu32, yd32)) {
         L = L32;
         yu = yu32;
         yd = yd32;
     }
-    if (mix_newton<double>(T, i, f, m.a, r, 8, 1e-7, L, yu, yd)) return L;
-    return mix_quantile<44, 32>(T, m, r);
+    return mix_newton<double>(T, i, f, m.a, r, 8, 1e-7, L, yu, yd);
 }
 
 // xi3 = F3 / F0 at u' = e^L from the Bessel polynomials (see xi3_at)
@@ -964,17 +965,24 @@ __global__ void __launch_bounds__(kTR) mlp_forward_kernel(const float* __restric
 // no Stokes outputs, so neither their check nor xi3 on the table path
 constexpr int kLnUpOnly = 4;
 
-// the table path for sample i (the exact mixture quantile, and xi3 there unless ln_up_only)
-__device__ __noinline__ void table_path(const TabP<double>& T, const TabP<float>& T32, const double* __restrict__ besp,
+// the table path for sample i (the exact mixture quantile, and xi3 there unless ln_up_only): by Newton, or with
+// bracket by the bracketing solver; false: Newton does not reach it, nothing is written
+__device__ __noinline__ bool table_path(const TabP<double>& T, const TabP<float>& T32, const double* __restrict__ besp,
                                         const double* __restrict__ chi_in, const double* __restrict__ r_in,
-                                        const double* __restrict__ s_in, int64_t i, float* __restrict__ out4, bool ln_up_only) {
+                                        const double* __restrict__ s_in, int64_t i, float* __restrict__ out4, bool ln_up_only,
+                                        bool bracket) {
     const double chi = chi_in[i], r = r_in[i], s = s_in[i];
     const MixPoint m = mix_point(T, chi, r, s);
-    const double L = mix_quantile_fast(T, T32, m, r);
+    double L;
+    if (bracket)
+        L = mix_quantile<44, 32>(T, m, r);
+    else if (!mix_quantile_fast(T, T32, m, r, L))
+        return false;
     out4[4 * i] = (float)L;
     out4[4 * i + 1] = 0.0f;
     out4[4 * i + 2] = 0.0f;
     out4[4 * i + 3] = ln_up_only ? 0.0f : (float)xi3_poly(besp, chi, L, s);
+    return true;
 }
 
 // The check of a network sample, first on the float tables: the FP32 CDF and xi3 errors are within ~1e-6
@@ -1019,7 +1027,10 @@ __global__ void __launch_bounds__(kTR, kTcPerSm) mlp_net_kernel(const float* __r
 // The check: samples that pass on the float tables are done; the others wait in a block-wide queue, and a full block
 // of them at a time goes through FP64 (the check again for those within kMargin32 of the bound, the table path for
 // those that fail it, and for all of them with flags bit 0).  One block of 1024 threads per SM: the queue's last,
-// partly filled pass then runs in a few warps of every SM.
+// partly filled pass then runs in a few warps of every SM.  Samples that need the bracketing solver (a logit above the
+// grid: uniforms within 2e-9 of 1) wait in a second queue: it takes ~20 times Newton's instructions, and run in the
+// lane that met it, it held that lane's whole warp (4e5 table samples, 1 in 24 of them such: 22.7 ms, with the queue
+// 14.8).
 constexpr int kCheckThreads = 1024;
 
 struct CheckItem {
@@ -1038,13 +1049,14 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
                                                                      unsigned long long* n_fallback,
                                                                      const unsigned long long* __restrict__ n_dev) {
     extern __shared__ __align__(16) unsigned char check_smem[];
-    CheckItem* queue = reinterpret_cast<CheckItem*>(check_smem);  // [2 kCheckThreads]
-    __shared__ int queued;
+    CheckItem* queue = reinterpret_cast<CheckItem*>(check_smem);             // [2 kCheckThreads]
+    int64_t* slow = reinterpret_cast<int64_t*>(queue + 2 * kCheckThreads);  // [2 kCheckThreads]
+    __shared__ int queued, n_slow;
     if (n_dev) {
         const int64_t nd = (int64_t)*n_dev;
         if (nd < n) n = nd;
     }
-    if (threadIdx.x == 0) queued = 0;
+    if (threadIdx.x == 0) queued = n_slow = 0;
     __syncthreads();
     const bool table_only = (flags & 1) != 0, ln_up_only = (flags & kLnUpOnly) != 0;
     const float ftol = (float)tol;
@@ -1065,7 +1077,8 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
         }
         if (fell) fell[q.i] = fb ? 1 : 0;
         if (fb) {
-            table_path(T, T32, besp, chi_in, r_in, s_in, q.i, out4, ln_up_only);
+            if (!table_path(T, T32, besp, chi_in, r_in, s_in, q.i, out4, ln_up_only, false))
+                slow[atomicAdd(&n_slow, 1)] = q.i;  // at most 2 kCheckThreads - 1 entries
             ++nf;
         }
     };
@@ -1125,12 +1138,22 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
         if (qn >= kCheckThreads) {
             finish(queue[qn - kCheckThreads + threadIdx.x]);
             __syncthreads();
-            if (threadIdx.x == 0) queued = qn - kCheckThreads;
+            const int sn = n_slow;  // the same in every thread
+            if (sn >= kCheckThreads)
+                table_path(T, T32, besp, chi_in, r_in, s_in, slow[sn - kCheckThreads + threadIdx.x], out4, ln_up_only, true);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                queued = qn - kCheckThreads;
+                if (sn >= kCheckThreads) n_slow = sn - kCheckThreads;
+            }
             __syncthreads();
         }
     }
     __syncthreads();
     if ((int)threadIdx.x < queued) finish(queue[threadIdx.x]);
+    __syncthreads();
+    for (int k = threadIdx.x; k < n_slow; k += kCheckThreads)
+        table_path(T, T32, besp, chi_in, r_in, s_in, slow[k], out4, ln_up_only, true);
     nf = __reduce_add_sync(0xffffffffu, nf);
     if ((threadIdx.x & 31) == 0 && n_fallback && nf) atomicAdd(n_fallback, (unsigned long long)nf);
 }
@@ -1351,7 +1374,7 @@ static qed_status mlp_sample_launch(qed_mlp_t m, const qed_tables_s* t, const do
                                     int64_t n, const unsigned long long* n_dev, double tol, int flags, float* out4,
                                     uint8_t* fell_back, float* err_out, unsigned long long* n_fallback, int grid,
                                     cudaStream_t st) {
-    const size_t smem = 2 * kCheckThreads * sizeof(CheckItem);
+    const size_t smem = 2 * kCheckThreads * (sizeof(CheckItem) + sizeof(int64_t));
     if (cudaFuncSetAttribute(mlp_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return QED_ERR_CUDA;
     if (!(flags & QED_MLP_ALWAYS_TABLE))

@@ -218,3 +218,20 @@ def test_training_chunks_and_single_steps_agree(tables):
     assert np.abs(a.params() - b.params()).max() < 2e-4
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n", [1, 1024, 400003])
+def test_sampler_above_the_grid(tables, n):
+    """Uniforms within 2e-9 of 1 (a logit above the grid) take the bracketing solver, up to several blocks' queues full
+    of them: every one is what it is in a call of its own kind, and between the two branch quantiles' ends."""
+    chi, r, s = _query(n, 8)
+    top = torch.arange(n, device="cuda") % 3 == 0
+    r = torch.where(top, 1.0 - 1.9e-9 * (r * 0.999 + 0.0005), r).contiguous()
+    smp = GM.Sampler(GM.init_params(4))
+    out, fell, nf = smp.sample(tables, chi, r, s, table_only=True)
+    assert bool(torch.isfinite(out).all()) and bool(fell.all()) and int(nf) == n
+    alone, _, _ = smp.sample(tables, chi[top].contiguous(), r[top].contiguous(), s[top].contiguous(), table_only=True)
+    rest, _, _ = (smp.sample(tables, chi[~top].contiguous(), r[~top].contiguous(), s[~top].contiguous(), table_only=True)
+                  if n > 1 else (out[:0], None, None))
+    assert torch.equal(out[top], alone) and torch.equal(out[~top], rest)
+    smp.close()
