@@ -1061,6 +1061,7 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
     const bool table_only = (flags & 1) != 0, ln_up_only = (flags & kLnUpOnly) != 0;
     const float ftol = (float)tol;
     unsigned nf = 0;  // this thread's fallbacks
+    int held = 0;     // queued samples (the same in every thread)
     // a queued sample: the FP64 check decides, then the table path
     auto finish = [&](const CheckItem& q) {
         bool fb = true;
@@ -1084,6 +1085,7 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
     };
     for (int64_t base = (int64_t)blockIdx.x * kCheckThreads; base < n; base += (int64_t)gridDim.x * kCheckThreads) {
         const int64_t i = base + threadIdx.x;
+        bool waits = false;  // this thread's sample went to the queue
         if (i < n) {
             CheckItem q{i, 0.0f, 0.0f, __int_as_float(0x7FC00000), 0.0f};
             bool done = false;
@@ -1131,26 +1133,28 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
                 if (fell) fell[i] = 0;
             } else {
                 queue[atomicAdd(&queued, 1)] = q;  // at most 2 kCheckThreads - 1 entries
+                waits = true;
             }
         }
-        __syncthreads();
-        const int qn = queued;  // the same in every thread
-        if (qn >= kCheckThreads) {
-            finish(queue[qn - kCheckThreads + threadIdx.x]);
+        // The tile's entries are counted by the barrier itself: `queued`, read behind it, could already hold what a
+        // faster warp added for the next tile, and the warps would part at the barriers below.
+        held += __syncthreads_count(waits);
+        if (held >= kCheckThreads) {
+            held -= kCheckThreads;
+            finish(queue[held + threadIdx.x]);
             __syncthreads();
             const int sn = n_slow;  // the same in every thread
             if (sn >= kCheckThreads)
                 table_path(T, T32, besp, chi_in, r_in, s_in, slow[sn - kCheckThreads + threadIdx.x], out4, ln_up_only, true);
             __syncthreads();
             if (threadIdx.x == 0) {
-                queued = qn - kCheckThreads;
+                queued = held;
                 if (sn >= kCheckThreads) n_slow = sn - kCheckThreads;
             }
             __syncthreads();
         }
     }
-    __syncthreads();
-    if ((int)threadIdx.x < queued) finish(queue[threadIdx.x]);
+    if ((int)threadIdx.x < held) finish(queue[threadIdx.x]);  // (written before the loop's last barrier)
     __syncthreads();
     for (int k = threadIdx.x; k < n_slow; k += kCheckThreads)
         table_path(T, T32, besp, chi_in, r_in, s_in, slow[k], out4, ln_up_only, true);

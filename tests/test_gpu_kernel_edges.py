@@ -235,3 +235,20 @@ def test_sampler_above_the_grid(tables, n):
                   if n > 1 else (out[:0], None, None))
     assert torch.equal(out[top], alone) and torch.equal(out[~top], rest)
     smp.close()
+
+
+def test_sampler_over_many_tiles_a_block(tables):
+    """Ten tiles of 1024 samples per block of the check, about a third of whose samples wait in the block's queue, so
+    that it fills up between tiles at every offset: each sample is what it is in calls of one tile per block, in which
+    the queue never fills."""
+    n = 10 * 1024 * torch.cuda.get_device_properties(0).multi_processor_count + 77
+    chi, r, s = _query(n, 12)
+    smp = GM.Sampler(GM.init_params(4))
+    for tol in (3e-3, 2e-2):
+        out, fell, nf = smp.sample(tables, chi, r, s, tol=tol)
+        assert int(nf) == int(fell.sum()) and 0 < int(nf) < n
+        for a in range(0, n, 100000):
+            part = slice(a, min(n, a + 100000))
+            o1, f1, _ = smp.sample(tables, chi[part], r[part], s[part], tol=tol)
+            assert torch.equal(o1, out[part]) and torch.equal(f1, fell[part])
+    smp.close()
