@@ -1146,12 +1146,13 @@ __device__ __forceinline__ bool photon_stream_one(const Ctx& C, const PartDev& G
 
 // Below this chi both pair rates are zero in FP32: J = exp(ln(J e^{8/(3 chi)}) - 8/(3 chi)) leaves the normal float
 // range (e^-88 is half its smallest number; results below it are flushed) whatever the table's entry, at most m, adds.
-// (all lanes of a warp; nbw: the rate rows)
+// At most the table's end: a photon beyond it has to be counted, rate or no rate.  (all lanes of a warp; nbw: the rate
+// rows)
 __device__ __forceinline__ float no_rate_chi(const TabP<float>& T, const float* nbw) {
     float m = 0.0f;
     for (int i = threadIdx.x & 31; i < 2 * T.n_chi; i += 32) m = fmaxf(m, nbw[i]);
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    return fmaxf(T.chi_min, (float)(8.0 / 3.0) / (88.0f + m));
+    return fminf(T.chi_max, fmaxf(T.chi_min, (float)(8.0 / 3.0) / (88.0f + m)));
 }
 
 // The first part of a photon's step in a plane wave: most photons are too soft, or outside the pulse, for a pair rate

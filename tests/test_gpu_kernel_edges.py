@@ -252,3 +252,34 @@ def test_sampler_over_many_tiles_a_block(tables):
             o1, f1, _ = smp.sample(tables, chi[part], r[part], s[part], tol=tol)
             assert torch.equal(o1, out[part]) and torch.equal(f1, fell[part])
     smp.close()
+
+
+# ---- the chi_clamped count of photons that the pair-rate bound lets go ----------------------------------
+def _photon_batch(tables, b, kind, flags, steps=3):
+    n = len(b["id"])
+    bt = Q.Batch(tables, [Q.field(kind, a0=150.0, n_cycles=6.0, phase=2.0, eta0=ETA0)], [3], [(64, 64, n)], 0.2, t0=8.0,
+                 flags=flags)
+    g = bt.buffers()[0][2]
+    g.load(b["pos"], b["mom"], b["spin"], b["w"], b["id"])
+    g.init_tau(3)
+    bt.step(steps)
+    c, q = bt.ctr.read().as_dict(), g.q.cpu().numpy().view(np.uint32)
+    c.pop("first_bad")
+    bt.close()
+    return q, c
+
+
+@pytest.mark.parametrize("kind", [B.QED_FIELD_LP, B.QED_FIELD_CP])
+@pytest.mark.parametrize("chi_max", [0.004, 0.02, 0.1])
+def test_pair_rate_bound_counts_clamped_photons(kind, chi_max):
+    """Tables that end below the chi at which pair rates begin (0.03): a photon above their end is counted in
+    chi_clamped although it has no rate, in the kernels with the bound as in those without."""
+    t = Q.Tables(chi_min=1e-3, chi_max=chi_max, n_chi=24, n_r=64)
+    b = _photons(20011, 60)
+    q0, _, c0 = _pair_steps(t, b, kind, B.QED_F_FULL)
+    q1, _, c1 = _pair_steps(t, b, kind, B.QED_F_FULL | B.QED_F_TBMT_PAPER)
+    assert c1["chi_clamped"] > 0 and c0 == c1 and np.array_equal(q0, q1)
+    for flags in (B.QED_F_FULL, B.QED_F_FULL | B.QED_F_TBMT_PAPER):
+        q, c = _photon_batch(t, b, kind, flags)
+        assert c["chi_clamped"] == c1["chi_clamped"] and np.array_equal(q, q1)
+    t.close()
