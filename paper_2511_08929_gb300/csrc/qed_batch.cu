@@ -781,8 +781,10 @@ static const BatchVariant& variant_of(const qed_batch_s* b, int v) { return kVar
 static int variant_occupancy(const qed_batch_s* b, int v) {
     int per_sm = 0;
     const size_t smem = variant_smem(b, v, fixed_kernel(b, v));
+    if (smem > kMaxBlockSmem) return 0;
     const BatchVariant& k = variant_of(b, v);
-    if (cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    // the limit belongs to the kernel, which every live batch launches with a size of its own: always the device's
+    if (cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBlockSmem) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.kern, k.warps * 32, smem) != cudaSuccess) return 0;
     return per_sm;
 }

@@ -283,3 +283,46 @@ def test_pair_rate_bound_counts_clamped_photons(kind, chi_max):
         q, c = _photon_batch(t, b, kind, flags)
         assert c["chi_clamped"] == c1["chi_clamped"] and np.array_equal(q, q1)
     t.close()
+
+
+# ---- the shared-memory limits of kernels that several batches, tables and threads use --------------------
+@pytest.mark.parametrize("graph_steps", [0, 2])
+def test_live_batches_keep_their_shared_memory(tables, graph_steps):
+    """A batch that needs more shared memory than one made or tuned after it (more instances, a longer table) steps
+    as it does alone."""
+    long_t = Q.Tables(chi_min=1e-3, chi_max=1e2, n_chi=200, n_r=16)
+
+    def make(t, n_inst):
+        fields = [Q.field(B.QED_FIELD_CP, a0=150.0, n_cycles=4.0, phase=4 * math.pi, eta0=ETA0)] * n_inst
+        bt = Q.Batch(t, fields, list(range(n_inst)), [(200, 200, 2000)] * n_inst, 0.2, t0=1.0)
+        bt.set_tuning(graph_steps=graph_steps)
+        for k, (e, _, _) in enumerate(bt.buffers()):
+            bm = I.lepton_beam(50, 3000.0, z_range=(-3.0, 3.0), seed=k, id_offset=k << 40)
+            e.load(bm["pos"], bm["mom"], bm["spin"], bm["w"], bm["id"])
+            e.init_tau(k)
+        return bt
+
+    def result(bt):
+        out = [{k: v[np.argsort(r["id"])] for k, v in r.items()} for trio in bt.buffers() for r in (b.read() for b in trio)]
+        st = bt.stats()
+        return out, (st.step, st.particle_steps)
+
+    shapes = [(tables, 96), (long_t, 8), (tables, 8)]
+    want = []
+    for t, n in shapes:
+        bt = make(t, n)
+        bt.step(4)
+        want.append(result(bt))
+        bt.close()
+    live = [make(t, n) for t, n in shapes]
+    for _ in range(2):
+        for bt in live:
+            bt.step(2)
+    for bt, (out, stats) in zip(live, want):
+        got, gs = result(bt)
+        assert gs == stats
+        for a, b in zip(got, out):
+            for k in a:
+                assert np.array_equal(a[k], b[k]), k
+        bt.close()
+    long_t.close()
