@@ -17,6 +17,8 @@
 //    and only its index goes to a per-warp queue; once 32 are queued the warp re-reads them (an L2 hit),
 //    recomputes the classical part, and runs the event branch (four Philox draws, the ICDF, Bessel
 //    functions, the spectra, the collapses, the daughter append) with all 32 lanes busy.
+#include <mutex>
+
 #include "qed_step32.cuh"
 
 namespace qed {
@@ -151,33 +153,42 @@ __global__ void __launch_bounds__(kT32, QED_MIN_BLOCKS) step32_kernel(TabP<float
 
 }  // namespace qed
 
-// grid = SMs x resident blocks of the kernel (persistent loop over tiles); cached per kernel
+// grid = SMs x resident blocks of the kernel (persistent loop over tiles); kept per device, kernel and table length
+// (shared by all threads: the kernels' shared-memory limit is raised to the device's once, not to each call's size)
 struct Launch32 {
+    int device = -1;
     const void* kern = nullptr;
     size_t smem = 0;
     int blocks = 0;
 };
 
-static int blocks32(int64_t capacity, const void* kern, size_t smem) {
-    static Launch32 cache[4];
-    Launch32* e = nullptr;
-    for (auto& c : cache)
-        if (c.kern == kern || c.kern == nullptr) {
-            e = &c;
-            break;
-        }
-    if (e->kern != kern || e->smem != smem) {
-        int dev = 0, sms = 1, per_sm = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, qed::kT32, smem);
-        e->kern = kern;
-        e->smem = smem;
-        e->blocks = sms * (per_sm < 1 ? 1 : per_sm);
+static int resident32(const void* kern, size_t smem) {
+    static std::mutex lock;
+    static Launch32 kept[32];
+    static unsigned next = 0;  // the entry that the next new one replaces
+    int dev = 0, sms = 1, per_sm = 1;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> hold(lock);
+    bool known = false;
+    for (const Launch32& e : kept) {
+        if (e.device != dev || e.kern != kern) continue;
+        if (e.smem == smem) return e.blocks;
+        known = true;
     }
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (!known) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qed::kMaxBlockSmem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, qed::kT32, smem);
+    Launch32& e = kept[next++ % 32];
+    e.device = dev;
+    e.kern = kern;
+    e.smem = smem;
+    e.blocks = sms * (per_sm < 1 ? 1 : per_sm);
+    return e.blocks;
+}
+
+static int blocks32(int64_t capacity, const void* kern, size_t smem) {
     const int64_t need = (capacity + 31) / 32;  // tiles of 32 particles
-    return (int)std::max<int64_t>(1, std::min<int64_t>((need + qed::kWarps32 - 1) / qed::kWarps32, (int64_t)e->blocks));
+    return (int)std::max<int64_t>(1, std::min<int64_t>((need + qed::kWarps32 - 1) / qed::kWarps32, (int64_t)resident32(kern, smem)));
 }
 
 // The full flag set in a single plane wave takes the kernels built for it (the batched kernels' arithmetic, bit for

@@ -326,3 +326,34 @@ def test_live_batches_keep_their_shared_memory(tables, graph_steps):
                 assert np.array_equal(a[k], b[k]), k
         bt.close()
     long_t.close()
+
+
+def test_single_buffer_steps_of_two_threads(tables):
+    """Threads that step their own particles with tables of different lengths (each on its own stream)."""
+    import threading
+    long_t = Q.Tables(chi_min=1e-3, chi_max=1e2, n_chi=4000, n_r=8)
+    f = Q.field(B.QED_FIELD_CP, a0=50.0, n_cycles=4.0, phase=4 * math.pi, eta0=ETA0)
+    failed = []
+
+    def run(t, seed):
+        try:
+            bm = I.lepton_beam(65, 3000.0, z_range=(-3.0, 3.0), seed=seed)
+            e, g, ctr = Q.ParticleBuffer(65, B.QED_FP32, B.QED_ELECTRON), Q.ParticleBuffer(40000, B.QED_FP32, B.QED_PHOTON), Q.Counters()
+            e.load(bm["pos"], bm["mom"], bm["spin"], bm["w"], bm["id"])
+            e.init_tau(seed)
+            stream = torch.cuda.Stream()
+            torch.cuda.synchronize()
+            for s in range(1500):
+                B.qed_push_step(t.handle, f, Q.step_desc(0.01, 0.01 * s, s, seed), e.s, g.s, ctr.ptr, stream.cuda_stream)
+            stream.synchronize()
+        except Exception as x:  # noqa: BLE001
+            failed.append(x)
+
+    threads = [threading.Thread(target=run, args=(t, k)) for k, t in enumerate((tables, long_t, tables, long_t))]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failed, failed
+    torch.cuda.synchronize()
+    long_t.close()
