@@ -433,13 +433,16 @@ qed_status qed_mlp_set_params(qed_mlp_t m, const float *host_in);
 qed_status qed_mlp_targets(qed_tables_t t, int64_t n, uint64_t seed, int64_t first_index, float *x_dev, float *y_dev,
                            double *raw_dev, void *stream);
 /* Forward and backward pass of one batch (n <= max_batch): grad_dev gets dL/dparameters for
- * L = mean over the batch of the squared error summed over the four outputs; loss_dev (may be NULL) L. */
+ * L = mean over the batch of the squared error summed over the four outputs; loss_dev (may be NULL) L.
+ * Up to 1024 samples the sums have a fixed order, and gradient and loss repeat bit for bit; above, the order of the
+ * FP32 sums over 128-sample tiles is the device's, and they repeat to rounding. */
 qed_status qed_mlp_grad(qed_mlp_t m, const float *x_dev, const float *y_dev, int64_t n, float *grad_dev,
                         float *loss_dev, void *stream);
 /* One AdamW step (beta 0.9 / 0.999, eps 1e-8, decoupled weight decay on weights only). */
 qed_status qed_mlp_adamw(qed_mlp_t m, const float *grad_dev, float lr, float weight_decay, void *stream);
 /* steps x (fresh batch of targets at first_index + k batch, forward, backward, AdamW), learning rate
- * decaying from lr to lr_final on a cosine; loss_per_step_dev (may be NULL) gets each step's loss. */
+ * decaying from lr to lr_final on a cosine; loss_per_step_dev (may be NULL) gets each step's loss.  Batches of up to
+ * 1024 samples train the same network bit for bit on every call; larger ones to the rounding of their gradients. */
 qed_status qed_mlp_train(qed_mlp_t m, qed_tables_t t, int64_t steps, int64_t batch, uint64_t seed, int64_t first_index,
                          float lr, float lr_final, float weight_decay, float *loss_per_step_dev, void *stream);
 /* Raw network outputs (n x 4) for feature rows x_dev (n x 3), on tensor cores. */

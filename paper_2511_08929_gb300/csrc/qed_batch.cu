@@ -620,10 +620,6 @@ __global__ void __launch_bounds__(256) batch_mlp_prep_kernel(const InstDev* __re
 // ------------------------------------------------------------------------------------------------
 constexpr int kFinishCluster = 8;
 
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
-}
-
 __global__ void __cluster_dims__(kFinishCluster, 1, 1)
     batch_finish_kernel(const InstDev* __restrict__ inst, int n_inst, SegDev* seg, int64_t* tile0, ClockDev* clk, SegCtx* ctx) {
     __shared__ bool last;

@@ -459,6 +459,11 @@ __device__ __forceinline__ void P_to_stokes(const V3<R>& P, const V3<R>& eps, co
     xi[2] = some ? (P1 * P1 - P2 * P2) * il : R(0);
 }
 
+// barrier over the blocks of a cluster (every thread of each)
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------------------------
 // block-level counter reduction: one atomic per block and counter
 // ---------------------------------------------------------------------------------------------

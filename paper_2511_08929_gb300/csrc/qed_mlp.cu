@@ -649,6 +649,15 @@ __device__ __forceinline__ uint32_t kmaj128(int r, int k) {
     return (uint32_t)((r >> 3) * 2048 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
 }
 
+// the float at p of this block's shared memory, in the block of the given rank of the cluster
+__device__ __forceinline__ float cluster_ld(const float* p, uint32_t rank) {
+    uint32_t addr;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(sm_u32(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ float bf16_round(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
 // one thread: D (+)= A B^T over ks steps of K = 16; group strides in bytes
@@ -738,6 +747,23 @@ __device__ __forceinline__ void column_sums(float v[kTU], float& s) {
     column_fold<1>(v);
     s += v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
+
+// What a block adds up over its warps: per unit b3, b2, b1, the four dW4 and the three dW1 values, then the loss and
+// dL/db4.  Four warps hold such sums of the same units, from a quarter of the tile's samples each.
+constexpr int kWarpSums = 10 * kH + 5;
+__device__ __forceinline__ int warp_sum_index(int e) {  // entry e's parameter (kParams: the loss)
+    const int f = e / kH, j = e % kH;
+    if (f >= 10) return e == 10 * kH ? kParams : kOffB4 + e - (10 * kH + 1);
+    if (f >= 7) return kOffW1 + 3 * j + (f - 7);
+    if (f >= 3) return kOffW4 + (f - 3) * kH + j;
+    return (f == 0 ? kOffB3 : (f == 1 ? kOffB2 : kOffB1)) + j;
+}
+
+// Batches of up to 8 tiles run as one cluster, whose blocks' sums are added in the order of their ranks through
+// distributed shared memory: the gradients of such a batch, and networks trained on it, repeat bit for bit.  Larger
+// batches add their blocks' sums atomically, in the order they arrive.  (The warps' sums are added in shared memory
+// first: 8836 atomic adds a block; 4 x 644 + 8192 of them, uncoalesced, cost 2 us of a step of 4096 samples.)
+constexpr int kTrainCluster = 8;
 
 // grad (zeroed by the caller) += dL/dparameters, loss (may be NULL) += L of the n samples (X, Tg)
 __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(const float* __restrict__ P, const float* __restrict__ X,
@@ -896,42 +922,70 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(const float
         }
         column_sums(v, sb1);
     }
-    // the block's sums to the gradient
+    // the block's sums, in the order of the parameters, the loss behind them (over the operand tiles, whose last MMAs
+    // have been awaited)
+    static_assert(sizeof(S.h1t) + sizeof(S.h2t) + sizeof(S.dzt) >= (kParams + 1) * sizeof(float), "the block's sums");
+    static_assert(sizeof(S.a) >= kTR / 32 * kWarpSums * sizeof(float), "the warps' sums");
+    float* sums = reinterpret_cast<float*>(S.h1t);
+    float* part = reinterpret_cast<float*>(S.a);
     const float bad = __int_as_float(0x7FC00000);
-    if (!first || !ok) {
-        const int u0 = tid & (kTR - 1);
-        if (u0 < kH) {  // (whole warps: the accumulator loads are collective)
-            float a[kTU], b[kTU];
+    const int u0 = tid & (kTR - 1);
+    if (u0 < kH) {  // (whole warps: the accumulator loads are collective)
+        float a[kTU] = {}, b[kTU] = {};
+        if (!first) {
             tc_ld16(row + kColW3 + c0, a);
             tc_ld16(row + kColW2 + c0, b);
-#pragma unroll
-            for (int q = 0; q < kTU; ++q) {
-                atomicAdd(&grad[kOffW3 + u0 * kH + c0 + q], ok ? a[q] : bad);
-                atomicAdd(&grad[kOffW2 + u0 * kH + c0 + q], ok ? b[q] : bad);
-            }
         }
-        if (!(lane & 1)) {
-            const int j = c0 + (lane >> 1);
-            atomicAdd(&grad[kOffB3 + j], ok ? sb3 : bad);
-            atomicAdd(&grad[kOffB2 + j], ok ? sb2 : bad);
-            atomicAdd(&grad[kOffB1 + j], ok ? sb1 : bad);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) atomicAdd(&grad[kOffW4 + q * kH + j], ok ? sw4[q] : bad);
-#pragma unroll
-            for (int q = 0; q < 3; ++q) atomicAdd(&grad[kOffW1 + 3 * j + q], ok ? sw1[q] : bad);
+        for (int q = 0; q < kTU; ++q) {
+            sums[kOffW3 + u0 * kH + c0 + q] = ok ? a[q] : bad;
+            sums[kOffW2 + u0 * kH + c0 + q] = ok ? b[q] : bad;
         }
-        if (c0 == 0) {  // one of a sample's four threads
-            for (int o = 16; o > 0; o >>= 1) {
-                lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+    }
+    float* mine = part + (u0 >> 5) * kWarpSums;
+    if (!(lane & 1)) {
+        const int j = c0 + (lane >> 1);
+        mine[j] = sb3;
+        mine[kH + j] = sb2;
+        mine[2 * kH + j] = sb1;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) sb4[q] += __shfl_down_sync(0xffffffffu, sb4[q], o);
-            }
-            if (lane == 0) {
-                if (loss) atomicAdd(loss, ok ? lsum : bad);
+        for (int q = 0; q < 4; ++q) mine[(3 + q) * kH + j] = sw4[q];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) atomicAdd(&grad[kOffB4 + q], ok ? sb4[q] : bad);
-            }
+        for (int q = 0; q < 3; ++q) mine[(7 + q) * kH + j] = sw1[q];
+    }
+    if (c0 == 0) {  // one of a sample's four threads
+        for (int o = 16; o > 0; o >>= 1) {
+            lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sb4[q] += __shfl_down_sync(0xffffffffu, sb4[q], o);
         }
+        if (lane == 0) {
+            mine[10 * kH] = lsum;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mine[10 * kH + 1 + q] = sb4[q];
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < kWarpSums; e += kTrainThreads) {
+        float v = part[e];
+        for (int k = 1; k < kTR / 32; ++k) v += part[k * kWarpSums + e];
+        sums[warp_sum_index(e)] = ok ? v : bad;
+    }
+    uint32_t rank, ranks;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(ranks));
+    cluster_sync();  // (a cluster of one where the launch names none)
+    if (ranks > 1) {  // the whole batch: one add per address, so their order is of no matter
+        for (int i = (int)rank * kTrainThreads + tid; i <= kParams; i += (int)ranks * kTrainThreads) {
+            float v = 0.0f;
+            for (uint32_t k = 0; k < ranks; ++k) v += cluster_ld(sums + i, k);
+            if (i < kParams) atomicAdd(&grad[i], v);
+            else if (loss) atomicAdd(loss, v);
+        }
+        cluster_sync();  // no block leaves while another reads its sums
+    } else {
+        for (int i = tid; i < kParams; i += kTrainThreads) atomicAdd(&grad[i], sums[i]);
+        if (tid == 0 && loss) atomicAdd(loss, sums[kParams]);
     }
     tc_fence_before();
     __syncthreads();
@@ -1296,8 +1350,27 @@ static qed_status mlp_grad_launch(qed_mlp_s* m, const float* x, const float* y, 
     if (cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainShared)) !=
         cudaSuccess)
         return QED_ERR_CUDA;
-    const int blocks = (int)std::min<int64_t>((n + kTR - 1) / kTR, sms);
-    mlp_train_kernel<<<blocks, kTrainThreads, sizeof(TrainShared), st>>>(m->P, x, y, n, grad, loss);
+    const int64_t tiles = (n + kTR - 1) / kTR;
+    cudaLaunchConfig_t launch = {};
+    launch.gridDim = dim3((unsigned)std::min<int64_t>(tiles, sms));
+    launch.blockDim = dim3(kTrainThreads);
+    launch.dynamicSmemBytes = sizeof(TrainShared);
+    launch.stream = st;
+    cudaLaunchAttribute cluster = {};
+    if (tiles > 1 && tiles <= kTrainCluster) {  // one cluster (of a power of two blocks; one without a tile adds zeros)
+        unsigned blocks = 1;
+        while (blocks < tiles) blocks *= 2;
+        launch.gridDim.x = blocks;
+        cluster.id = cudaLaunchAttributeClusterDimension;
+        cluster.val.clusterDim.x = blocks;
+        cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+        launch.attrs = &cluster;
+        launch.numAttrs = 1;
+    }
+    if (cudaLaunchKernelEx(&launch, mlp_train_kernel, (const float*)m->P, x, y, n, grad, loss) != cudaSuccess) {
+        cudaGetLastError();
+        return QED_ERR_CUDA;
+    }
     return QED_OK;
 }
 

@@ -357,3 +357,24 @@ def test_single_buffer_steps_of_two_threads(tables):
     assert not failed, failed
     torch.cuda.synchronize()
     long_t.close()
+
+
+# ---- repeatability of the training of small batches ------------------------------------------------------
+@pytest.mark.parametrize("n", [1, 64, 128, 129, 300, 640, 1000, 1024])
+def test_small_batches_train_bit_for_bit(tables, n):
+    """Up to 1024 samples a gradient is summed in a fixed order, so it, its loss and the networks trained on it repeat
+    bit for bit."""
+    smp = GM.Sampler(GM.init_params(6), max_batch=1024)
+    x, y, _ = GM.targets(tables, n, 5, 0)
+    g0, l0 = smp.grad(x, y)
+    for _ in range(50):
+        g, loss = smp.grad(x, y)
+        assert torch.equal(g, g0) and torch.equal(loss, l0)
+    nets = []
+    for _ in range(4):
+        smp.set_params(GM.init_params(6))
+        loss = smp.train(tables, 12, batch=n, seed=4)
+        nets.append((loss, smp.params()))
+    for loss, p in nets[1:]:
+        assert np.array_equal(loss, nets[0][0]) and np.array_equal(p, nets[0][1])
+    smp.close()
