@@ -278,7 +278,7 @@ using BatchRateQ = RateQT<int>;  // (a batch's buffers hold at most INT32_MAX pa
 
 // shared memory of the batched kernel: the 1-D rate tables (the Bessel table, read only by the event
 // kernel, stays in global memory behind L1), the tile list, the per-warp segment state, the tiles, the
-// event queues, the chunk rings and (plane-wave kernels) the rate queues
+// event queues, the chunk rings and (kernels with them) the rate queues
 __host__ __device__ inline size_t batch_smem_bytes(int warps, int stages, int n_chi, int n_seg, bool rate_queue) {
     size_t off = align128((size_t)4 * n_chi * 4);
     off += align128((size_t)(n_seg + 1) * 4);
@@ -290,8 +290,9 @@ __host__ __device__ inline size_t batch_smem_bytes(int warps, int stages, int n_
     return off;
 }
 
-// FIX: the step flags fixed at compile time (0: read from the context)
-template <int WARPS, int STAGES, int MINB, uint32_t FIX>
+// FIX: the step flags fixed at compile time (0: read from the context); RQ: photons that may have a pair rate go through
+// the rate queues (plane waves), the others only move
+template <int WARPS, int STAGES, int MINB, uint32_t FIX, bool RQ>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
     batch_step_kernel(TabP<float> T, float* bes_g, const InstDev* __restrict__ inst,
                       const SegDev* __restrict__ seg, const SegCtx* __restrict__ ctx,
@@ -314,8 +315,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     off += (size_t)WARPS * kWQ * 8;
     int2* s_chunks = (int2*)(smem + off);
     off += (size_t)WARPS * kChunkRing * 8;
-    BatchRateQ* s_rq = (BatchRateQ*)(smem + off);  // plane-wave kernels only (the offset so far is a multiple of 8)
-    constexpr bool PW = plane_waves_only<FIX>();
+    BatchRateQ* s_rq = (BatchRateQ*)(smem + off);  // (the offset so far is a multiple of 8)
+    static_assert(!RQ || plane_waves_only<FIX>(), "the rate queues' bound is that of a plane wave");
 
     for (int i = threadIdx.x; i < 2 * T.n_chi; i += blockDim.x) {
         sh.rates[i] = T.nlc_rate[i];
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     BatchRateQ& rq = s_rq[warp];
     int rn = 0;  // queued photons of the current segment (warp-uniform)
     float chi_z = 0.0f;
-    if (PW) chi_z = no_rate_chi(T, Tl.nbw_rate);
+    if (RQ) chi_z = no_rate_chi(T, Tl.nbw_rate);
     // the events of a pass to the warp's queue, and from there to the list
     auto list = [&](bool event, int j) {
         const unsigned m = __ballot_sync(0xffffffffu, event);
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
     while (true) {
         const bool more = t < te;
         // photons that may have a pair rate, 32 at a time (or what is left of a segment, whose context goes)
-        if (PW && (rn >= 32 || (rn > 0 && (!more || t >= WS.t1)))) {
+        if (RQ && (rn >= 32 || (rn > 0 && (!more || t >= WS.t1)))) {
             const int cnt = min(rn, 32);
             rn -= cnt;
             bool event = false;
@@ -472,7 +473,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
         }
         if (++st == STAGES) st = 0;
         bool event = false;
-        if (PW && sp == 2) {
+        if (RQ && sp == 2) {
             const bool rate = valid && photon_needs_rate<FIX ? FIX : QED_F_FULL>(C, WS.L, j, a, b, cc, chi_z, ctr, c);
             const unsigned m = __ballot_sync(0xffffffffu, rate);
             if (rate) rq.put(rn + __popc(m & ((1u << lane) - 1u)), j, a, b, cc);
@@ -480,7 +481,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
             __syncwarp();
         } else {
             if (valid)
-                event = !PW && sp == 2 ? photon_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl)
+                event = !RQ && sp == 2 ? photon_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl)
                                        : lepton_stream_one<FIX>(C, WS.L, j, a, b, cc, ctr, c, &Tl);
             list(event, j);
         }
@@ -702,6 +703,7 @@ typedef void (*batch_launch_fn)(const qed_batch_s* b, int grid, cudaStream_t st)
 struct BatchVariant {
     const void* kern;
     int warps, stages;
+    bool rate_queue;
     batch_launch_fn launch;
 };
 
@@ -725,7 +727,8 @@ struct qed_batch_s {
     unsigned char* d_ws;
     int64_t capacity_total;
     qed_batch_tuning tuning;
-    int grid;  // persistent grid of the current tuning
+    const BatchVariant* kern;  // the kernel and
+    int grid;                  // persistent grid of the current tuning
     cudaStream_t cap_stream;
     cudaGraphExec_t exec;
     int exec_steps;
@@ -742,47 +745,52 @@ struct qed_batch_s {
     unsigned long long* d_mfb;
 };
 
-template <int WARPS, int STAGES, int MINB, uint32_t FIX>
+template <int WARPS, int STAGES, int MINB, uint32_t FIX, bool RQ>
 static void launch_variant(const qed_batch_s* b, int grid, cudaStream_t st) {
     const qed_tables_s* t = b->tables;
-    const size_t smem = batch_smem_bytes(WARPS, STAGES, t->desc.n_chi, kSpecies * b->n_inst, plane_waves_only<FIX>());
-    batch_step_kernel<WARPS, STAGES, MINB, FIX><<<grid, WARPS * 32, smem, st>>>(
+    const size_t smem = batch_smem_bytes(WARPS, STAGES, t->desc.n_chi, kSpecies * b->n_inst, RQ);
+    batch_step_kernel<WARPS, STAGES, MINB, FIX, RQ><<<grid, WARPS * 32, smem, st>>>(
         tab_params<float>(t), t->bes32, b->d_inst, b->d_seg, b->d_ctx, b->d_tile0, b->n_inst, b->tuning.chunk,
         &b->d_clk->next_tile, b->d_ev, b->capacity_total, b->d_clk->n_list, b->ctr);
 }
 
-#define QED_VARIANTS(FIX)                                                                \
-    {{(const void*)batch_step_kernel<8, 3, 3, FIX>, 8, 3, launch_variant<8, 3, 3, FIX>},      \
-     {(const void*)batch_step_kernel<8, 3, 2, FIX>, 8, 3, launch_variant<8, 3, 2, FIX>},      \
-     {(const void*)batch_step_kernel<8, 2, 4, FIX>, 8, 2, launch_variant<8, 2, 4, FIX>},      \
-     {(const void*)batch_step_kernel<16, 2, 1, FIX>, 16, 2, launch_variant<16, 2, 1, FIX>},   \
-     {(const void*)batch_step_kernel<16, 2, 2, FIX>, 16, 2, launch_variant<16, 2, 2, FIX>}}
+#define QED_VARIANT(W, S, M, FIX, RQ) \
+    {(const void*)batch_step_kernel<W, S, M, FIX, RQ>, W, S, RQ, launch_variant<W, S, M, FIX, RQ>}
+#define QED_VARIANTS(FIX, RQ)                                                                               \
+    {QED_VARIANT(8, 3, 3, FIX, RQ), QED_VARIANT(8, 3, 2, FIX, RQ), QED_VARIANT(8, 2, 4, FIX, RQ),           \
+     QED_VARIANT(16, 2, 1, FIX, RQ), QED_VARIANT(16, 2, 2, FIX, RQ)}
 
-// [0]: flags read at run time; [1]: built for QED_F_FULL (every flag test of the streaming pass folded)
-static const BatchVariant kVariants[2][QED_BATCH_VARIANTS] = {QED_VARIANTS(0u), QED_VARIANTS(QED_F_FULL)};
+// [0]: flags read at run time; [1]: built for QED_F_FULL in plane waves (every flag test of the streaming pass folded);
+// [2]: that with the rate queues
+static const BatchVariant kVariants[3][QED_BATCH_VARIANTS] = {QED_VARIANTS(0u, false), QED_VARIANTS(QED_F_FULL, false),
+                                                              QED_VARIANTS(QED_F_FULL, true)};
 
-static size_t variant_smem(const qed_batch_s* b, int v, bool fixed) {
-    return batch_smem_bytes(kVariants[fixed][v].warps, kVariants[fixed][v].stages, b->tables->desc.n_chi,
-                            kSpecies * b->n_inst, fixed);
-}
-
-// the kernel built for the full flag set, where the batch is plane waves and its rate queues fit beside the tables
-static bool fixed_kernel(const qed_batch_s* b, int v) {
-    return b->desc.flags == QED_F_FULL && b->plane_waves && variant_smem(b, v, true) <= kMaxBlockSmem;
-}
-
-static const BatchVariant& variant_of(const qed_batch_s* b, int v) { return kVariants[fixed_kernel(b, v) ? 1 : 0][v]; }
-
-// resident blocks per SM of variant v for this batch (0 if it does not fit)
-static int variant_occupancy(const qed_batch_s* b, int v) {
+// resident blocks per SM of a kernel for this batch (0 if it does not fit)
+static int resident_blocks(const qed_batch_s* b, const BatchVariant& k) {
     int per_sm = 0;
-    const size_t smem = variant_smem(b, v, fixed_kernel(b, v));
+    const size_t smem = batch_smem_bytes(k.warps, k.stages, b->tables->desc.n_chi, kSpecies * b->n_inst, k.rate_queue);
     if (smem > kMaxBlockSmem) return 0;
-    const BatchVariant& k = variant_of(b, v);
     // the limit belongs to the kernel, which every live batch launches with a size of its own: always the device's
     if (cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBlockSmem) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.kern, k.warps * 32, smem) != cudaSuccess) return 0;
     return per_sm;
+}
+
+// The kernel of variant v for this batch and its resident blocks per SM (0 if it does not fit).  The full flag set in
+// plane waves takes the kernels built for it, with the rate queues where those leave at least three quarters of the
+// resident blocks: their 3 KB a warp come on top of the rate tables and the tile list.  96 collisions of up to 2e5
+// electrons, us a step with and without them: 740 / 803 at equal blocks (variant 0, 256 chi nodes), 764 / 791 at 3
+// blocks of 4 (variant 2), but 850 / 803 at 2 of 3 (variant 0, 448 nodes) and 1374 / 985 at 1 of 2 (3000 nodes), where
+// too few warps are left to hide the loads.  The kernels that read the flags take 923, 925 and 1123 there.
+static const BatchVariant& variant_of(const qed_batch_s* b, int v, int* blocks) {
+    const bool full = b->desc.flags == QED_F_FULL && b->plane_waves;
+    const BatchVariant& plain = kVariants[full][v];
+    *blocks = resident_blocks(b, plain);
+    if (!full) return plain;
+    const int queued = resident_blocks(b, kVariants[2][v]);
+    if (queued < 1 || 4 * queued < 3 * *blocks) return plain;
+    *blocks = queued;
+    return kVariants[2][v];
 }
 
 static bool valid_batch(const qed_batch_s* b) { return b != nullptr && b->magic == kBatchMagic; }
@@ -793,7 +801,7 @@ static void launch_batch_step(const qed_batch_s* b, cudaStream_t st, cudaEvent_t
                               bool capturing = false) {
     const unsigned rec = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (e0) cudaEventRecordWithFlags(e0, st, rec);
-    variant_of(b, b->tuning.variant).launch(b, b->grid, st);
+    b->kern->launch(b, b->grid, st);
     if (b->mlp) {  // the learned sampler draws every listed emission's energy fraction
         batch_mlp_prep_kernel<<<b->sms * 8, 256, 0, st>>>(b->d_inst, b->d_ctx, b->d_ev, b->d_clk, b->d_mchi, b->d_mr,
                                                           b->d_ms, b->d_mlep);
@@ -852,12 +860,14 @@ extern "C" qed_status qed_batch_set_tuning(qed_batch_t b, const qed_batch_tuning
     if (!tn || tn->variant < 0 || tn->variant >= QED_BATCH_VARIANTS || tn->blocks_per_sm < 0 || tn->chunk < 1 ||
         tn->chunk > 4096 || tn->graph_steps < 0 || tn->graph_steps > 4096)
         return QED_ERR_ARG;
-    const int occ = variant_occupancy(b, tn->variant);
+    int occ;
+    const BatchVariant& kern = variant_of(b, tn->variant, &occ);
     if (occ < 1) return QED_ERR_ARG;  // this variant does not fit this batch (shared memory)
     const int bps = tn->blocks_per_sm == 0 ? occ : std::min(tn->blocks_per_sm, occ);
     drop_graph(b);
     b->tuning = *tn;
     b->tuning.blocks_per_sm = bps;
+    b->kern = &kern;
     b->grid = b->sms * bps;
     return QED_OK;
 }
@@ -1199,7 +1209,8 @@ extern "C" qed_status qed_batch_tune(qed_batch_t b, int32_t steps_per_candidate,
     // runs of the guided schedule capped at 32, 64 or 128 tiles
     std::vector<qed_batch_tuning> cand;
     for (int v = 0; v < QED_BATCH_VARIANTS; ++v) {
-        const int occ = variant_occupancy(b, v);
+        int occ;
+        variant_of(b, v, &occ);
         for (int bps = occ; bps >= 1 && bps >= occ - 1; --bps)
             for (int ch : {32, 64, 128}) cand.push_back(qed_batch_tuning{v, bps, ch, 0});
     }

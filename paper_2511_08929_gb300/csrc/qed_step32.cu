@@ -193,7 +193,9 @@ static int blocks32(int64_t capacity, const void* kern, size_t smem) {
 
 // The full flag set in a single plane wave takes the kernels built for it (the batched kernels' arithmetic, bit for
 // bit).  With the kernels that read the flags, 64 steps of 1e4 electrons took 3.06 ms, 48 steps of 1e6 electrons with
-// 1e7 photons 31.9 ms; with these 2.94 and 30.5.
+// 1e7 photons 31.9 ms; with these 2.94 and 30.5.  They are taken wherever their rate queues fit beside the tables (up
+// to ~9000 chi nodes), also where those cost a block per SM: a step of 3e6 photons takes 113 us with the kernel that
+// reads the flags and 108 with this one at 256 nodes, 116 and 102 at 600, 185 and 141 at 4096, 199 and 162 at 8000.
 static bool fixed_flags32(const qed_field& f, const qed_step_desc& s, size_t smem) {
     return s.flags == QED_F_FULL && (f.kind == QED_FIELD_LP || f.kind == QED_FIELD_CP) && smem <= qed::kMaxBlockSmem;
 }

@@ -185,7 +185,7 @@ struct Shared32 {
 
 __host__ __device__ inline size_t align128(size_t b) { return (b + 127) & ~size_t(127); }
 
-// Photons that may have a pair rate, queued per warp by the plane-wave kernels (photon_needs_rate): the state words of
+// Photons that may have a pair rate, queued per warp by plane-wave kernels (photon_needs_rate): the state words of
 // the step (x, P_x; P_y, P_z, tau; k) and the index, a column per photon.
 constexpr int kRateQ = 64;  // drained 32 at a time
 template <class J>  // the index type
@@ -207,8 +207,7 @@ struct RateQT {
 };
 using RateQ = RateQT<int64_t>;
 
-// dynamic shared memory a block can have; the plane-wave kernels, whose rate queues come on top of the rate tables, run
-// only where their tables leave room (n_chi up to ~9000), else the kernels that read the flags do
+// dynamic shared memory a block can have
 constexpr size_t kMaxBlockSmem = 227 * 1024;
 
 // the single-buffer kernels' shared memory; bes: the Bessel table is staged too (the plane-wave kernels, which read it

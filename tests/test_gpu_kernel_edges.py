@@ -378,3 +378,50 @@ def test_small_batches_train_bit_for_bit(tables, n):
     for loss, p in nets[1:]:
         assert np.array_equal(loss, nets[0][0]) and np.array_equal(p, nets[0][1])
     smp.close()
+
+
+# ---- the choice of the plane-wave kernels ---------------------------------------------------------------
+@pytest.mark.parametrize("n_chi,n_inst", [(24, 1), (256, 96), (448, 96), (24, 300), (256, 1024), (2048, 8), (4096, 96), (9000, 3)])
+def test_plane_wave_kernels_keep_the_blocks_per_sm(n_chi, n_inst):
+    """The plane-wave kernels' rate queues cost no variant more than a quarter of the blocks per SM that the kernels
+    that read the flags have."""
+    t = Q.Tables(chi_min=1e-3, chi_max=1e2, n_chi=n_chi, n_r=4)
+    fields = [Q.field(B.QED_FIELD_LP, a0=10.0, n_cycles=4.0, eta0=ETA0)] * n_inst
+    got = []
+    for flags in (B.QED_F_FULL, B.QED_F_FULL | B.QED_F_TBMT_PAPER):
+        bt = Q.Batch(t, fields, [1] * n_inst, [(8, 8, 8)] * n_inst, 0.1, flags=flags)
+        per = []
+        for v in range(5):
+            try:
+                bt.set_tuning(variant=v, blocks_per_sm=0, chunk=4, graph_steps=0)
+                per.append(bt.tuning().blocks_per_sm)
+            except B.QedError:
+                per.append(0)
+        got.append(per)
+        bt.close()
+    t.close()
+    assert all(4 * a >= 3 * b for a, b in zip(*got)), got
+
+
+@pytest.mark.parametrize("n_chi", [24, 448, 600, 3000, 6000])
+def test_plane_wave_kernels_agree(n_chi):
+    """Table lengths on either side of where the rate queues are left out: the photons of a batch are word for word
+    those of the kernels that read the flags."""
+    t = Q.Tables(chi_min=1e-3, chi_max=1e2, n_chi=n_chi, n_r=8)
+    b = _photons(20011, 61)
+    got = []
+    for flags in (B.QED_F_FULL, B.QED_F_FULL | B.QED_F_TBMT_PAPER):  # (T-BMT concerns leptons only: one step)
+        bt = Q.Batch(t, [Q.field(B.QED_FIELD_CP, a0=150.0, n_cycles=6.0, phase=2.0, eta0=ETA0)], [3],
+                     [(20011, 20011, 20011)], 0.2, t0=8.0, flags=flags)
+        bt.buffers()[0][2].load(b["pos"], b["mom"], b["spin"], b["w"], b["id"])
+        bt.buffers()[0][2].init_tau(3)
+        bt.step(1)
+        c = bt.ctr.read().as_dict()
+        c.pop("first_bad")
+        got.append(([{k: v[np.argsort(r["id"])] for k, v in r.items()} for r in (x.read() for x in bt.buffers()[0])], c))
+        bt.close()
+    assert got[0][1] == got[1][1] and got[0][1]["events"] > 0 and got[0][1]["nonfinite"] == 3
+    for x, y in zip(got[0][0], got[1][0]):
+        for k in x:
+            assert np.array_equal(x[k], y[k], equal_nan=True), k
+    t.close()
