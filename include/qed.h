@@ -392,7 +392,8 @@ qed_status qed_batch_set_kernel_events(qed_batch_t b, void *const *events, int32
 /* Autotuner: times the persistent and event kernels of every launch shape it considers on the batch's
  * own next steps (they are real steps: results do not depend on the shape), picks the one with the least
  * time per particle-step and sets it.  steps_per_candidate >= 1.  cache_path (may be NULL): a text file of
- * one JSON object per line, keyed by device, SM count and workload size; a matching line is used
+ * one JSON object per line, keyed by device, SM count, workload size and kernels (the full flag set in
+ * plane waves has its own; a build with other kernels times again); a matching line is used
  * without timing, a new result is appended.  Synchronizes `stream`. */
 qed_status qed_batch_tune(qed_batch_t b, int32_t steps_per_candidate, const char *cache_path, qed_batch_tuning *out,
                           void *stream);

@@ -776,6 +776,8 @@ static int resident_blocks(const qed_batch_s* b, const BatchVariant& k) {
     return per_sm;
 }
 
+static bool full_plane_waves(const qed_batch_s* b) { return b->desc.flags == QED_F_FULL && b->plane_waves; }
+
 // The kernel of variant v for this batch and its resident blocks per SM (0 if it does not fit).  The full flag set in
 // plane waves takes the kernels built for it, with the rate queues where those leave at least three quarters of the
 // resident blocks: their 3 KB a warp come on top of the rate tables and the tile list.  96 collisions of up to 2e5
@@ -783,7 +785,7 @@ static int resident_blocks(const qed_batch_s* b, const BatchVariant& k) {
 // blocks of 4 (variant 2), but 850 / 803 at 2 of 3 (variant 0, 448 nodes) and 1374 / 985 at 1 of 2 (3000 nodes), where
 // too few warps are left to hide the loads.  The kernels that read the flags take 923, 925 and 1123 there.
 static const BatchVariant& variant_of(const qed_batch_s* b, int v, int* blocks) {
-    const bool full = b->desc.flags == QED_F_FULL && b->plane_waves;
+    const bool full = full_plane_waves(b);
     const BatchVariant& plain = kVariants[full][v];
     *blocks = resident_blocks(b, plain);
     if (!full) return plain;
@@ -1149,6 +1151,12 @@ extern "C" qed_status qed_batch_stats_read(qed_batch_t b, qed_batch_stats* out, 
 }
 
 // ---- autotuner ------------------------------------------------------------------------------------
+// revision of the step kernels' registers and shared memory: a shape timed with another one is timed again
+constexpr int kKernelRevision = 3;
+
+// What a shape was timed on: device, workload size and which kernels the batch runs (the best variant differs: 96
+// collisions of up to 2e5 electrons take 912 us in variant 4 and 923 in variant 0 with the kernels that read the flags,
+// 770 and 740 with those of the full flag set).
 static std::string tune_key(const qed_batch_s* b) {
     cudaDeviceProp p;
     std::string name = "unknown";
@@ -1158,7 +1166,8 @@ static std::string tune_key(const qed_batch_s* b) {
     int lg = 0;
     while (lg < 62 && (1ll << (lg + 1)) <= b->capacity_total) ++lg;
     char buf[512];
-    snprintf(buf, sizeof buf, "%s|sm%d|inst%d|cap2^%d|nchi%d", name.c_str(), b->sms, b->n_inst, lg, b->tables->desc.n_chi);
+    snprintf(buf, sizeof buf, "%s|sm%d|inst%d|cap2^%d|nchi%d|%s%d", name.c_str(), b->sms, b->n_inst, lg,
+             b->tables->desc.n_chi, full_plane_waves(b) ? "full" : "flags", kKernelRevision);
     return buf;
 }
 

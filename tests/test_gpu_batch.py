@@ -9,6 +9,7 @@ the step counter on the device, CUDA-graph replay, autotuned launch shape).
 * The launch shape (kernel variant, blocks per SM, chunk, graph or direct launches) changes nothing.
 * The autotuner picks a valid shape, records it in its cache and reuses it.
 """
+import json
 import math
 import os
 
@@ -311,3 +312,28 @@ def test_autotuner_picks_and_caches(gpu_tables, tmp_path):
     torch.cuda.synchronize()
     assert bt.ctr.read().status == 0
     bt.close()
+
+
+@pytest.mark.gpu
+def test_autotuner_keeps_kernels_apart(gpu_tables, tmp_path):
+    """A shape timed with the kernels of the full flag set is not taken for a batch that runs the others, nor one whose
+    key an older build wrote."""
+    specs = [s for s in _specs() if s["field"].kind in (B.QED_FIELD_LP, B.QED_FIELD_CP)]
+    path = str(tmp_path / "tune.jsonl")
+    first = _make_batch(gpu_tables, specs)
+    first.tune(1, path)
+    other = _make_batch(gpu_tables, specs, flags=B.QED_F_FULL | B.QED_F_AMM)
+    s0 = other.stats().step
+    other.tune(1, path)
+    lines = open(path).read().strip().splitlines()
+    keys = [json.loads(line)["key"] for line in lines]
+    assert other.stats().step > s0 and len(set(keys)) == 2
+    first.close()
+    other.close()
+    with open(path, "w") as f:  # the same shape under the key without the kernels
+        f.write(lines[0].replace(keys[0], keys[0].rsplit("|", 1)[0]) + "\n")
+    again = _make_batch(gpu_tables, specs)
+    s0 = again.stats().step
+    again.tune(1, path)
+    assert again.stats().step > s0 and len(open(path).read().strip().splitlines()) == 2
+    again.close()
