@@ -1081,11 +1081,14 @@ __global__ void __launch_bounds__(kTR, kTcPerSm) mlp_net_kernel(const float* __r
 // The check: samples that pass on the float tables are done; the others wait in a block-wide queue, and a full block
 // of them at a time goes through FP64 (the check again for those within kMargin32 of the bound, the table path for
 // those that fail it, and for all of them with flags bit 0).  One block of 1024 threads per SM: the queue's last,
-// partly filled pass then runs in a few warps of every SM.  Samples that need the bracketing solver (a logit above the
+// partly filled pass then runs in a few warps of every SM.  The tiles are cut so that every SM has as many samples, and
+// few samples get blocks of 128 threads: in tiles of 1024, the FP64 passes of 2000 samples ran on two SMs (551 us at
+// a bound of 1e-5, longer than the 502 of the fused kernel's tiles of 128; 105 so).  Samples that need the bracketing solver (a logit above the
 // grid: uniforms within 2e-9 of 1) wait in a second queue: it takes ~20 times Newton's instructions, and run in the
 // lane that met it, it held that lane's whole warp (4e5 table samples, 1 in 24 of them such: 22.7 ms, with the queue
 // 14.8).
 constexpr int kCheckThreads = 1024;
+constexpr int kCheckFew = 128;  // threads of a block when one tile of that size per SM takes all samples
 
 struct CheckItem {
     int64_t i;
@@ -1103,8 +1106,9 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
                                                                      unsigned long long* n_fallback,
                                                                      const unsigned long long* __restrict__ n_dev) {
     extern __shared__ __align__(16) unsigned char check_smem[];
-    CheckItem* queue = reinterpret_cast<CheckItem*>(check_smem);             // [2 kCheckThreads]
-    int64_t* slow = reinterpret_cast<int64_t*>(queue + 2 * kCheckThreads);  // [2 kCheckThreads]
+    const int threads = blockDim.x;
+    CheckItem* queue = reinterpret_cast<CheckItem*>(check_smem);             // [2 blockDim.x]
+    int64_t* slow = reinterpret_cast<int64_t*>(queue + 2 * threads);         // [2 blockDim.x]
     __shared__ int queued, n_slow;
     if (n_dev) {
         const int64_t nd = (int64_t)*n_dev;
@@ -1133,14 +1137,17 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
         if (fell) fell[q.i] = fb ? 1 : 0;
         if (fb) {
             if (!table_path(T, T32, besp, chi_in, r_in, s_in, q.i, out4, ln_up_only, false))
-                slow[atomicAdd(&n_slow, 1)] = q.i;  // at most 2 kCheckThreads - 1 entries
+                slow[atomicAdd(&n_slow, 1)] = q.i;  // at most 2 blockDim.x - 1 entries
             ++nf;
         }
     };
-    for (int64_t base = (int64_t)blockIdx.x * kCheckThreads; base < n; base += (int64_t)gridDim.x * kCheckThreads) {
+    // tiles of equal size for every block: as many rounds as 1024 samples a block would take, in full warps
+    const int64_t most = (int64_t)gridDim.x * threads, rounds = max((int64_t)1, (n + most - 1) / most);
+    const int tile = (int)((n + gridDim.x * rounds - 1) / (gridDim.x * rounds) + 31) & ~31;
+    for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
         const int64_t i = base + threadIdx.x;
         bool waits = false;  // this thread's sample went to the queue
-        if (i < n) {
+        if ((int)threadIdx.x < tile && i < n) {
             CheckItem q{i, 0.0f, 0.0f, __int_as_float(0x7FC00000), 0.0f};
             bool done = false;
             if (table_only) {
@@ -1186,31 +1193,31 @@ __global__ void __launch_bounds__(kCheckThreads, 1) mlp_check_kernel(TabP<double
             if (done) {
                 if (fell) fell[i] = 0;
             } else {
-                queue[atomicAdd(&queued, 1)] = q;  // at most 2 kCheckThreads - 1 entries
+                queue[atomicAdd(&queued, 1)] = q;  // at most 2 blockDim.x - 1 entries
                 waits = true;
             }
         }
         // The tile's entries are counted by the barrier itself: `queued`, read behind it, could already hold what a
         // faster warp added for the next tile, and the warps would part at the barriers below.
         held += __syncthreads_count(waits);
-        if (held >= kCheckThreads) {
-            held -= kCheckThreads;
+        if (held >= threads) {
+            held -= threads;
             finish(queue[held + threadIdx.x]);
             __syncthreads();
             const int sn = n_slow;  // the same in every thread
-            if (sn >= kCheckThreads)
-                table_path(T, T32, besp, chi_in, r_in, s_in, slow[sn - kCheckThreads + threadIdx.x], out4, ln_up_only, true);
+            if (sn >= threads)
+                table_path(T, T32, besp, chi_in, r_in, s_in, slow[sn - threads + threadIdx.x], out4, ln_up_only, true);
             __syncthreads();
             if (threadIdx.x == 0) {
                 queued = held;
-                if (sn >= kCheckThreads) n_slow = sn - kCheckThreads;
+                if (sn >= threads) n_slow = sn - threads;
             }
             __syncthreads();
         }
     }
     if ((int)threadIdx.x < held) finish(queue[threadIdx.x]);  // (written before the loop's last barrier)
     __syncthreads();
-    for (int k = threadIdx.x; k < n_slow; k += kCheckThreads)
+    for (int k = threadIdx.x; k < n_slow; k += threads)
         table_path(T, T32, besp, chi_in, r_in, s_in, slow[k], out4, ln_up_only, true);
     nf = __reduce_add_sync(0xffffffffu, nf);
     if ((threadIdx.x & 31) == 0 && n_fallback && nf) atomicAdd(n_fallback, (unsigned long long)nf);
@@ -1451,14 +1458,20 @@ static qed_status mlp_sample_launch(qed_mlp_t m, const qed_tables_s* t, const do
                                     int64_t n, const unsigned long long* n_dev, double tol, int flags, float* out4,
                                     uint8_t* fell_back, float* err_out, unsigned long long* n_fallback, int grid,
                                     cudaStream_t st) {
-    const size_t smem = 2 * kCheckThreads * (sizeof(CheckItem) + sizeof(int64_t));
-    if (cudaFuncSetAttribute(mlp_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    constexpr size_t kPerThread = 2 * (sizeof(CheckItem) + sizeof(int64_t));
+    if (cudaFuncSetAttribute(mlp_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kCheckThreads * kPerThread)) != cudaSuccess)
         return QED_ERR_CUDA;
     if (!(flags & QED_MLP_ALWAYS_TABLE))
         mlp_net_kernel<<<grid, kTR, 0, st>>>(m->P, chi, r, s, n, out4, n_dev);
-    const int blocks = (int)std::min<int64_t>((n + kCheckThreads - 1) / kCheckThreads, (grid + kTcPerSm - 1) / kTcPerSm);
-    mlp_check_kernel<<<blocks, kCheckThreads, smem, st>>>(tab_params<double>(t), tab_params<float>(t), t->bes32, t->besp, chi,
-                                                          r, s, n, tol, flags, out4, fell_back, err_out, n_fallback, n_dev);
+    const int blocks = (int)std::min<int64_t>((n + 31) / 32, sms);
+    const int threads = n <= (int64_t)kCheckFew * sms ? kCheckFew : kCheckThreads;
+    mlp_check_kernel<<<blocks, threads, threads * kPerThread, st>>>(tab_params<double>(t), tab_params<float>(t), t->bes32,
+                                                                    t->besp, chi, r, s, n, tol, flags, out4, fell_back,
+                                                                    err_out, n_fallback, n_dev);
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
 }
 

@@ -425,3 +425,21 @@ def test_plane_wave_kernels_agree(n_chi):
         for k in x:
             assert np.array_equal(x[k], y[k], equal_nan=True), k
     t.close()
+
+
+@pytest.mark.parametrize("per_sm", [128, 1024])
+@pytest.mark.parametrize("over", [-1, 0, 1, 33])
+def test_sampler_at_the_edges_of_its_block_sizes(tables, per_sm, over):
+    """The check's blocks have 128 threads up to 128 samples an SM, then 1024, and its tiles are cut so that every
+    block takes as many: each sample is what it is in small calls."""
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + over
+    chi, r, s = _query(n, 14)
+    smp = GM.Sampler(GM.init_params(4))
+    for kw in ({}, {"table_only": True}):
+        out, fell, nf = smp.sample(tables, chi, r, s, tol=3e-3, **kw)
+        assert int(nf) == int(fell.sum()) > 0
+        for a in (0, 1000, n // 2, n - 700):
+            part = slice(a, min(n, a + 1001))
+            o1, f1, _ = smp.sample(tables, chi[part].contiguous(), r[part].contiguous(), s[part].contiguous(), tol=3e-3, **kw)
+            assert torch.equal(o1, out[part]) and torch.equal(f1, fell[part])
+    smp.close()
