@@ -131,15 +131,15 @@ __device__ __forceinline__ double nlc_integral(const double* bes, double chi, do
     return s * r;
 }
 
-constexpr int kNlcThreads = 64;
+constexpr int kNlcThreads = 64, kNlcMaxThreads = 128;
 constexpr int kNlcPanels = 70;  // cbrt(80) * 16 = 68.9
 
 // One block per (sign, chi row).  FP64-bound, 13 densities an iteration, and an entry takes 5 to 60 iterations (a
 // root approached from the left, where the density falls, is bracketed by bisection): a lane that has finished an
 // entry takes the row's next one, so no lane waits for the longest of its warp (256 x 256 entries a sign: 36.5 ms
 // with one entry a thread, 29.7 ms so).
-__global__ void __launch_bounds__(kNlcThreads) nlc_rows_kernel(const double* __restrict__ bes, qed_table_desc d,
-                                                               double* rates, double* icdf) {
+__global__ void __launch_bounds__(kNlcMaxThreads) nlc_rows_kernel(const double* __restrict__ bes, qed_table_desc d,
+                                                                  double* rates, double* icdf) {
     __shared__ double cum[kNlcPanels + 1];
     __shared__ int next;
     const int n_chi = d.n_chi;
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kNlcThreads) nlc_rows_kernel(const double* __r
         cum[p + 1] = nlc_integral(bes, chi, sigma, p * kPanel, fmin(tend, (p + 1) * kPanel));
     __syncthreads();
     if (threadIdx.x == 0) {
-        next = kNlcThreads;
+        next = blockDim.x;
         cum[0] = 0.0;
         for (int p = 0; p < np; ++p) cum[p + 1] += cum[p];
         rates[s * n_chi + i] = log(cum[np]);
@@ -523,7 +523,13 @@ extern "C" qed_status qed_tables_build(const qed_table_desc* desc, qed_tables_t*
         return QED_ERR_CUDA;
     }
     bessel_table_kernel<<<(kBesN + 127) / 128, 128, 0, st>>>(t->bes64, t->bes32);
-    nlc_rows_kernel<<<2 * d.n_chi, kNlcThreads, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
+    int sms = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, t->device);
+    // Where every row has an SM of its own, four warps keep its four FP64 pipes busy (2 x 4096 entries a sign: 160 ms
+    // with two warps, 91 with four, 92 with eight; 76 x 256: 16.2, 13.2, 12.2); rows that share an SM do better with
+    // two, whose last entries hold fewer idle warps (77 x 256: 16.7, 20.4, 19.2; 256 x 256: 31.6, 41.1, 37.7).
+    const int nlc_threads = 2 * (int64_t)d.n_chi <= sms ? kNlcMaxThreads : kNlcThreads;
+    nlc_rows_kernel<<<2 * d.n_chi, nlc_threads, 0, st>>>(t->bes64, d, t->rate64, t->icdf64);
     bessel_poly_kernel<<<(kBpN + 3) / 4, 128, 0, st>>>(t->besp);
     nbw_rows_kernel<<<d.n_chi, 256, 0, st>>>(t->besp, d, t->rate64, t->icdf64);
     to_float_kernel<<<64, 256, 0, st>>>(t->rate64, t->rate32, nr);

@@ -34,3 +34,19 @@ def test_table_edges_match_oracle(chi_min, chi_max, n_chi, n_r, y_lo, y_hi):
         assert np.all(np.isfinite(e[k]))
         assert np.all(np.abs(e[k] - getattr(o, k)) <= tol), (k, np.abs(e[k] - getattr(o, k)).max(axis=(0, 1)))
     np.testing.assert_allclose(amm, o.ensure_amm().amm, rtol=0, atol=1e-12)
+
+
+@pytest.mark.parametrize("n_r", [64, 65, 129, 1000])
+def test_rows_do_not_depend_on_how_many_there_are(n_r):
+    """The NLC rows take blocks of 128 threads where every row has an SM, else of 64: the entries of a grid's end rows
+    are the same in a grid of two rows and in one that has them among many."""
+    lo, hi = 1e-3, 1e2
+    few = Q.Tables(lo, hi, 2, n_r)
+    many = Q.Tables(lo, hi, 201, n_r)
+    a, b = few.export(), many.export()
+    few.close()
+    many.close()
+    for k in ("nlc_rate", "nbw_rate"):
+        np.testing.assert_allclose(a[k], b[k][:, [0, -1]], rtol=0, atol=1e-13)  # (chi_max = chi_min e^(n d) to rounding)
+    for k in ("nlc_icdf", "nbw_icdf"):
+        assert np.array_equal(a[k][:, 0], b[k][:, 0]), k
