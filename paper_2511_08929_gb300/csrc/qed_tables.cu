@@ -313,21 +313,29 @@ __global__ void __launch_bounds__(256) nbw_rows_kernel(const double* __restrict_
         double t = a + w * u;
         // where the series has not converged within its 12 terms (the lowest panels of rows with large chi, whose
         // spectrum varies over t ~ chi^{-1/2}) the root is finished on the quadrature itself, one step from the
-        // series' root
+        // series' root; where it is no series at all (chi above ~1e5) from the panel's chord, inside a bracket
         const double* c = coef[s][lo];
-        if (fabs(c[kGL - 1]) + fabs(c[kGL - 2]) > 2e-14 * fabs(c[0]) && t > a) {
-            for (int it = 0; it < 4; ++it) {
+        const double rest = fabs(c[kGL - 1]) + fabs(c[kGL - 2]);
+        if (rest > 2e-14 * fabs(c[0]) && target > 0.0) {
+            const bool far = rest > 1e-2 * fabs(c[0]);
+            if (far) t = a + w * fmin(T / whole, 1.0);
+            double tl = a, th = a + w;
+            for (int it = 0; it < 100 && t > a; ++it) {
                 double dens[2], sum = 0.0;
                 for (int k = 0; k < kGL; ++k) {
                     nbw_density(besp, chi, 0.5 * (a + t) + 0.5 * (t - a) * c_gl_x[k], dens[0], dens[1]);
                     sum += c_gl_w[k] * (s ? dens[1] : dens[0]);
                 }
+                const double F = sum * 0.5 * (t - a) - T;
                 nbw_density(besp, chi, t, dens[0], dens[1]);
-                const double tn = t - (sum * 0.5 * (t - a) - T) / (s ? dens[1] : dens[0]);
-                if (!(tn >= a && tn <= a + w)) break;
-                const bool found = fabs(tn - t) <= 1e-9 * t;
-                t = tn;
-                if (found) break;
+                const double tn = t - F / (s ? dens[1] : dens[0]);
+                if (fabs(tn - t) <= (far ? 1e-15 : 1e-9) * t && tn >= a && tn <= a + w) {
+                    t = tn;
+                    break;
+                }
+                if (F > 0.0) th = t; else tl = t;
+                t = tn > tl && tn < th ? tn : 0.5 * (tl + th);
+                if (th - tl <= 1e-15 * th) break;
             }
         }
         icdf[((size_t)(2 + s) * n_chi + i) * d.n_r + m] = 2.0 * log(t);

@@ -50,3 +50,23 @@ def test_rows_do_not_depend_on_how_many_there_are(n_r):
         np.testing.assert_allclose(a[k], b[k][:, [0, -1]], rtol=0, atol=1e-13)  # (chi_max = chi_min e^(n d) to rounding)
     for k in ("nlc_icdf", "nbw_icdf"):
         assert np.array_equal(a[k][:, 0], b[k][:, 0]), k
+
+
+@pytest.mark.parametrize("chi_min,chi_max", [(1e4, 3e5), (1e5, 1e7), (1e6, 1e10)])
+def test_rows_of_very_large_chi_invert_their_quadrature(chi_min, chi_max):
+    """Rows whose spectrum the panels' nodes do not resolve (chi above 1e5) still invert the CDF of their 12-point
+    quadrature: the oracle's tables under the same rule, each row rising.  1e-5: where that CDF is nearly flat an entry
+    hangs on its rounding."""
+    d = (chi_min, chi_max, 9, 65, -20.0, 20.0)
+    g = Q.Tables(*d)
+    e = g.export()
+    g.close()
+    O.set_quadrature(12, 1.0 / 16.0)
+    try:
+        o = O.tables(*d)
+        want = {k: np.array(getattr(o, k)) for k in ("nbw_rate", "nbw_icdf")}
+    finally:
+        O.set_quadrature(10, 1.0 / 16.0)
+    np.testing.assert_allclose(e["nbw_rate"], want["nbw_rate"], rtol=0, atol=1e-11)
+    assert np.all(np.diff(e["nbw_icdf"], axis=2) > 0)
+    assert np.abs(e["nbw_icdf"] - want["nbw_icdf"]).max() <= 1e-5
