@@ -356,7 +356,12 @@ __device__ __noinline__ bool mix_quantile_fast(const TabP<double>& T, const TabP
         yu = yu32;
         yd = yd32;
     }
-    return mix_newton<double>(T, i, f, m.a, r, 8, 1e-7, L, yu, yd);
+    if (!mix_newton<double>(T, i, f, m.a, r, 8, 1e-7, L, yu, yd)) return false;
+    // between the branch quantiles, as the bracketing solver: with |s| > 1 the blend has a negative weight and its root
+    // lies beyond them (tested on the high word, since every FP64 instruction counts here)
+    if ((__double2hiint(m.s) & 0x7FFFFFFF) >= 0x3FF00000)
+        L = fmin(fmax(L, fmin(m.qu, m.qd) - 1e-9), fmax(m.qu, m.qd) + 1e-9);
+    return true;
 }
 
 // xi3 = F3 / F0 at u' = e^L from the Bessel polynomials (see xi3_at)

@@ -443,3 +443,17 @@ def test_sampler_at_the_edges_of_its_block_sizes(tables, per_sm, over):
             o1, f1, _ = smp.sample(tables, chi[part].contiguous(), r[part].contiguous(), s[part].contiguous(), tol=3e-3, **kw)
             assert torch.equal(o1, out[part]) and torch.equal(f1, fell[part])
     smp.close()
+
+
+def test_mixture_quantile_stays_between_the_branches(tables):
+    """s_beta beyond +-1 (a spin of length above 1): the table path's quantile lies between those of the two branches,
+    which s_beta = 1 and -1 give."""
+    chi, r, _ = _query(20003, 15)
+    smp = GM.Sampler(GM.init_params(4))
+    at = {s: smp.sample(tables, chi, r, torch.full_like(chi, s), table_only=True)[0][:, 0].double()
+          for s in (-4.0, -1.5, -1.0000005, -1.0, 1.0, 1.0000005, 1.2, 3.0)}
+    lo, hi = torch.minimum(at[-1.0], at[1.0]), torch.maximum(at[-1.0], at[1.0])
+    slack = 1e-8 + 2.0 ** -23 * torch.maximum(lo.abs(), hi.abs())  # one rounding of each float
+    for s, got in at.items():
+        assert bool(((got >= lo - slack) & (got <= hi + slack)).all()), s
+    smp.close()
