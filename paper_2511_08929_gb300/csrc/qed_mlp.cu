@@ -628,7 +628,7 @@ __device__ void tc_teardown(uint32_t tmem) {
 // BF16 and sums are FP32; biases, layer 1 and the 4-wide layer's gradient are FP32 sums over the warp's lanes.
 // TMEM columns: Z2, Z3, a scratch accumulator, dW3, dW2.
 // Nine GEMM launches that staged their operands from FP32 arrays in global memory (13-80 us each on 32 blocks) and
-// ten elementwise and column-sum launches took 0.34 ms for a batch of 4096; this pass takes 25 us.
+// ten elementwise and column-sum launches took 0.34 ms for a batch of 4096; this pass takes 23 us.
 constexpr uint32_t kTrainCols = 512;
 constexpr uint32_t kColZ2 = 0, kColZ3 = 64, kColT = 128, kColW3 = 192, kColW2 = 256;
 
@@ -710,7 +710,7 @@ __device__ __forceinline__ bool tc_await(uint64_t* bar, uint32_t& phase) {
 
 // Four threads share a sample, 16 units each (a warp reads the TMEM lanes of its index modulo 4): the elementwise work
 // and the column sums are what a pass costs, and one thread per sample left a single warp on each scheduler (61 us a
-// pass of 32 tiles against 25).
+// pass of 32 tiles against 25 with four; 23 now).
 constexpr int kTrainThreads = 4 * kTR;
 constexpr int kTU = 16;  // units per thread
 

@@ -110,8 +110,10 @@ __global__ void __launch_bounds__(128) bessel_poly_kernel(double* tab) {
 }
 
 // NLC rows.  An entry is the value at which Newton's method on the 12-point quadrature, kept inside its bracket,
-// stops (a bracket or a step of one part in 1e15): the learned sampler is trained on differences of two of these
-// entries down to 1e-7, so the rows keep every bit of that definition, and only the work's distribution is free.
+// stops (a bracket or a step of one part in 1e15).  The learned sampler is trained on differences of two of these
+// entries down to 1e-7, and a network follows their last bits: so that networks stay the same from build to build the
+// rows keep every bit of that definition, and only the work's distribution is free.  A choice that costs 29 ms (every
+// row on the panels' series, as the NBW rows are: 2.2 ms a build, entries within an ulp of these).
 __device__ __forceinline__ double nlc_density(const double* __restrict__ bes, double chi, double sigma, double t) {
     double b[3];
     const double up = t * t * t;
